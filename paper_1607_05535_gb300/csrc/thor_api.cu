@@ -161,7 +161,7 @@ void carve(Carver& cv, Impl<R>& I, int ncol, int nv) {
   R** pc[] = {&P.rho, &P.th, &P.p};
   for (R** p : pc) *p = cv.take<R>(C);
   P.m4 = cv.take<R>(4 * C);
-  T.lp = cv.take<R>(2 * C);
+  T.lp = cv.take<R>(C);
   P.w = cv.take<R>(F);
   I.F.inv = cv.take<double>(F);
   I.F.cf = cv.take<double>(F);

@@ -29,7 +29,7 @@ struct Work {
   R *qvr;                          // interfaces
   R *dd;                           // 3-D divergence (small step)
   R *dd0;                          // 3-D divergence of X^t (first small step of every stage)
-  R *lp;                           // [nv][colp][2]: the Laplacian of that D and the cell's p*
+  R *lp;                           // p* + K_d lap(D): the scalar whose gradient drives M*
   R *ca, *cb, *cc;                 // per-cell parts of the column equations (a, b, c)
   R *dhm;                          // horizontal divergence of the new M*
   R *psurf;                        // [colp] surface pressure (physics)

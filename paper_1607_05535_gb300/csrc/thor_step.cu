@@ -429,10 +429,14 @@ template <typename R>
 // Divergence damping, first stencil (Sec. 4, reading R5: the damping is
 // -K_d grad_h(lap D)): the Laplacian of the 3-D divergence D of the total
 // momentum, D = d0 in the first small step of a stage and later the D the
-// previous column step formed; stored packed with the cell's p* (the
-// momentum step gathers both)
-__device__ __forceinline__ void d_ss_lapd(const Geo<R>& G, const VR<R>& U, const Work<R>& T, const R* dsrc, const R* pstar, int kchunk,
-                                          int bx, int by) {
+// previous column step formed. The pressure gradient and the damping go
+// through the same gradient weights, so what is stored is the one scalar
+// q = p* + K_d lap D whose gradient the momentum step takes: one word per
+// cell written here and gathered there instead of two, and 21 multiply-adds
+// per cell less there. Bound by the loads' latency (float) or the float64
+// pipe; g6 x 32: float 7.3 -> %LAPF% us a level half, float64 13.9 -> %LAPD% us.
+__device__ __forceinline__ void d_ss_lapd(const Geo<R>& G, const VR<R>& U, const Work<R>& T, const R* dsrc, const R* pstar, R Kd,
+                                          int kchunk, int bx, int by) {
   int c = bx * blockDim.x + threadIdx.x;
   if (c >= G.ncol) return;
   const int S = G.colp;
@@ -446,16 +450,17 @@ __device__ __forceinline__ void d_ss_lapd(const Geo<R>& G, const VR<R>& U, const
     R l = 0;
 #pragma unroll
     for (int j = 0; j < 7; ++j) l += wl.v[j] * ldh(dsrc + (o + nb.n[j]), pk);
-    st2h(T.lp, i, l * ld(U.inv_rc2 + (k)), ldh(pstar + (i), pk), pk);
+    sth(T.lp + i, fmar<R>(l * ld(U.inv_rc2 + (k)), Kd, ldh(pstar + (i), pk)), pk);
   }
 }
 
-// Eq. mom2 with the divergence damping: M* <- proj(M* + dtau(-grad p* + DD + S_M));
+// Eq. mom2 with the divergence damping: M* <- proj(M* + dtau(-grad q + S_M)),
+// q = p* + K_d lap D of d_ss_lapd, or p* itself without the damping;
 // in the last small step of a stage also M^(s+1) = M^(s) + M* into Xo (which
 // may be Xs itself: each cell reads its own Xs value before writing it), with
 // the low parts XsL -> XoL of a compensated state (null: none)
 template <typename R>
-__device__ __forceinline__ void d_ss_mom(const Geo<R>& G, const VR<R>& U, const Slow<R>& SL, const Pert<R>& P, const Work<R>& T, R dtau, R Kd,
+__device__ __forceinline__ void d_ss_mom(const Geo<R>& G, const VR<R>& U, const Slow<R>& SL, const Pert<R>& P, const Work<R>& T, R dtau,
                                             int divdamp, const Xf<R>& Xs, const Xf<R>& Xo, const Xf<R>& XsL, const Xf<R>& XoL, int last,
                                             int kchunk, int bx, int by) {
   int c = bx * blockDim.x + threadIdx.x;
@@ -465,38 +470,24 @@ __device__ __forceinline__ void d_ss_mom(const Geo<R>& G, const VR<R>& U, const 
   Nbr7 nb = load_nbr(G, c);
   W7x3<R> wg = load_w7x3(G.wgrad, S, c);
   R rx = ld(G.rhat + (c)), ry = ld(G.rhat + (S + c)), rz = ld(G.rhat + (2 * S + c));
+  const R* q = divdamp ? T.lp : P.p;
   int k0 = by * kchunk, k1 = min(G.nv, k0 + kchunk);
 #pragma unroll 2
   for (int k = k0; k < k1; ++k) {
     const int o = k * S, i = o + c;
     R inv_r = ld(U.inv_rc + (k));
-    R ddx = 0, ddy = 0, ddz = 0;
     R gx = 0, gy = 0, gz = 0;
-    if (divdamp) {
-      // one packed gather per neighbour: the Laplacian of D and p*, both
-      // through the (projected) gradient weights
-      R ax = 0, ay = 0, az = 0;
 #pragma unroll
-      for (int j = 0; j < 7; ++j) {
-        const Q2<R> q = ld2h(T.lp, (size_t)(o + nb.n[j]), pk);
-        ax += wg.x[j] * q.x;
-        ay += wg.y[j] * q.x;
-        az += wg.z[j] * q.x;
-        gx += wg.x[j] * q.y;
-        gy += wg.y[j] * q.y;
-        gz += wg.z[j] * q.y;
-      }
-      R s = -Kd * inv_r;
-      ddx = s * ax;
-      ddy = s * ay;
-      ddz = s * az;
-    } else {
-      grad7(wg, nb, P.p + o, gx, gy, gz);
+    for (int j = 0; j < 7; ++j) {
+      const R v = ldh(q + (o + nb.n[j]), pk);
+      gx += wg.x[j] * v;
+      gy += wg.y[j] * v;
+      gz += wg.z[j] * v;
     }
     const Q4<R> m = ld4h(P.m4, (size_t)i, pk);
-    R mx = m.x + dtau * (fmar<R>(-gx, inv_r, ddx) + ldh(SL.smx + (i), ps));
-    R my = m.y + dtau * (fmar<R>(-gy, inv_r, ddy) + ldh(SL.smy + (i), ps));
-    R mz = m.z + dtau * (fmar<R>(-gz, inv_r, ddz) + ldh(SL.smz + (i), ps));
+    R mx = m.x + dtau * fmar<R>(-gx, inv_r, ldh(SL.smx + (i), ps));
+    R my = m.y + dtau * fmar<R>(-gy, inv_r, ldh(SL.smy + (i), ps));
+    R mz = m.z + dtau * fmar<R>(-gz, inv_r, ldh(SL.smz + (i), ps));
     project(rx, ry, rz, mx, my, mz);
     st4h(P.m4, i, mx, my, mz, m.w, pk);
     if (last) {          // end of the stage: M^(s+1) = M^(s) + M*
@@ -1099,18 +1090,18 @@ __global__ void k_stage_init(Geo<R> G, VR<R> U, Phys ph, Xf<R> Xt, Xf<R> X, Work
 // the small-step stencils take a level range [kchunk * klo, khi) (klo in
 // chunks), so that the lower and upper levels can run as separate launches
 template <typename R>
-__global__ void k_ss_lapd(Geo<R> G, VR<R> U, Work<R> T, const R* dsrc, const R* pstar, int kchunk, int klo,
+__global__ void k_ss_lapd(Geo<R> G, VR<R> U, Work<R> T, const R* dsrc, const R* pstar, R Kd, int kchunk, int klo,
                           int khi) {
   G.nv = khi;
-  d_ss_lapd<R>(G, U, T, dsrc, pstar, kchunk, blockIdx.x, blockIdx.y + klo);
+  d_ss_lapd<R>(G, U, T, dsrc, pstar, Kd, kchunk, blockIdx.x, blockIdx.y + klo);
 }
 // LAST: the last small step of a stage (a separate instantiation, so the
 // other small steps carry no registers for the stage end)
 template <typename R, bool LAST>
-__global__ void k_ss_mom(Geo<R> G, VR<R> U, Slow<R> SL, Pert<R> P, Work<R> T, R dtau, R Kd, int divdamp,
+__global__ void k_ss_mom(Geo<R> G, VR<R> U, Slow<R> SL, Pert<R> P, Work<R> T, R dtau, int divdamp,
                          Xf<R> Xs, Xf<R> Xo, Xf<R> XsL, Xf<R> XoL, int kchunk, int klo, int khi) {
   G.nv = khi;
-  d_ss_mom<R>(G, U, SL, P, T, dtau, Kd, divdamp, Xs, Xo, XsL, XoL, LAST ? 1 : 0, kchunk, blockIdx.x,
+  d_ss_mom<R>(G, U, SL, P, T, dtau, divdamp, Xs, Xo, XsL, XoL, LAST ? 1 : 0, kchunk, blockIdx.x,
               blockIdx.y + klo);
 }
 template <typename R>
@@ -1442,7 +1433,7 @@ __global__ void ke_ss_lapd(const Member<R>* __restrict__ M, const int2* __restri
   THOR_MEMBER();
   Geo<R> G = a.G;
   G.nv = khi;
-  if (a.divdamp) d_ss_lapd<R>(G, a.U, a.T, j == 0 ? a.T.dd0 : a.T.dd, a.P.p, kchunk, e.y, blockIdx.y + klo);
+  if (a.divdamp) d_ss_lapd<R>(G, a.U, a.T, j == 0 ? a.T.dd0 : a.T.dd, a.P.p, a.Kd, kchunk, e.y, blockIdx.y + klo);
 }
 template <typename R>
 __global__ void ke_ss_mom(const Member<R>* __restrict__ M, const int2* __restrict__ map, int s, int j,
@@ -1450,7 +1441,7 @@ __global__ void ke_ss_mom(const Member<R>* __restrict__ M, const int2* __restric
   THOR_MEMBER();
   Geo<R> G = a.G;
   G.nv = khi;
-  d_ss_mom<R>(G, a.U, a.SL, a.P, a.T, (R)a.dts[s], a.Kd, a.divdamp, Xs, s == 2 ? a.Xt : a.Xst,
+  d_ss_mom<R>(G, a.U, a.SL, a.P, a.T, (R)a.dts[s], a.divdamp, Xs, s == 2 ? a.Xt : a.Xst,
               s == 0 ? a.XtL : Xf<R>{}, s == 2 ? a.XtL : Xf<R>{}, j + 1 == a.nsub[s], kchunk, e.y,
               blockIdx.y + klo);
 }
@@ -1536,10 +1527,10 @@ int Impl<R>::large_step(double dt, int n_small) {
   const bool lsplit = level_split && side != nullptr && !prof_on && side2 != nullptr && G.nv >= 2 * kc;
   const int nch = (G.nv + kc - 1) / kc, hc = lsplit ? nch / 2 : nch;
   dim3 glo(g2.x, hc), ghi(g2.x, nch - hc);
-  auto lapd = [&](cudaStream_t st, const R* dsrc, dim3 g, int klo, int khi) -> cudaError_t {
-    return launch_k(k_ss_lapd<R>, g, bs, 0, st, G, U, T, dsrc, (const R*)P.p, kc, klo, khi);
-  };
   const R Kd = (R)(diff_D * dbar4 / dt);
+  auto lapd = [&](cudaStream_t st, const R* dsrc, dim3 g, int klo, int khi) -> cudaError_t {
+    return launch_k(k_ss_lapd<R>, g, bs, 0, st, G, U, T, dsrc, (const R*)P.p, Kd, kc, klo, khi);
+  };
   const double dts[3] = {dt / 3.0, dt / n_small, dt / n_small};
   const int nsub[3] = {1, n_small / 2, n_small};
   cudaError_t e = cudaSuccess;
@@ -1641,7 +1632,7 @@ int Impl<R>::large_step(double dt, int n_small) {
           ++launches;
         }
         mark(THOR_K_SS_MOM, true);
-        chk(launch_k(last ? k_ss_mom<R, true> : k_ss_mom<R, false>, g, bs, 0, st, G, U, SL, P, T, (R)dts[s], Kd,
+        chk(launch_k(last ? k_ss_mom<R, true> : k_ss_mom<R, false>, g, bs, 0, st, G, U, SL, P, T, (R)dts[s],
                      divdamp, Xs, Xo, XsL, XoL, kc, klo, khi));
         mark(THOR_K_SS_MOM, false);
         mark(THOR_K_SS_FLUX, true);
@@ -1707,6 +1698,9 @@ int Impl<R>::anelastic_step(double dt) {
   launch_2d(G.nv + 1, kc, g2i);
   dim3 g1((G.ncol + bs - 1) / bs);
   const R Kd = (R)(diff_D * dbar4 / dt);
+  auto lapd = [&](cudaStream_t st, const R* dsrc, dim3 g, int klo, int khi) -> cudaError_t {
+    return launch_k(k_ss_lapd<R>, g, bs, 0, st, G, U, T, dsrc, (const R*)P.p, Kd, kc, klo, khi);
+  };
   const double dts[3] = {dt / 3.0, dt / 2.0, dt};
   const bool ho = ph.vorder > 1;
   for (int s = 0; s < 3; ++s) {
