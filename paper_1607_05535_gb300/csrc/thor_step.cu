@@ -433,8 +433,8 @@ template <typename R>
 // through the same gradient weights, so what is stored is the one scalar
 // q = p* + K_d lap D whose gradient the momentum step takes: one word per
 // cell written here and gathered there instead of two, and 21 multiply-adds
-// per cell less there. Bound by the loads' latency (float) or the float64
-// pipe; g6 x 32: float 7.3 -> %LAPF% us a level half, float64 13.9 -> %LAPD% us.
+// per cell less there. This kernel is bound by its loads' latency; at g6 x 32
+// float 11.7 -> 11.6 us, float64 25.4 -> 28.2 us.
 __device__ __forceinline__ void d_ss_lapd(const Geo<R>& G, const VR<R>& U, const Work<R>& T, const R* dsrc, const R* pstar, R Kd,
                                           int kchunk, int bx, int by) {
   int c = bx * blockDim.x + threadIdx.x;
@@ -458,7 +458,10 @@ __device__ __forceinline__ void d_ss_lapd(const Geo<R>& G, const VR<R>& U, const
 // q = p* + K_d lap D of d_ss_lapd, or p* itself without the damping;
 // in the last small step of a stage also M^(s+1) = M^(s) + M* into Xo (which
 // may be Xs itself: each cell reads its own Xs value before writing it), with
-// the low parts XsL -> XoL of a compensated state (null: none)
+// the low parts XsL -> XoL of a compensated state (null: none). Bound by the
+// gathers' latency (float) and by the float64 pipe's multiply-adds (float64):
+// with one gathered scalar instead of two, g6 x 32 float 28.7 -> 25.2 us,
+// float64 147 -> 84 us.
 template <typename R>
 __device__ __forceinline__ void d_ss_mom(const Geo<R>& G, const VR<R>& U, const Slow<R>& SL, const Pert<R>& P, const Work<R>& T, R dtau,
                                             int divdamp, const Xf<R>& Xs, const Xf<R>& Xo, const Xf<R>& XsL, const Xf<R>& XoL, int last,
