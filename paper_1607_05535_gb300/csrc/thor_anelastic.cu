@@ -61,9 +61,11 @@ __global__ void k_an_predict(Geo<R> G, Xf<R> Xt, Slow<R> SL, Xf<R> Xo, double dt
       continue;
     }
     if (k < nv) {
-      mx[i] = d_of(Xt.mx[i]) + dts * d_of(SL.smx[i]);
-      my[i] = d_of(Xt.my[i]) + dts * d_of(SL.smy[i]);
-      mz[i] = d_of(Xt.mz[i]) + dts * d_of(SL.smz[i]);
+      R sx, sy, sz;
+      tan_from(load_tan(G.tb, S, c), ld2(SL.sm2, i), sx, sy, sz);
+      mx[i] = d_of(Xt.mx[i]) + dts * d_of(sx);
+      my[i] = d_of(Xt.my[i]) + dts * d_of(sy);
+      mz[i] = d_of(Xt.mz[i]) + dts * d_of(sz);
       Xo.th[i] = (R)(d_of(Xt.th[i]) + dts * d_of(SL.sth[i]));
       Xo.rho[i] = R(0);
     }

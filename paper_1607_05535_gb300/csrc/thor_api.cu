@@ -153,14 +153,15 @@ void carve(Carver& cv, Impl<R>& I, int ncol, int nv) {
   T.wc = cv.take<R>(C);
   T.psurf = cv.take<R>(S);
   Slow<R>& SL = I.SL;
-  R** sc[] = {&SL.smx, &SL.smy, &SL.smz, &SL.srho, &SL.sth, &SL.dsc, &SL.acr, &SL.pi};
+  R** sc[] = {&SL.srho, &SL.sth, &SL.dsc, &SL.acr, &SL.pi};
   for (R** p : sc) *p = cv.take<R>(C);
+  SL.sm2 = cv.take<R>(2 * C);
   SL.sw = cv.take<R>(F);
   SL.thi = cv.take<R>(F);
   Pert<R>& P = I.P;
   R** pc[] = {&P.rho, &P.th, &P.p};
   for (R** p : pc) *p = cv.take<R>(C);
-  P.m4 = cv.take<R>(4 * C);
+  P.m2 = cv.take<R>(2 * C);
   T.lp = cv.take<R>(C);
   P.w = cv.take<R>(F);
   I.F.inv = cv.take<double>(F);
@@ -174,6 +175,9 @@ void carve(Carver& cv, Impl<R>& I, int ncol, int nv) {
   I.G.wlap = cv.take<R>(7 * S);
   I.G.rhat = cv.take<R>(3 * S);
   I.G.gcor = cv.take<R>(3 * S);
+  I.G.tb = cv.take<R>(3 * S);
+  I.G.wg2 = cv.take<R>(14 * S);
+  I.G.wd2 = cv.take<R>(14 * S);
   I.G.sinlat = cv.take<R>(S);
   I.G.coslat = cv.take<R>(S);
   I.G.xdir = cv.take<R>(S);
@@ -208,14 +212,42 @@ int upload_tables(Impl<R>& I, const HostGrid& h, const std::vector<double>* vert
   const int ncol = h.ncol, S = colp_of(ncol), nv = h.nv;
   std::vector<int> nbr(6 * (size_t)S, 0);
   std::vector<R> wdiv(28 * (size_t)S, 0), wgrad(28 * (size_t)S, 0), wlap(7 * (size_t)S, 0),
-      rhat(3 * (size_t)S, 0), gcor(3 * (size_t)S, 0), sl(S, 0), cl(S, 0), clon(S, 0);
+      rhat(3 * (size_t)S, 0), gcor(3 * (size_t)S, 0), sl(S, 0), cl(S, 0), clon(S, 0), tb(3 * (size_t)S, 0),
+      wg2(14 * (size_t)S, 0), wd2(14 * (size_t)S, 0);
+  // e1 and e2 of the tangent basis at column c (thor_kernels.cuh)
+  auto basis = [&](int c, double e[2][3]) {
+    const double x = h.P[3 * c], y = h.P[3 * c + 1], z = h.P[3 * c + 2], s = z < 0.0 ? -1.0 : 1.0;
+    const double X = s * x, Y = s * y, A = -1.0 / (1.0 + std::fabs(z));
+    e[0][0] = 1.0 + A * X * X;
+    e[0][1] = e[1][0] = A * X * Y;
+    e[1][1] = 1.0 + A * Y * Y;
+    e[0][2] = -X;
+    e[1][2] = -Y;
+    tb[c] = (R)X;
+    tb[S + c] = (R)Y;
+    tb[2 * (size_t)S + c] = (R)A;
+  };
   std::vector<double> area(S, 0.0);
   for (int c = 0; c < ncol; ++c) {
     for (int j = 0; j < 6; ++j) {
       int q = h.nbr[6 * c + j];
       nbr[(size_t)j * S + c] = q < 0 ? c : q;
     }
+    double own[2][3];
+    basis(c, own);
     for (int j = 0; j < 7; ++j) {
+      const int m = j == 0 || h.nbr[6 * c + j - 1] < 0 ? c : h.nbr[6 * c + j - 1];
+      double there[2][3];
+      basis(m, there);
+      for (int a = 0; a < 2; ++a) {
+        double g = 0.0, d = 0.0;
+        for (int k = 0; k < 3; ++k) {
+          g += h.w_grad[21 * c + 3 * j + k] * own[a][k];
+          d += h.w_div[21 * c + 3 * j + k] * there[a][k];
+        }
+        wg2[((size_t)j * S + c) * 2 + a] = (R)g;
+        wd2[((size_t)j * S + c) * 2 + a] = (R)d;
+      }
       const size_t q = ((size_t)j * S + c) * 4;        // packed [7][colp][4]
       for (int d = 0; d < 3; ++d) {
         wdiv[q + d] = (R)h.w_div[21 * c + 3 * j + d];
@@ -245,6 +277,9 @@ int upload_tables(Impl<R>& I, const HostGrid& h, const std::vector<double>* vert
   e = e ? e : up(I.G.wgrad, wgrad.data(), wgrad.size() * sizeof(R));
   e = e ? e : up(I.G.wlap, wlap.data(), wlap.size() * sizeof(R));
   e = e ? e : up(I.G.rhat, rhat.data(), rhat.size() * sizeof(R));
+  e = e ? e : up(I.G.tb, tb.data(), tb.size() * sizeof(R));
+  e = e ? e : up(I.G.wg2, wg2.data(), wg2.size() * sizeof(R));
+  e = e ? e : up(I.G.wd2, wd2.data(), wd2.size() * sizeof(R));
   e = e ? e : up(I.G.gcor, gcor.data(), gcor.size() * sizeof(R));
   e = e ? e : up(I.G.sinlat, sl.data(), sl.size() * sizeof(R));
   e = e ? e : up(I.G.coslat, cl.data(), cl.size() * sizeof(R));

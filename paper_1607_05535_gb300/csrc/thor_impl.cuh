@@ -38,7 +38,8 @@ struct Work {
 // Slow tendencies and small-step coefficients of a stage
 template <typename R>
 struct Slow {
-  R *smx, *smy, *smz, *srho, *sth, *dsc, *acr, *pi;  // centres
+  R *sm2;                                 // [nv][colp][2]: S_M in the column's tangent basis
+  R *srho, *sth, *dsc, *acr, *pi;         // centres
   R *sw, *thi;                                        // interfaces
 };
 
@@ -46,7 +47,7 @@ struct Slow {
 template <typename R>
 struct Pert {
   R *rho, *th, *p;                 // centres
-  R *m4;                           // [nv][colp][4]: M* (x, y, z) and theta of the stage state
+  R *m2;                           // [nv][colp][2]: M* in the column's tangent basis
   R *w;                            // interfaces
 };
 

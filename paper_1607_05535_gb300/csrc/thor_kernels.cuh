@@ -81,6 +81,11 @@ struct Geo {
   const R* gcor;
   const R* wlap;        // [7][colp]
   const R* rhat;        // [3][colp]
+  // Tangent basis e1, e2 of every column as [3][colp] X, Y, A (tan_to,
+  // tan_from), and the stencils of tangent fields in it, [7][colp][2]:
+  // wg2 = the gradient weights of the point on the column's own basis, wd2 =
+  // the divergence weights of the point on the neighbour's basis.
+  const R *tb, *wg2, *wd2;
   const R* sinlat;      // [colp]
   const R* coslat;
   const R* xdir;        // cos(lon) cos(lat) = x of the unit position
@@ -373,6 +378,37 @@ __device__ __forceinline__ void st2h(double* base, size_t cell, double x, double
                : "memory");
 }
 
+// Tangent vectors in two components. A column's orthonormal basis follows
+// from its unit position r (the construction of Duff et al. 2017, J. Comput.
+// Graph. Tech. 6, with r mirrored into the upper half space): with s = sign(z),
+// X = s x, Y = s y, A = -1 / (1 + |z|),
+//   e1 = (1 + A X X, A X Y, -X),  e2 = (A X Y, 1 + A Y Y, -Y).
+// The small step keeps M*, and the stage its S_M, as (M . e1, M . e2): both
+// are tangent, so the projection of Eq. proj_h after every update, a third of
+// the stencils' multiply-adds and a third of the words go.
+template <typename R>
+struct Tan {
+  R X, Y, A;
+};
+template <typename R>
+__device__ __forceinline__ Tan<R> load_tan(const R* tb, int colp, int c) {
+  return {ld(tb + c), ld(tb + (colp + c)), ld(tb + (2 * colp + c))};
+}
+// components of the tangential part of a Cartesian vector
+template <typename R>
+__device__ __forceinline__ Q2<R> tan_to(const Tan<R>& b, R x, R y, R z) {
+  const R t = b.A * (b.X * x + b.Y * y) - z;
+  return {x + b.X * t, y + b.Y * t};
+}
+// the Cartesian vector u e1 + v e2
+template <typename R>
+__device__ __forceinline__ void tan_from(const Tan<R>& b, const Q2<R>& m, R& x, R& y, R& z) {
+  const R q = b.X * m.x + b.Y * m.y, t = b.A * q;
+  x = m.x + b.X * t;
+  y = m.y + b.Y * t;
+  z = -q;
+}
+
 struct Nbr7 {
   int n[7];
 };
@@ -415,6 +451,22 @@ __device__ __forceinline__ W7x3<R> load_w7x3(const R* w, int colp, int c) {
     o.x[j] = q.x;
     o.y[j] = q.y;
     o.z[j] = q.z;
+  }
+  return o;
+}
+// two-component weights of the seven points, packed [7][colp][2]
+template <typename R>
+struct W7x2 {
+  R x[7], y[7];
+};
+template <typename R>
+__device__ __forceinline__ W7x2<R> load_w7x2(const R* w, int colp, int c) {
+  W7x2<R> o;
+#pragma unroll
+  for (int j = 0; j < 7; ++j) {
+    const Q2<R> q = ld2(w, (size_t)j * colp + c);
+    o.x[j] = q.x;
+    o.y[j] = q.y;
   }
   return o;
 }

@@ -144,6 +144,7 @@ __device__ __forceinline__ void d_slow(const Geo<R>& G, const VR<R>& U, const Ph
   load_w7x3_lap(G.wdiv, S, c, wd, wl);
   const R gcx = ld(G.gcor + (c)), gcy = ld(G.gcor + (S + c)), gcz = ld(G.gcor + (2 * S + c));
   R rx = ld(G.rhat + (c)), ry = ld(G.rhat + (S + c)), rz = ld(G.rhat + (2 * S + c));
+  const Tan<R> tb = load_tan(G.tb, S, c);
   const R two_om = pc<R>(ph.two_omega, ph.two_omega_f), gamma = pc<R>(ph.gamma, ph.gamma_f),
           Rd = pc<R>(ph.Rd, ph.Rd_f);
   int k0 = by * kchunk, k1 = min(kend, k0 + kchunk);
@@ -202,7 +203,6 @@ __device__ __forceinline__ void d_slow(const Geo<R>& G, const VR<R>& U, const Ph
       FMx = -hx * inv_r2;
       FMy = -hy * inv_r2;
       FMz = -hz * inv_r2;
-      project(rx, ry, rz, FMx, FMy, FMz);
       R Fp = -Rd * hT * inv_r2;
       Fth = thfull / (gamma * p) * Fp;
     }
@@ -235,7 +235,7 @@ __device__ __forceinline__ void d_slow(const Geo<R>& G, const VR<R>& U, const Ph
       R ah = sa[j] * inv_r;
       A[j] = ah + sqh * whi_w * vhi3[j] - sql * wlo_w * vlo3[j];
     }
-    R acr, ahx, ahy, ahz;
+    R acr;
     if constexpr (SH) {
       // traditional Coriolis f r x M_h, f = 2 Omega sin(lat); w advected as a scalar
       const R mx = ld(X.mx + (i)), my = ld(X.my + (i)), mz = ld(X.mz + (i)), f = two_om * rz;
@@ -251,10 +251,6 @@ __device__ __forceinline__ void d_slow(const Geo<R>& G, const VR<R>& U, const Ph
         if (k + 1 < G.nv) whi_c = ld(U.wlo + (k + 1)) * ld(T.wc + (i)) + ld(U.whi + (k + 1)) * ld(T.wc + (i + S));
       }
       acr = sa3 * inv_r + sqh * whi_w * whi_c - sql * wlo_w * wlo_c;
-      const R d = A[0] * rx + A[1] * ry + A[2] * rz;
-      ahx = A[0] - d * rx;
-      ahy = A[1] - d * ry;
-      ahz = A[2] - d * rz;
     } else {
       // Coriolis 2 Omega z x (rho v) with the full momentum
       R wc = HO ? vint_centre(U, X.w, k, c, S, G.nv) : ld(U.clo + (k)) * wlo_w + ld(U.chi + (k)) * whi_w;
@@ -263,18 +259,13 @@ __device__ __forceinline__ void d_slow(const Geo<R>& G, const VR<R>& U, const Ph
       A[0] += -two_om * fy;
       A[1] += two_om * fx;
       acr = A[0] * rx + A[1] * ry + A[2] * rz;
-      ahx = A[0] - acr * rx;
-      ahy = A[1] - acr * ry;
-      ahz = A[2] - acr * rz;
     }
 
     // the anelastic switch leaves the pressure force to the projection
     const R pgr = ph.anelastic ? R(0) : inv_r;
-    R smx = -gx * pgr - ahx + FMx, smy = -gy * pgr - ahy + FMy, smz = -gz * pgr - ahz + FMz;
-    project(rx, ry, rz, smx, smy, smz);
-    SL.smx[i] = smx;
-    SL.smy[i] = smy;
-    SL.smz[i] = smz;
+    // the tangential part of the sum, in the basis the small step works in
+    const Q2<R> sm = tan_to(tb, -gx * pgr - A[0] + FMx, -gy * pgr - A[1] + FMy, -gz * pgr - A[2] + FMz);
+    st2(SL.sm2, i, sm.x, sm.y);
 
     R dh = sdh * inv_r;
     R dv = sqh * whi_w - sql * wlo_w;
@@ -309,6 +300,7 @@ __device__ __forceinline__ void d_slow_w(const Geo<R>& G, const VR<R>& U, const 
   const int S = G.colp;
   Nbr7 nb = load_nbr(G, c);
   W7<R> wl = load_w7(G.wlap, S, c);
+  const Tan<R> tb = load_tan(G.tb, S, c);
   const R g = pc<R>(ph.g, ph.g_f), gamma = pc<R>(ph.gamma, ph.gamma_f);
   int k0 = by * kchunk, k1 = min(G.nv + 1, k0 + kchunk);
 #pragma unroll 2
@@ -322,8 +314,8 @@ __device__ __forceinline__ void d_slow_w(const Geo<R>& G, const VR<R>& U, const 
     };
     if (init && k < G.nv) {
       P.rho[i] = dif(Xt.rho, X.rho, XtL.rho);
-      st4(P.m4, i, dif(Xt.mx, X.mx, XtL.mx), dif(Xt.my, X.my, XtL.my), dif(Xt.mz, X.mz, XtL.mz),
-          ld(T.theta + (i)));
+      const Q2<R> m = tan_to(tb, dif(Xt.mx, X.mx, XtL.mx), dif(Xt.my, X.my, XtL.my), dif(Xt.mz, X.mz, XtL.mz));
+      st2(P.m2, i, m.x, m.y);
       P.th[i] = dif(Xt.th, X.th, XtL.th);
       const R tht = XtL.th ? ld(Xt.th + (i)) + ld(XtL.th + (i)) : ld(Xt.th + (i));
       R ppt = eos_dev<R>(ld(U.pb + (k)), ld(U.thb + (k)), tht, gamma);
@@ -364,8 +356,8 @@ __device__ __forceinline__ void d_slow_w(const Geo<R>& G, const VR<R>& U, const 
 // The perturbations at the start of a stage on their own (the state's step
 // runs this beside the slow terms): Phi* = Phi^t - Phi^(s), p* from the
 // nonlinear Eq. theta_to_p; all zero in the first stage, where Phi^(s) =
-// Phi^t and p^(s) = EOS(Th^t). M* goes into the packed plane with theta of
-// the stage state beside it (the column fluxes gather both). XtL: the low
+// Phi^t and p^(s) = EOS(Th^t). M* is tangent (the difference of two states
+// with the same radial part) and kept in the column's basis. XtL: the low
 // parts of a compensated X^t (null pointers: none), XL those of the stage
 // state (null: stored as floats), so that Phi^t - Phi^(s) is taken from the
 // full values.
@@ -376,6 +368,7 @@ __device__ __forceinline__ void d_stage_init(const Geo<R>& G, const VR<R>& U, co
   if (c >= G.ncol) return;
   const int S = G.colp;
   const R gamma = pc<R>(ph.gamma, ph.gamma_f);
+  const Tan<R> tb = load_tan(G.tb, S, c);
   const bool cmp = XtL.rho != nullptr;
   int k0 = by * kchunk, k1 = min(G.nv + 1, k0 + kchunk);
 #pragma unroll 2
@@ -392,11 +385,12 @@ __device__ __forceinline__ void d_stage_init(const Geo<R>& G, const VR<R>& U, co
     if (k < G.nv) {
       if (zero) {
         P.rho[i] = P.th[i] = P.p[i] = R(0);
-        st4(P.m4, i, R(0), R(0), R(0), ld(T.theta + (i)));
+        st2(P.m2, i, R(0), R(0));
       } else {
         P.rho[i] = dif(Xt.rho, X.rho, XtL.rho, XL.rho);
-        st4(P.m4, i, dif(Xt.mx, X.mx, XtL.mx, XL.mx), dif(Xt.my, X.my, XtL.my, XL.my),
-            dif(Xt.mz, X.mz, XtL.mz, XL.mz), ld(T.theta + (i)));
+        const Q2<R> m = tan_to(tb, dif(Xt.mx, X.mx, XtL.mx, XL.mx), dif(Xt.my, X.my, XtL.my, XL.my),
+                               dif(Xt.mz, X.mz, XtL.mz, XL.mz));
+        st2(P.m2, i, m.x, m.y);
         P.th[i] = dif(Xt.th, X.th, XtL.th, XL.th);
         const R tht = cmp ? ld(Xt.th + (i)) + ld(XtL.th + (i)) : ld(Xt.th + (i));
         R ppt = eos_dev<R>(ld(U.pb + (k)), ld(U.thb + (k)), tht, gamma);
@@ -454,14 +448,16 @@ __device__ __forceinline__ void d_ss_lapd(const Geo<R>& G, const VR<R>& U, const
   }
 }
 
-// Eq. mom2 with the divergence damping: M* <- proj(M* + dtau(-grad q + S_M)),
+// Eq. mom2 with the divergence damping: M* <- M* + dtau(-grad q + S_M), in the
+// column's tangent basis (so Eq. proj_h is built into the weights),
 // q = p* + K_d lap D of d_ss_lapd, or p* itself without the damping;
 // in the last small step of a stage also M^(s+1) = M^(s) + M* into Xo (which
 // may be Xs itself: each cell reads its own Xs value before writing it), with
 // the low parts XsL -> XoL of a compensated state (null: none). Bound by the
 // gathers' latency (float) and by the float64 pipe's multiply-adds (float64):
-// with one gathered scalar instead of two, g6 x 32 float 28.7 -> 25.2 us,
-// float64 147 -> 84 us.
+// at g6 x 32, float 28.7 us with two gathered scalars and three Cartesian
+// components, 25.2 with one scalar, 18.1 in the tangent basis (80 -> 48
+// registers); float64 147 -> 84 -> 54 us.
 template <typename R>
 __device__ __forceinline__ void d_ss_mom(const Geo<R>& G, const VR<R>& U, const Slow<R>& SL, const Pert<R>& P, const Work<R>& T, R dtau,
                                             int divdamp, const Xf<R>& Xs, const Xf<R>& Xo, const Xf<R>& XsL, const Xf<R>& XoL, int last,
@@ -471,29 +467,28 @@ __device__ __forceinline__ void d_ss_mom(const Geo<R>& G, const VR<R>& U, const 
   const int S = G.colp;
   const uint64_t ps = pol_stream(), pk = pol_keep<R>();
   Nbr7 nb = load_nbr(G, c);
-  W7x3<R> wg = load_w7x3(G.wgrad, S, c);
-  R rx = ld(G.rhat + (c)), ry = ld(G.rhat + (S + c)), rz = ld(G.rhat + (2 * S + c));
+  W7x2<R> wg = load_w7x2(G.wg2, S, c);
   const R* q = divdamp ? T.lp : P.p;
   int k0 = by * kchunk, k1 = min(G.nv, k0 + kchunk);
 #pragma unroll 2
   for (int k = k0; k < k1; ++k) {
     const int o = k * S, i = o + c;
     R inv_r = ld(U.inv_rc + (k));
-    R gx = 0, gy = 0, gz = 0;
+    R g1 = 0, g2 = 0;
 #pragma unroll
     for (int j = 0; j < 7; ++j) {
       const R v = ldh(q + (o + nb.n[j]), pk);
-      gx += wg.x[j] * v;
-      gy += wg.y[j] * v;
-      gz += wg.z[j] * v;
+      g1 += wg.x[j] * v;
+      g2 += wg.y[j] * v;
     }
-    const Q4<R> m = ld4h(P.m4, (size_t)i, pk);
-    R mx = m.x + dtau * fmar<R>(-gx, inv_r, ldh(SL.smx + (i), ps));
-    R my = m.y + dtau * fmar<R>(-gy, inv_r, ldh(SL.smy + (i), ps));
-    R mz = m.z + dtau * fmar<R>(-gz, inv_r, ldh(SL.smz + (i), ps));
-    project(rx, ry, rz, mx, my, mz);
-    st4h(P.m4, i, mx, my, mz, m.w, pk);
+    Q2<R> m = ld2h(P.m2, (size_t)i, pk);
+    const Q2<R> sm = ld2h(SL.sm2, (size_t)i, ps);
+    m.x += dtau * fmar<R>(-g1, inv_r, sm.x);
+    m.y += dtau * fmar<R>(-g2, inv_r, sm.y);
+    st2h(P.m2, i, m.x, m.y, pk);
     if (last) {          // end of the stage: M^(s+1) = M^(s) + M*
+      R mx, my, mz;
+      tan_from(load_tan(G.tb, S, c), m, mx, my, mz);
       if (XoL.mx) {
         comp_add<R>(Xs.mx, XsL.mx, Xo.mx, XoL.mx, i, mx);
         comp_add<R>(Xs.my, XsL.my, Xo.my, XoL.my, i, my);
@@ -512,22 +507,25 @@ __device__ __forceinline__ void d_ss_mom(const Geo<R>& G, const VR<R>& U, const 
 //   a_k = rho*_k + dtau (S_rho,k - div_h M*_k)
 //   b_k = Th*_k + dtau (S_th,k - div_h(theta M*)_k)
 //   c_k = p*_k + Pi_k (b_k - Th*_k)        (p* advanced linearly in Th)
+// M* comes in the tangent basis of each neighbour (two multiply-adds per edge
+// instead of three); at g6 x 32 float64 107 -> 90 us (float64 pipe), float
+// 22.5 -> 22.9 us (latency: the gather of theta beside M* is its own load now)
 template <typename R>
 struct FluxCell {
   R dhm, a, b, c;
 };
 // the four values of cell i = o + column (o = level k's plane offset)
 template <typename R>
-__device__ __forceinline__ FluxCell<R> flux_cell(const W7x3<R>& wd, const Nbr7& nb, const VR<R>& U,
+__device__ __forceinline__ FluxCell<R> flux_cell(const W7x2<R>& wd, const Nbr7& nb, const VR<R>& U,
                                                  const Slow<R>& SL, const Pert<R>& P, const Work<R>& T, R dtau,
                                                  int k, int o, int i, uint64_t ps, uint64_t pk) {
   R dh = 0, dht = 0;
 #pragma unroll
   for (int j = 0; j < 7; ++j) {
-    const Q4<R> m = ld4h(P.m4, (size_t)(o + nb.n[j]), pk);    // M* and theta of the neighbour
-    R f = fmar<R>(wd.z[j], m.z, fmar<R>(wd.y[j], m.y, wd.x[j] * m.x));
+    const Q2<R> m = ld2h(P.m2, (size_t)(o + nb.n[j]), pk);    // M* of the neighbour in its basis
+    const R f = fmar<R>(wd.y[j], m.y, wd.x[j] * m.x);
     dh += f;
-    dht += m.w * f;
+    dht += ldh(T.theta + (o + nb.n[j]), ps) * f;
   }
   const R inv_r = ld(U.inv_rc + (k));
   const R thk = ldh(P.th + (i), pk);
@@ -547,7 +545,7 @@ __device__ __forceinline__ void d_ss_flux(const Geo<R>& G, const VR<R>& U, const
   const int S = G.colp;
   const uint64_t ps = pol_stream(), pk = pol_keep<R>();
   Nbr7 nb = load_nbr(G, c);
-  W7x3<R> wd = load_w7x3(G.wdiv, S, c);
+  W7x2<R> wd = load_w7x2(G.wd2, S, c);
   int k0 = by * kchunk, k1 = min(G.nv, k0 + kchunk);
 #pragma unroll 2
   for (int k = k0; k < k1; ++k) {
