@@ -697,6 +697,27 @@ int make_impl(thor_grid* grid, const thor_planet& pl, const thor_init& in, cudaS
   I->ph.kappa_f = (float)I->ph.kappa;
   I->ph.g_f = (float)I->ph.g;
   I->ph.two_omega_f = (float)I->ph.two_omega;
+  {
+    // g_k and the ranges of the truncated series: the remainder after g_n,
+    // sum over k > n of |g_k| x^k, at most eps
+    double gk[65] = {1.0};
+    for (int k = 1; k <= 64; ++k) gk[k] = gk[k - 1] * (I->ph.gamma - k) / (k + 1);
+    auto range = [&](int n, double eps) {
+      for (int e = 3; e < 60; ++e) {
+        const double x = std::ldexp(1.0, -e);
+        double rest = 0.0;
+        for (int k = 64; k > n; --k) rest = (rest + std::fabs(gk[k])) * x;
+        for (int k = 0; k < n; ++k) rest *= x;
+        if (rest <= eps) return x;
+      }
+      return 0.0;
+    };
+    for (int k = 0; k < 7; ++k) I->ph.pg[k] = gk[k + 1];
+    for (int k = 0; k < 3; ++k) I->ph.pg_f[k] = (float)gk[k + 1];
+    I->ph.x4 = range(4, std::ldexp(1.0, -55));
+    I->ph.x7 = range(7, std::ldexp(1.0, -55));
+    I->ph.x3_f = (float)range(3, std::ldexp(1.0, -26));
+  }
   I->ph.hydrostatic = in.hydrostatic ? 1 : 0;
   I->ph.vorder = in.vorder > 1 ? in.vorder : 1;
   I->ph.anelastic = in.anelastic ? 1 : 0;

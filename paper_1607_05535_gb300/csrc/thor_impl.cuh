@@ -54,7 +54,7 @@ struct Pert {
 // TMA descriptors of the planes the staged column solve reads (float storage):
 // each a 2-D map (x = column, y = plane) with a box of 32 columns x all planes
 struct SolveMaps {
-  CUtensorMap w, sw, cc, ca, thi, cb, pp, th_t, th_s, dsc, dhm;   // float
+  CUtensorMap w, sw, cc, ca, thi, cb, pi, th_t, th_s, dsc, dhm;   // float
   CUtensorMap q, inv, cf, junction;                             // float64 factors
 };
 

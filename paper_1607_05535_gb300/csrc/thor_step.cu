@@ -38,13 +38,14 @@ cudaError_t launch_k(void (*kern)(K...), dim3 grid, dim3 block, size_t smem, cud
 
 // ---------------------------------------------------------------- slow terms
 
-// Pointwise derived quantities at the stage state: p', T', theta, the full
+// Pointwise derived quantities at the stage state: p', Pi = gamma p / rho theta,
+// T', theta, the full
 // 3-D velocity, v_h = M/rho (centres) and v_r = W/rho (interfaces); the
 // velocities go into packed planes with theta (v4) and T' (vh4) beside them,
 // the fields the next stencils gather together.
 // HO: the order-k interpolation of the explicit terms (thor_init.vorder > 1)
 template <typename R, bool HO = false>
-__device__ __forceinline__ void d_derived(const Geo<R>& G, const VR<R>& U, const Phys& ph, const Xf<R>& X, const Work<R>& T, int shallow, int kchunk,
+__device__ __forceinline__ void d_derived(const Geo<R>& G, const VR<R>& U, const Phys& ph, const Xf<R>& X, const Work<R>& T, R* pi, int shallow, int kchunk,
                                           int bx, int by) {
   int c = bx * blockDim.x + threadIdx.x;
   if (c >= G.ncol) return;
@@ -65,8 +66,10 @@ __device__ __forceinline__ void d_derived(const Geo<R>& G, const VR<R>& U, const
       R wc = HO ? vint_centre(U, X.w, k, c, S, G.nv)
                            : ld(U.clo + (k)) * ld(X.w + (i)) + ld(U.chi + (k)) * ld(X.w + (i + S));
       R mx = ld(X.mx + (i)), my = ld(X.my + (i)), mz = ld(X.mz + (i));
-      const R theta = (ld(U.thb + (k)) + thp) * inv;
+      const R thfull = ld(U.thb + (k)) + thp;
+      const R theta = thfull * inv;
       T.pp[i] = pp;
+      pi[i] = gamma * p / thfull;
       T.theta[i] = theta;
       st4(T.v4, i, (mx + wc * rx) * inv, (my + wc * ry) * inv, (mz + wc * rz) * inv, theta);
       st4(T.vh4, i, mx * inv, my * inv, mz * inv, Temp - ld(U.Tb + (k)));
@@ -121,8 +124,7 @@ __device__ __forceinline__ void d_lap1(const Geo<R>& G, const VR<R>& U, const Xf
 // Slow tendencies at the centres (right-hand sides of Eqs. mom2, dens2, pt2):
 // S_M = -grad_h p - A_h - C_h + F_M, S_rho = -div(M) - div(W) + F_rho,
 // S_th = F_th - div(theta M) - div(theta W), plus Dsc = div(M) + div(W) of the
-// stage state (divergence damping), the radial advection+Coriolis and
-// Pi = gamma p / rho theta. In the first stage (stage state = X^t) Dsc is also
+// stage state (divergence damping) and the radial advection+Coriolis. In the first stage (stage state = X^t) Dsc is also
 // kept in d0: it is the divergence D that the first small step of every
 // stage damps, since there M^(s) + M* = M^t and W^(s) + W* = W^t.
 // SH: the shallow-atmosphere approximation of Sec. 3 (r = A in the tables;
@@ -144,9 +146,8 @@ __device__ __forceinline__ void d_slow(const Geo<R>& G, const VR<R>& U, const Ph
   load_w7x3_lap(G.wdiv, S, c, wd, wl);
   const R gcx = ld(G.gcor + (c)), gcy = ld(G.gcor + (S + c)), gcz = ld(G.gcor + (2 * S + c));
   R rx = ld(G.rhat + (c)), ry = ld(G.rhat + (S + c)), rz = ld(G.rhat + (2 * S + c));
-  const Tan<R> tb = load_tan(G.tb, S, c);
-  const R two_om = pc<R>(ph.two_omega, ph.two_omega_f), gamma = pc<R>(ph.gamma, ph.gamma_f),
-          Rd = pc<R>(ph.Rd, ph.Rd_f);
+  const R tA = ld(G.tb + (2 * S + c));
+  const R two_om = pc<R>(ph.two_omega, ph.two_omega_f), Rd = pc<R>(ph.Rd, ph.Rd_f);
   int k0 = by * kchunk, k1 = min(kend, k0 + kchunk);
   constexpr int kUnroll = sizeof(R) == sizeof(float) ? 2 : 1;   // float64: registers
 #pragma unroll kUnroll
@@ -154,9 +155,6 @@ __device__ __forceinline__ void d_slow(const Geo<R>& G, const VR<R>& U, const Ph
     const int o = k * S, i = o + c;
     const R inv_r = ld(U.inv_rc + (k)), inv_r2 = ld(U.inv_rc2 + (k));
     const R sql = ld(U.sq_lo + (k)), sqh = ld(U.sq_hi + (k));
-    R thfull = ld(U.thb + (k)) + ld(X.th + (i));
-    R p = ld(U.pb + (k)) + ld(T.pp + (i));
-
     // one pass over the 7-point neighbourhood, each neighbour value loaded
     // once: the edge flux f = w . M of the momentum (shared by the continuity,
     // advection and rho-theta divergences), the pressure gradient and the
@@ -203,8 +201,7 @@ __device__ __forceinline__ void d_slow(const Geo<R>& G, const VR<R>& U, const Ph
       FMx = -hx * inv_r2;
       FMy = -hy * inv_r2;
       FMz = -hz * inv_r2;
-      R Fp = -Rd * hT * inv_r2;
-      Fth = thfull / (gamma * p) * Fp;
+      Fth = -Rd * hT * inv_r2 / ld(SL.pi + (i));     // Th / (gamma p) F_p
     }
 
     // advection div(rho v v_j) of the Cartesian components (Sec. 3)
@@ -264,8 +261,10 @@ __device__ __forceinline__ void d_slow(const Geo<R>& G, const VR<R>& U, const Ph
     // the anelastic switch leaves the pressure force to the projection
     const R pgr = ph.anelastic ? R(0) : inv_r;
     // the tangential part of the sum, in the basis the small step works in
-    const Q2<R> sm = tan_to(tb, -gx * pgr - A[0] + FMx, -gy * pgr - A[1] + FMy, -gz * pgr - A[2] + FMz);
-    st2(SL.sm2, i, sm.x, sm.y);
+    // (tan_to with X = s rx, Y = s ry, s = sign(rz): one register instead of three)
+    const R sx = -gx * pgr - A[0] + FMx, sy = -gy * pgr - A[1] + FMy, sz = -gz * pgr - A[2] + FMz;
+    const R t = tA * (rx * sx + ry * sy) - (rz < R(0) ? -sz : sz);
+    st2(SL.sm2, i, sx + rx * t, sy + ry * t);
 
     R dh = sdh * inv_r;
     R dv = sqh * whi_w - sql * wlo_w;
@@ -280,7 +279,6 @@ __device__ __forceinline__ void d_slow(const Geo<R>& G, const VR<R>& U, const Ph
     R dvt = sqh * thhi * whi_w - sql * thlo * wlo_w;
     SL.sth[i] = Fth - dht - dvt;
     SL.acr[i] = acr;
-    SL.pi[i] = gamma * p / thfull;
   }
 }
 
@@ -301,7 +299,7 @@ __device__ __forceinline__ void d_slow_w(const Geo<R>& G, const VR<R>& U, const 
   Nbr7 nb = load_nbr(G, c);
   W7<R> wl = load_w7(G.wlap, S, c);
   const Tan<R> tb = load_tan(G.tb, S, c);
-  const R g = pc<R>(ph.g, ph.g_f), gamma = pc<R>(ph.gamma, ph.gamma_f);
+  const R g = pc<R>(ph.g, ph.g_f);
   int k0 = by * kchunk, k1 = min(G.nv + 1, k0 + kchunk);
 #pragma unroll 2
   for (int k = k0; k < k1; ++k) {
@@ -316,10 +314,9 @@ __device__ __forceinline__ void d_slow_w(const Geo<R>& G, const VR<R>& U, const 
       P.rho[i] = dif(Xt.rho, X.rho, XtL.rho);
       const Q2<R> m = tan_to(tb, dif(Xt.mx, X.mx, XtL.mx), dif(Xt.my, X.my, XtL.my), dif(Xt.mz, X.mz, XtL.mz));
       st2(P.m2, i, m.x, m.y);
-      P.th[i] = dif(Xt.th, X.th, XtL.th);
-      const R tht = XtL.th ? ld(Xt.th + (i)) + ld(XtL.th + (i)) : ld(Xt.th + (i));
-      R ppt = eos_dev<R>(ld(U.pb + (k)), ld(U.thb + (k)), tht, gamma);
-      P.p[i] = ppt - ld(T.pp + (i));
+      const R d = dif(Xt.th, X.th, XtL.th);
+      P.th[i] = d;
+      P.p[i] = p_pert(ph, ld(SL.pi + (i)), ld(U.thb + (k)) + ld(X.th + (i)), d);
     }
     if (init) P.w[i] = dif(Xt.w, X.w, XtL.w);
     // slow terms of Eq. momr2
@@ -355,19 +352,18 @@ __device__ __forceinline__ void d_slow_w(const Geo<R>& G, const VR<R>& U, const 
 
 // The perturbations at the start of a stage on their own (the state's step
 // runs this beside the slow terms): Phi* = Phi^t - Phi^(s), p* from the
-// nonlinear Eq. theta_to_p; all zero in the first stage, where Phi^(s) =
-// Phi^t and p^(s) = EOS(Th^t). M* is tangent (the difference of two states
+// nonlinear Eq. theta_to_p about the stage state (p_pert); all zero in the
+// first stage, where Phi^(s) = Phi^t. M* is tangent (the difference of two states
 // with the same radial part) and kept in the column's basis. XtL: the low
 // parts of a compensated X^t (null pointers: none), XL those of the stage
 // state (null: stored as floats), so that Phi^t - Phi^(s) is taken from the
 // full values.
 template <typename R>
-__device__ __forceinline__ void d_stage_init(const Geo<R>& G, const VR<R>& U, const Phys& ph, const Xf<R>& Xt, const Xf<R>& X, const Work<R>& T, const Pert<R>& P,
+__device__ __forceinline__ void d_stage_init(const Geo<R>& G, const VR<R>& U, const Phys& ph, const Xf<R>& Xt, const Xf<R>& X, const R* pi, const Pert<R>& P,
                                              const Xf<R>& XtL, const Xf<R>& XL, int zero, int kchunk, int bx, int by) {
   int c = bx * blockDim.x + threadIdx.x;
   if (c >= G.ncol) return;
   const int S = G.colp;
-  const R gamma = pc<R>(ph.gamma, ph.gamma_f);
   const Tan<R> tb = load_tan(G.tb, S, c);
   const bool cmp = XtL.rho != nullptr;
   int k0 = by * kchunk, k1 = min(G.nv + 1, k0 + kchunk);
@@ -391,10 +387,9 @@ __device__ __forceinline__ void d_stage_init(const Geo<R>& G, const VR<R>& U, co
         const Q2<R> m = tan_to(tb, dif(Xt.mx, X.mx, XtL.mx, XL.mx), dif(Xt.my, X.my, XtL.my, XL.my),
                                dif(Xt.mz, X.mz, XtL.mz, XL.mz));
         st2(P.m2, i, m.x, m.y);
-        P.th[i] = dif(Xt.th, X.th, XtL.th, XL.th);
-        const R tht = cmp ? ld(Xt.th + (i)) + ld(XtL.th + (i)) : ld(Xt.th + (i));
-        R ppt = eos_dev<R>(ld(U.pb + (k)), ld(U.thb + (k)), tht, gamma);
-        P.p[i] = ppt - ld(T.pp + (i));
+        const R d = dif(Xt.th, X.th, XtL.th, XL.th);
+        P.th[i] = d;
+        P.p[i] = p_pert(ph, ld(pi + (i)), ld(U.thb + (k)) + ld(X.th + (i)), d);
       }
     }
     P.w[i] = zero ? R(0) : dif(Xt.w, X.w, XtL.w, XL.w);
@@ -874,7 +869,6 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
   __syncthreads();
   // Eqs. dens2, pt2, theta_to_p with the new W*; the two warps share the levels
   if (valid) {
-    const R gamma = pc<R>(ph.gamma, ph.gamma_f);
 #pragma unroll 4
     for (int k = half; k < nv; k += 2) {
       const int i = k * S + c;
@@ -886,10 +880,8 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
       const R rho_new = ld(T.ca + i) - rdt * (eh * wh - el * wl);
       P.rho[i] = rho_new;
       P.th[i] = th_new;
-      // p* = EOS(Th^(s) + Th*) - p^(s) = p^(s) ((1 + Th*/Th^(s))^gamma - 1)
-      R ps = ld(U.pb + k) + ld(T.pp + i);
-      R ths = ld(U.thb + k) + ld(Xs.th + i);
-      P.p[i] = ps * rexpm1<R>(gamma * rlog1p<R>(th_new / ths));
+      // p* = EOS(Th^(s) + Th*) - p^(s)
+      P.p[i] = p_pert(ph, ld(SL.pi + i), ld(U.thb + k) + ld(Xs.th + i), th_new);
       if (k >= 1) P.w[i] = wl;
       // 3-D divergence of the new total momentum, for the next small step's
       // divergence damping: D^(s) + div_h M* (from k_ss_flux) + div_v W*
@@ -1065,8 +1057,8 @@ __global__ void k_energy_fix(Geo<R> G, VR<R> U, Phys ph, Xf<R> X, Xf<R> XL, cons
 // ---------------------------------------------------------------- kernels: one state
 
 template <typename R, bool HO>
-__global__ void k_derived(Geo<R> G, VR<R> U, Phys ph, Xf<R> X, Work<R> T, int shallow, int kchunk) {
-  d_derived<R, HO>(G, U, ph, X, T, shallow, kchunk, blockIdx.x, blockIdx.y);
+__global__ void k_derived(Geo<R> G, VR<R> U, Phys ph, Xf<R> X, Work<R> T, R* pi, int shallow, int kchunk) {
+  d_derived<R, HO>(G, U, ph, X, T, pi, shallow, kchunk, blockIdx.x, blockIdx.y);
 }
 template <typename R, bool HO>
 __global__ void k_lap1(Geo<R> G, VR<R> U, Xf<R> X, Work<R> T, R Kd, int kchunk, int klo, int kend) {
@@ -1084,9 +1076,9 @@ __global__ void k_slow_w(Geo<R> G, VR<R> U, Phys ph, Xf<R> Xt, Xf<R> X, Work<R> 
   d_slow_w<R, HO>(G, U, ph, Xt, X, T, SL, P, hyper, init, kchunk, blockIdx.x, blockIdx.y);
 }
 template <typename R>
-__global__ void k_stage_init(Geo<R> G, VR<R> U, Phys ph, Xf<R> Xt, Xf<R> X, Work<R> T, Pert<R> P, Xf<R> XtL,
+__global__ void k_stage_init(Geo<R> G, VR<R> U, Phys ph, Xf<R> Xt, Xf<R> X, const R* pi, Pert<R> P, Xf<R> XtL,
                              Xf<R> XL, int zero, int kchunk) {
-  d_stage_init<R>(G, U, ph, Xt, X, T, P, XtL, XL, zero, kchunk, blockIdx.x, blockIdx.y);
+  d_stage_init<R>(G, U, ph, Xt, X, pi, P, XtL, XL, zero, kchunk, blockIdx.x, blockIdx.y);
 }
 // the small-step stencils take a level range [kchunk * klo, khi) (klo in
 // chunks), so that the lower and upper levels can run as separate launches
@@ -1187,7 +1179,7 @@ __device__ __forceinline__ void solve_issue(const SolveSm& s, const SolveMaps& M
   tma_load_2d(s.junc, &M.junction, c0, 0, bar, ps);
   tma_prefetch_2d(&M.thi, c0, 0, ps);
   tma_prefetch_2d(&M.cb, c0, 0, pk);
-  tma_prefetch_2d(&M.pp, c0, 0, ps);
+  tma_prefetch_2d(&M.pi, c0, 0, ps);
   tma_prefetch_2d(stage0 ? &M.th_t : &M.th_s, c0, 0, ps);
   if (want_div) {
     tma_prefetch_2d(&M.dsc, c0, 0, ps);
@@ -1269,7 +1261,7 @@ __device__ __forceinline__ void solve_sweeps(const SolveSm& s, float2* sx, const
 // Operands of the final updates (Eqs. dens2, pt2, theta_to_p) of one cell
 // that do not depend on the solved W*.
 struct UpdOps {
-  float thl, thh, cb, ps, ths, dsc, dhm;
+  float thl, thh, cb, pi, ths, dsc, dhm;
 };
 __device__ __forceinline__ UpdOps upd_load(const Geo<float>& G, const VR<float>& U, const Xf<float>& Xs,
                                            const Slow<float>& SL, const Work<float>& T, int want_div, int k,
@@ -1279,7 +1271,7 @@ __device__ __forceinline__ UpdOps upd_load(const Geo<float>& G, const VR<float>&
   o.thl = k > 0 ? ldh(SL.thi + i, ps) : 0.f;
   o.thh = k + 1 < nv ? ldh(SL.thi + (i + S), ps) : 0.f;
   o.cb = ldh(T.cb + i, pk);
-  o.ps = ld(U.pb + k) + ldh(T.pp + i, ps);
+  o.pi = ldh(SL.pi + i, ps);
   o.ths = ld(U.thb + k) + ldh(Xs.th + i, ps);
   o.dsc = want_div ? ldh(SL.dsc + i, ps) : 0.f;
   o.dhm = want_div ? ldh(T.dhm + i, pk) : 0.f;
@@ -1302,7 +1294,7 @@ __device__ __forceinline__ void upd_apply(const SolveSm& s, const UpdOps& o, con
   const float rho_new = s.ca[q] - rdt * (eh * wh - el * wl);
   sth(P.rho + i, rho_new, pk);
   sth(P.th + i, th_new, pk);
-  sth(P.p + i, o.ps * rexpm1<float>(ph.gamma_f * rlog1p<float>(th_new / o.ths)), pk);
+  sth(P.p + i, p_pert(ph, o.pi, o.ths, th_new), pk);
   if (k >= 1) sth(P.w + i, wl, pk);
   if (want_div) sth(T.dd + i, o.dsc + o.dhm + (eh * wh - el * wl), pk);
   if (last) stage_end_cell(Xs, Xo, XsL, XoL, P, rho_new, th_new, wl, k, i, S, nv);
@@ -1385,9 +1377,9 @@ template <typename R>
 __global__ void ke_derived(const Member<R>* __restrict__ M, const int2* __restrict__ map, int s, int kchunk) {
   THOR_MEMBER();
   if (a.ph.vorder > 1)
-    d_derived<R, true>(a.G, a.U, a.ph, Xs, a.T, a.shallow, kchunk, e.y, blockIdx.y);
+    d_derived<R, true>(a.G, a.U, a.ph, Xs, a.T, a.SL.pi, a.shallow, kchunk, e.y, blockIdx.y);
   else
-    d_derived<R>(a.G, a.U, a.ph, Xs, a.T, a.shallow, kchunk, e.y, blockIdx.y);
+    d_derived<R>(a.G, a.U, a.ph, Xs, a.T, a.SL.pi, a.shallow, kchunk, e.y, blockIdx.y);
 }
 template <typename R>
 __global__ void ke_lap1(const Member<R>* __restrict__ M, const int2* __restrict__ map, int s, int kchunk) {
@@ -1569,7 +1561,7 @@ int Impl<R>::large_step(double dt, int n_small) {
     cudaStream_t aux = fork ? side : stream;
     mark(THOR_K_DERIVED, true);
     const bool ho = ph.vorder > 1;
-    chk(launch_k(ho ? k_derived<R, true> : k_derived<R, false>, g2i, bs, 0, stream, G, U, ph, Xs, T, shallow, kc));
+    chk(launch_k(ho ? k_derived<R, true> : k_derived<R, false>, g2i, bs, 0, stream, G, U, ph, Xs, T, SL.pi, shallow, kc));
     mark(THOR_K_DERIVED, false);
     ++launches;
     if (fork) {
@@ -1577,7 +1569,7 @@ int Impl<R>::large_step(double dt, int n_small) {
       chk(cudaStreamWaitEvent(side, ev_fork, 0));
     }
     mark(THOR_K_STAGE_INIT, true);
-    chk(launch_k(k_stage_init<R>, g2i, bs, 0, aux, G, U, ph, Xt, Xs, T, P, XtL, XsL, (int)(s == 0), kc));
+    chk(launch_k(k_stage_init<R>, g2i, bs, 0, aux, G, U, ph, Xt, Xs, (const R*)SL.pi, P, XtL, XsL, (int)(s == 0), kc));
     mark(THOR_K_STAGE_INIT, false);
     ++launches;
     const bool early_grad = divdamp && s > 0;    // D of X^t is ready before the slow terms
@@ -1706,7 +1698,7 @@ int Impl<R>::anelastic_step(double dt) {
   const bool ho = ph.vorder > 1;
   for (int s = 0; s < 3; ++s) {
     Xf<R> Xs = s == 0 ? Xt : Xst, Xo = s == 2 ? Xt : Xst;
-    if (launch_k(ho ? k_derived<R, true> : k_derived<R, false>, g2i, bs, 0, stream, G, U, ph, Xs, T, shallow, kc))
+    if (launch_k(ho ? k_derived<R, true> : k_derived<R, false>, g2i, bs, 0, stream, G, U, ph, Xs, T, SL.pi, shallow, kc))
       return -3;
     if (hyper && launch_k(ho ? k_lap1<R, true> : k_lap1<R, false>, g2i, bs, 0, stream, G, U, Xs, T, Kd, kc, 0,
                           G.nv + 1))
@@ -1785,7 +1777,7 @@ int Impl<float>::build_solve_maps() {
   make(&map->cc, T.cc, nv, false);
   make(&map->ca, T.ca, nv, false);
   make(&map->cb, T.cb, nv, false);
-  make(&map->pp, T.pp, nv, false);
+  make(&map->pi, SL.pi, nv, false);
   make(&map->th_t, Xt.th, nv, false);
   make(&map->th_s, Xst.th, nv, false);
   make(&map->dsc, SL.dsc, nv, false);
