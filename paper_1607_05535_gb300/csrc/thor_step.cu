@@ -9,7 +9,7 @@
 //
 // The vertical solve is split: k_ss_flux (a stencil kernel like the others)
 // forms the per-cell parts of the column equations, and k_ss_solve runs the
-// float64 tridiagonal elimination with two warps per 32 columns.
+// tridiagonal elimination with two sweeping warps per 32 columns.
 #include "../../include/thor.h"
 #include "thor_impl.cuh"
 #include "thor_reduce.cuh"
@@ -520,7 +520,7 @@ __device__ __forceinline__ FluxCell<R> flux_cell(const W7x2<R>& wd, const Nbr7& 
     const Q2<R> m = ld2h(P.m2, (size_t)(o + nb.n[j]), pk);    // M* of the neighbour in its basis
     const R f = fmar<R>(wd.y[j], m.y, wd.x[j] * m.x);
     dh += f;
-    dht += ldh(T.theta + (o + nb.n[j]), ps) * f;
+    dht += ldh(T.theta + (o + nb.n[j]), pk) * f;
   }
   const R inv_r = ld(U.inv_rc + (k));
   const R thk = ldh(P.th + (i), pk);
@@ -705,6 +705,8 @@ __device__ __forceinline__ void stage_end_cell(const Xf<R>& Xs, const Xf<R>& Xo,
   if (k == nv - 1) Xo.w[i + S] = ld(Xs.w + (i + S)) + ld(P.w + (i + S));
 }
 
+constexpr int kSolveWarps = 8;     // warps of a column solve's block
+
 // the solved W* of row o of the direct solve's shared array: a float64
 // value, or for float storage the float in the first word of the row
 template <typename R>
@@ -724,7 +726,13 @@ __device__ __forceinline__ R solved_w(const double* sdp, int o) {
 // x_p+1 = f'_p+1 - e'_p+1 x_p, then back substitution outwards), in float64
 // for float64 states and in double-float for float-storage states; then
 // rho* and Th* follow from Eqs. dens2 and pt2 and p* from the nonlinear Eq.
-// theta_to_p. One block = 32 columns x 2 warps.
+// theta_to_p. One block = 32 columns x 8 warps: two of them sweep, all share
+// the levels of the final updates and, in float64, of the right-hand sides
+// (rh_m / piv_m into shared memory before the sweeps, which then hold one
+// multiply-add per row). A float64 warp instruction holds its sub-partition's
+// pipe for 80 cycles, so work on two warps alone takes four times as long on
+// a grid with fewer blocks than SMs: g4 x 20 float64 31.8 -> 17.3 us;
+// at g6 x 32, where the pipe is busy either way, 105.8 -> 105.5 us.
 template <typename R>
 __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, const Phys& ph, const Xf<R>& Xs, const Slow<R>& SL,
                                             const Pert<R>& P, const Work<R>& T, const Fac<R>& F, double dtau,
@@ -732,13 +740,13 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
                                             int by) {
   extern __shared__ double sm[];
   const int nv = G.nv, S = G.colp, N = nv - 1;
-  const int tx = threadIdx.x & 31, half = threadIdx.x >> 5;
+  const int tx = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int c = bx * 32 + tx;
   const bool valid = c < G.ncol;
   const int cs = valid ? c : 0;          // padding lanes read column 0 and store nothing
   double* sdp = sm;                      // [nv + 1][32] d' / f', then W
   double* sx = sdp + (nv + 1) * 32;      // [2][32] junction values
-  double* scf = sx + 64;                 // [nv + 1][32] c' / e', fetched during the sweeps
+  double* scf = sx + 64;                 // [nv + 1][32] c' / e', fetched during the sweeps (float64: q before)
   const int p = N / 2 > 0 ? N / 2 : 1;
   const R rdt = (R)dtau, g = pc<R>(ph.g, ph.g_f), delta = pc<R>(ph.delta, ph.delta_f);
 
@@ -758,7 +766,7 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
     float2* dp2 = reinterpret_cast<float2*>(sdp);
     float2* sx2 = reinterpret_cast<float2*>(sx);
     float2* cf2 = reinterpret_cast<float2*>(scf);
-    if (half == 0) {
+    if (warp == 0) {
       float2 d1 = make_float2(0.f, 0.f);
 #pragma unroll 4
       for (int m = 1; m <= p; ++m) {
@@ -767,7 +775,7 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
         d1 = df_sweep(rhs_r(m), Finv[i], Fq[i], d1);
         dp2[m * 32 + tx] = d1;
       }
-    } else {
+    } else if (warp == 1) {
       float2 f1 = make_float2(0.f, 0.f);
 #pragma unroll 4
       for (int m = N; m > p; --m) {
@@ -778,7 +786,7 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
       }
     }
     __syncthreads();
-    if (half == 0) {
+    if (warp == 0) {
       float2 xp, xq = make_float2(0.f, 0.f);
       if (p < N) {
         const float2 dp_ = dp2[p * 32 + tx], fq = dp2[(p + 1) * 32 + tx];
@@ -791,7 +799,7 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
       sx2[32 + tx] = xq;
     }
     __syncthreads();
-    if (half == 0) {
+    if (warp == 0) {
       float2 x = sx2[tx];
       dp2[p * 32 + tx] = make_float2(df_to_float(x), 0.f);
       for (int m = p - 1; m >= 1; --m) {
@@ -800,7 +808,7 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
         dp2[m * 32 + tx] = make_float2(df_to_float(x), 0.f);
       }
       dp2[tx] = make_float2(0.f, 0.f);             // bottom interface
-    } else {
+    } else if (warp == 1) {
       float2 x = sx2[32 + tx];
       if (p < N) dp2[(p + 1) * 32 + tx] = make_float2(df_to_float(x), 0.f);
       for (int m = p + 2; m <= N; ++m) {
@@ -812,28 +820,33 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
     }
   } else {
     // float64 storage: the elimination in float64
-    auto rhs = [&](int m) { return (double)rhs_r(m); };
-    if (half == 0) {
+    for (int m = 1 + warp; m <= N; m += kSolveWarps) {
+      const int i = m * S + cs;
+      sdp[m * 32 + tx] = rhs_r(m) * ld(F.inv + i);
+      scf[m * 32 + tx] = ld(F.q + i);
+    }
+    __syncthreads();
+    if (warp == 0) {
       double d1 = 0.0;
 #pragma unroll 4
       for (int m = 1; m <= p; ++m) {
-        const int i = m * S + cs;
-        scf[m * 32 + tx] = ld(F.cf + i);
-        d1 = fma(-ld(F.q + i), d1, rhs(m) * ld(F.inv + i));
-        sdp[m * 32 + tx] = d1;
+        const int o = m * 32 + tx;
+        d1 = fma(-scf[o], d1, sdp[o]);
+        sdp[o] = d1;
+        scf[o] = ld(F.cf + (m * S + cs));
       }
-    } else {
+    } else if (warp == 1) {
       double f1 = 0.0;
 #pragma unroll 4
       for (int m = N; m > p; --m) {
-        const int i = m * S + cs;
-        scf[m * 32 + tx] = ld(F.cf + i);
-        f1 = fma(-ld(F.q + i), f1, rhs(m) * ld(F.inv + i));
-        sdp[m * 32 + tx] = f1;
+        const int o = m * 32 + tx;
+        f1 = fma(-scf[o], f1, sdp[o]);
+        sdp[o] = f1;
+        scf[o] = ld(F.cf + (m * S + cs));
       }
     }
     __syncthreads();
-    if (half == 0) {
+    if (warp == 0) {
       double xp, xq = 0.0;
       if (p < N) {
         const double cp_ = scf[p * 32 + tx], eq = scf[(p + 1) * 32 + tx];
@@ -848,7 +861,7 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
     }
     __syncthreads();
     // back substitution, each warp over its own rows
-    if (half == 0) {
+    if (warp == 0) {
       double x = sx[tx];
       sdp[p * 32 + tx] = x;
       for (int m = p - 1; m >= 1; --m) {
@@ -856,7 +869,7 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
         sdp[m * 32 + tx] = x;
       }
       sdp[tx] = 0.0;                 // bottom interface
-    } else {
+    } else if (warp == 1) {
       double x = sx[32 + tx];
       if (p < N) sdp[(p + 1) * 32 + tx] = x;
       for (int m = p + 2; m <= N; ++m) {
@@ -867,10 +880,10 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
     }
   }
   __syncthreads();
-  // Eqs. dens2, pt2, theta_to_p with the new W*; the two warps share the levels
+  // Eqs. dens2, pt2, theta_to_p with the new W*; the warps share the levels
   if (valid) {
 #pragma unroll 4
-    for (int k = half; k < nv; k += 2) {
+    for (int k = warp; k < nv; k += kSolveWarps) {
       const int i = k * S + c;
       const R wl = solved_w<R>(sdp, k * 32 + tx), wh = solved_w<R>(sdp, (k + 1) * 32 + tx);
       const R thl = k > 0 ? ld(SL.thi + i) : R(0);
@@ -1108,7 +1121,7 @@ __global__ void __launch_bounds__(64) k_ss_factor(Geo<R> G, VR<R> U, Phys ph, Sl
   d_ss_factor<R>(G, U, ph, SL, F, dtau, blockIdx.x, 0);
 }
 template <typename R>
-__global__ void __launch_bounds__(64) k_ss_solve(Geo<R> G, VR<R> U, Phys ph, Xf<R> Xs, Slow<R> SL, Pert<R> P,
+__global__ void __launch_bounds__(32 * kSolveWarps) k_ss_solve(Geo<R> G, VR<R> U, Phys ph, Xf<R> Xs, Slow<R> SL, Pert<R> P,
                                                  Work<R> T, Fac<R> F, double dtau, int want_div, Xf<R> Xo,
                                                  Xf<R> XsL, Xf<R> XoL, int last) {
   d_ss_solve<R>(G, U, ph, Xs, SL, P, T, F, dtau, want_div, Xo, XsL, XoL, last, blockIdx.x, 0);
@@ -1135,8 +1148,6 @@ __global__ void k_physics(Geo<R> G, VR<R> U, Phys ph, Xf<R> X, Xf<R> XL, Work<R>
 // used); afterwards all eight warps share the levels of Eqs. dens2, pt2 and
 // theta_to_p, whose loads now hit L2. Same operations in the same order as
 // d_ss_solve.
-
-constexpr int kSolveWarps = 8;
 
 // one column group's planes in shared memory (32 columns)
 struct SolveSm {
@@ -1447,7 +1458,7 @@ __global__ void ke_ss_flux(const Member<R>* __restrict__ M, const int2* __restri
   d_ss_flux<R>(G, a.U, a.SL, a.P, a.T, (R)a.dts[s], kchunk, e.y, blockIdx.y + klo);
 }
 template <typename R>
-__global__ void __launch_bounds__(64)
+__global__ void __launch_bounds__(32 * kSolveWarps)
     ke_ss_solve(const Member<R>* __restrict__ M, const int2* __restrict__ map, int s, int j) {
   THOR_MEMBER();
   const int want_div = a.divdamp && j + 1 < a.nsub[s];
@@ -1649,7 +1660,7 @@ int Impl<R>::large_step(double dt, int n_small) {
       if (staged)
         chk(launch_solve_tma(gsolve, s, Xo, XsL, XoL, dts[s], want_div, last));
       else
-        chk(launch_k(k_ss_solve<R>, gsolve, 64, solve_smem, stream, G, U, ph, Xs, SL, P, T, F, dts[s],
+        chk(launch_k(k_ss_solve<R>, gsolve, 32 * kSolveWarps, solve_smem, stream, G, U, ph, Xs, SL, P, T, F, dts[s],
                      want_div, Xo, XsL, XoL, last));
       mark(THOR_K_SS_SOLVE, false);
       ++launches;
@@ -1851,9 +1862,9 @@ int ensemble_large_step(const EnsPlan<R>& E, cudaStream_t stream, long long* lau
         if (E.staged)
           ke_ss_solve_tma<<<nbc, 32 * kSolveWarps, solve_tma_smem_bytes(E.nv), stream>>>(M, E.mapc, s, j);
         else
-          ke_ss_solve<R><<<nbc, 64, solve_smem, stream>>>(M, E.mapc, s, j);
+          ke_ss_solve<R><<<nbc, 32 * kSolveWarps, solve_smem, stream>>>(M, E.mapc, s, j);
       } else {
-        ke_ss_solve<R><<<nbc, 64, solve_smem, stream>>>(M, E.mapc, s, j);
+        ke_ss_solve<R><<<nbc, 32 * kSolveWarps, solve_smem, stream>>>(M, E.mapc, s, j);
       }
       ++n;
     }
