@@ -129,7 +129,8 @@ struct Carver {
 template <typename R>
 std::vector<const R**> vr_slots(VR<R>& U) {
   return {&U.inv_rc, &U.inv_rc2, &U.sv, &U.ri2, &U.wlo, &U.whi, &U.clo, &U.chi, &U.inv_dzc,
-          &U.rhob, &U.thb, &U.pb, &U.Tb, &U.Rb, &U.zc, &U.sq_lo, &U.sq_hi};
+          &U.rhob, &U.thb, &U.pb, &U.Tb, &U.Rb, &U.zc, &U.sq_lo, &U.sq_hi, &U.inv_thb, &U.inv_ri2,
+          &U.lnp0, &U.pk0, &U.hjT};
 }
 
 template <typename R>
@@ -188,6 +189,7 @@ void carve(Carver& cv, Impl<R>& I, int ncol, int nv) {
   const double** vi[] = {&I.V.ri, &I.V.dzc, &I.V.wlo, &I.V.whi, &I.V.Rb, &I.V.ri2, &I.V.inv_dzc};
   for (const double** p : vi) *p = cv.take<double>(nv + 1);
   for (const R** p : vr_slots(I.U)) *p = cv.take<R>(nv + 1);
+  I.U.pw = sizeof(R) == sizeof(double) ? cv.take<double>(kPowRows * kPowCols) : nullptr;
   I.U.iw = cv.take<R>(4 * (size_t)(nv + 1));
   I.U.cw = cv.take<R>(4 * (size_t)nv);
   I.U.ij0 = cv.take<int>(nv + 1);
@@ -206,6 +208,35 @@ struct HostSetup {
   std::vector<double> iw, cw;     // [4][nv + 1], [4][nv]
   std::vector<int> ij0, cj0;      // [nv + 1], [nv]
 };
+// ((1 + x)^a - 1) / (a x) = 1 + g_1 x + g_2 x^2 + ... (Newton's binomial
+// series), and the largest power of two x at which the remainder after g_n,
+// sum over k > n of |g_k| x^k, is at most eps
+struct PowSeries {
+  double g[65];
+  explicit PowSeries(double a) {
+    g[0] = 1.0;
+    for (int k = 1; k <= 64; ++k) g[k] = g[k - 1] * (a - k) / (k + 1);
+  }
+  double range(int n, double eps) const {
+    for (int e = 3; e < 60; ++e) {
+      const double x = std::ldexp(1.0, -e);
+      double rest = 0.0;
+      for (int k = 64; k > n; --k) rest = (rest + std::fabs(g[k])) * x;
+      for (int k = 0; k < n; ++k) rest *= x;
+      if (rest <= eps) return x;
+    }
+    return 0.0;
+  }
+};
+// pow1p and the physics' (1 + y)^(1 / gamma) keep g1 .. g6: exact to float64
+// rounding up to 1/128, where the result can be small, and to 2^-46 of the
+// last table interval's small share beyond
+bool pow_series_ok(double gamma) {
+  const double eps = std::ldexp(1.0, -55);
+  return PowSeries(gamma).range(6, eps) >= 1.0 / 128 && PowSeries(1.0 / gamma).range(6, eps) >= 1.0 / 128 &&
+         PowSeries(gamma).range(6, std::ldexp(1.0, -47)) >= 1.0 / 64;
+}
+
 template <typename R>
 int upload_tables(Impl<R>& I, const HostGrid& h, const std::vector<double>* vert, const HostSetup* lag,
                   cudaStream_t st) {
@@ -295,7 +326,7 @@ int upload_tables(Impl<R>& I, const HostGrid& h, const std::vector<double>* vert
   // storage-type copies with the reciprocals precomputed
   {
     const std::vector<double>& rc = vert[0];
-    std::vector<std::vector<R>> vr(17, std::vector<R>(nv + 1, R(0)));
+    std::vector<std::vector<R>> vr(22, std::vector<R>(nv + 1, R(0)));
     for (int k = 0; k < nv; ++k) {
       vr[0][k] = (R)(1.0 / rc[k]);
       vr[1][k] = (R)(1.0 / (rc[k] * rc[k]));
@@ -309,16 +340,35 @@ int upload_tables(Impl<R>& I, const HostGrid& h, const std::vector<double>* vert
       vr[14][k] = (R)vert[4][k];
       vr[15][k] = (R)vert[10][k];
       vr[16][k] = (R)vert[11][k];
+      vr[17][k] = (R)(1.0 / vert[6][k]);
+      vr[19][k] = (R)std::log(vert[7][k] / 1.0e5);
+      vr[20][k] = (R)std::pow(vert[7][k] / 1.0e5, I.ph.kappa);
+      // Eq. tvert: z_stra 2e6 m, T_surf 1600 K, Gamma 2e-4 K/m, dT 10 K
+      const double d = 0.5 * 2.0e-4 * (vert[4][k] - 2.0e6);
+      vr[21][k] = (R)(vert[4][k] <= 2.0e6 ? 1600.0 - 2.0e-4 * 2.0e6 - d + std::sqrt(d * d + 100.0)
+                                          : 1600.0 - 2.0e-4 * 2.0e6 + 10.0);
     }
     for (int i = 0; i <= nv; ++i) {
       vr[3][i] = (R)vert[17][i];
+      vr[18][i] = (R)(1.0 / vert[17][i]);
       vr[4][i] = (R)vert[14][i];
       vr[5][i] = (R)vert[15][i];
       vr[8][i] = (R)vert[18][i];
       vr[13][i] = (R)vert[16][i];
     }
     std::vector<const R**> slots = vr_slots(I.U);
-    for (int j = 0; j < 17; ++j) e = e ? e : up(*slots[j], vr[j].data(), (nv + 1) * sizeof(R));
+    for (size_t j = 0; j < slots.size(); ++j) e = e ? e : up(*slots[j], vr[j].data(), (nv + 1) * sizeof(R));
+    // pow1p's table, where its series reach float64 precision for this gamma
+    std::vector<double> pw((size_t)kPowRows * kPowCols, 0.0);
+    if (I.U.pw && !pow_series_ok(I.ph.gamma)) I.U.pw = nullptr;
+    if (I.U.pw) {
+      for (int j = 0; j < kPowRows; ++j) {
+        const double c = 0.5 + j / 64.0, l = std::log1p(c - 1.0);
+        const double row[kPowCols] = {c - 1.0, 1.0 / c, std::expm1(I.ph.gamma * l), std::exp(I.ph.gamma * l), l, 0.0};
+        std::copy(row, row + kPowCols, pw.begin() + (size_t)j * kPowCols);
+      }
+      e = e ? e : up(I.U.pw, pw.data(), pw.size() * sizeof(double));
+    }
     std::vector<R> iw(lag->iw.begin(), lag->iw.end()), cw(lag->cw.begin(), lag->cw.end());
     e = e ? e : up(I.U.iw, iw.data(), iw.size() * sizeof(R));
     e = e ? e : up(I.U.cw, cw.data(), cw.size() * sizeof(R));
@@ -698,25 +748,13 @@ int make_impl(thor_grid* grid, const thor_planet& pl, const thor_init& in, cudaS
   I->ph.g_f = (float)I->ph.g;
   I->ph.two_omega_f = (float)I->ph.two_omega;
   {
-    // g_k and the ranges of the truncated series: the remainder after g_n,
-    // sum over k > n of |g_k| x^k, at most eps
-    double gk[65] = {1.0};
-    for (int k = 1; k <= 64; ++k) gk[k] = gk[k - 1] * (I->ph.gamma - k) / (k + 1);
-    auto range = [&](int n, double eps) {
-      for (int e = 3; e < 60; ++e) {
-        const double x = std::ldexp(1.0, -e);
-        double rest = 0.0;
-        for (int k = 64; k > n; --k) rest = (rest + std::fabs(gk[k])) * x;
-        for (int k = 0; k < n; ++k) rest *= x;
-        if (rest <= eps) return x;
-      }
-      return 0.0;
-    };
-    for (int k = 0; k < 7; ++k) I->ph.pg[k] = gk[k + 1];
-    for (int k = 0; k < 3; ++k) I->ph.pg_f[k] = (float)gk[k + 1];
-    I->ph.x4 = range(4, std::ldexp(1.0, -55));
-    I->ph.x7 = range(7, std::ldexp(1.0, -55));
-    I->ph.x3_f = (float)range(3, std::ldexp(1.0, -26));
+    const PowSeries a(I->ph.gamma), b(I->ph.inv_gamma);
+    for (int k = 0; k < 7; ++k) I->ph.pg[k] = a.g[k + 1];
+    for (int k = 0; k < 6; ++k) I->ph.qg[k] = b.g[k + 1];
+    for (int k = 0; k < 3; ++k) I->ph.pg_f[k] = (float)a.g[k + 1];
+    I->ph.x4 = a.range(4, std::ldexp(1.0, -55));
+    I->ph.x7 = a.range(7, std::ldexp(1.0, -55));
+    I->ph.x3_f = (float)a.range(3, std::ldexp(1.0, -26));
   }
   I->ph.hydrostatic = in.hydrostatic ? 1 : 0;
   I->ph.vorder = in.vorder > 1 ? in.vorder : 1;

@@ -60,6 +60,10 @@ struct VR {
   const R *inv_rc, *inv_rc2, *sv, *ri2, *wlo, *whi, *clo, *chi, *inv_dzc;
   const R *rhob, *thb, *pb, *Tb, *Rb, *zc;
   const R *sq_lo, *sq_hi;
+  const R *inv_thb, *inv_ri2;      // 1 / thb, 1 / ri2
+  // Held-Suarez: ln(pb / p0) and (pb / p0)^kappa, p0 = 1e5 Pa; hot Jupiter: T_vert of the level
+  const R *lnp0, *pk0, *hjT;
+  const double* pw;                // pow1p's table (float64 states; null: not valid for this gamma)
   // Lagrange interpolation of order k > 1 in the explicit terms (Sec. 2.1):
   // interface m (1..nv-1) from centres ij0[m] + j with weights iw[j][m];
   // centre c from interfaces cj0[c] + j with weights cw[j][c]; j < 4, the
@@ -104,6 +108,7 @@ struct Phys {
   // through g4 and g7 in float64, through g3 in float32 (p_pert); set on the host
   double pg[7] = {};
   double x4 = 0.0, x7 = 0.0;
+  double qg[6] = {};                // the same for the exponent 1 / gamma
   float pg_f[3] = {};
   float x3_f = 0.0f;
   // hydrostatic switch (Sec. 3): delta on the vertical momentum's inertia,
@@ -157,6 +162,9 @@ template <> __device__ __forceinline__ float rexp<float>(float x) { return expf(
 template <typename R> __device__ __forceinline__ R rpow(R x, R y);
 template <> __device__ __forceinline__ double rpow<double>(double x, double y) { return pow(x, y); }
 template <> __device__ __forceinline__ float rpow<float>(float x, float y) { return powf(x, y); }
+template <typename R> __device__ __forceinline__ R rsinpi(R x);      // sin(pi x)
+template <> __device__ __forceinline__ double rsinpi<double>(double x) { return sinpi(x); }
+template <> __device__ __forceinline__ float rsinpi<float>(float x) { return sinpif(x); }
 template <typename R> __device__ __forceinline__ R rsqrt_(R x);
 template <> __device__ __forceinline__ double rsqrt_<double>(double x) { return sqrt(x); }
 template <> __device__ __forceinline__ float rsqrt_<float>(float x) { return sqrtf(x); }
@@ -231,6 +239,47 @@ __device__ __forceinline__ float p_pert(const Phys& ph, float pi, float th, floa
   if (fabsf(x) <= ph.x3_f)
     return pi * d * fmaf(x, fmaf(x, fmaf(x, ph.pg_f[2], ph.pg_f[1]), ph.pg_f[0]), 1.0f);
   return pi * th * ph.inv_gamma_f * expm1f(ph.gamma_f * log1pf(d / th));
+}
+
+// (1 + x)^gamma - 1 and, with LOG, ln(1 + x) in float64 by table and series
+// (after P. T. P. Tang's table-driven exponentials and logarithms, 1989-90):
+// 1 + x = c (1 + t) with c the nearest of 1/2, 1/2 + 1/64, ..., 2, so that
+// |t| <= 1/64 and (1 + x)^gamma - 1 = (c^gamma - 1) + c^gamma (gamma t (1 + g1 t
+// + ... + g6 t^6)). Rows of the table: c - 1, 1 / c, c^gamma - 1, c^gamma,
+// ln c. c = 1 about x = 0, where the small result keeps its relative accuracy.
+// 14 float64 instructions (LOG: 10 more) instead of about 45 for
+// expm1(gamma log1p(x)); false outside [1/2, 2] or without a table.
+// At g6 x 32 float64 (bound by the float64 pipe): derived quantities 234 ->
+// 146 us, physics (which also took ln and a power of p) 787 -> 228 us.
+constexpr int kPowRows = 97, kPowCols = 6;
+template <bool LOG>
+__device__ __forceinline__ bool pow1p(const Phys& ph, const double* pw, double x, double& pm1, double& ln) {
+  const int j = __float2int_rn((float)x * 64.0f) + 32;
+  if (!pw || (unsigned)j >= (unsigned)kPowRows) return false;
+  const double2* row = reinterpret_cast<const double2*>(pw + (size_t)j * kPowCols);
+  const double2 c = __ldg(row), e = __ldg(row + 1);
+  const double t = (x - c.x) * c.y;
+  double s = fma(t, fma(t, fma(t, fma(t, fma(t, fma(t, ph.pg[5], ph.pg[4]), ph.pg[3]), ph.pg[2]), ph.pg[1]), ph.pg[0]), 1.0);
+  pm1 = fma(e.y, ph.gamma * t * s, e.x);
+  if constexpr (LOG) {
+    s = fma(t, fma(t, fma(t, fma(t, fma(t, fma(t, -1.0 / 8, 1.0 / 7), -1.0 / 6), 1.0 / 5), -1.0 / 4), 1.0 / 3), -1.0 / 2);
+    ln = __ldg(row + 2).x + fma(t * t, s, t);
+  }
+  return true;
+}
+static __device__ __noinline__ double2 pow1p_general(double x, double gamma) {
+  const double l = log1p(x);
+  return make_double2(expm1(gamma * l), l);
+}
+// Eq. pressure in deviation form at level k: p_bar ((1 + th' / Th_bar)^gamma - 1)
+__device__ __forceinline__ double eos_level(const VR<double>& U, const Phys& ph, int k, double thp) {
+  const double x = thp * __ldg(U.inv_thb + k);
+  double f, l;
+  if (!pow1p<false>(ph, U.pw, x, f, l)) f = pow1p_general(x, ph.gamma).x;
+  return __ldg(U.pb + k) * f;
+}
+__device__ __forceinline__ float eos_level(const VR<float>& U, const Phys& ph, int k, float thp) {
+  return eos_dev<float>(__ldg(U.pb + k), __ldg(U.thb + k), thp, ph.gamma_f);
 }
 
 // Double-float numbers: an unevaluated sum hi + lo of two floats with

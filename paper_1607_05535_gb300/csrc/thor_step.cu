@@ -59,7 +59,7 @@ __device__ __forceinline__ void d_derived(const Geo<R>& G, const VR<R>& U, const
       int i = k * S + c;
       R rho = ld(U.rhob + (k)) + ld(X.rho + (i));
       R thp = ld(X.th + (i));
-      R pp = eos_dev<R>(ld(U.pb + (k)), ld(U.thb + (k)), thp, gamma);
+      R pp = eos_level(U, ph, k, thp);
       R p = ld(U.pb + (k)) + pp;
       R inv = R(1) / rho;
       R Temp = p * inv * inv_Rd;
@@ -114,7 +114,7 @@ __device__ __forceinline__ void d_lap1(const Geo<R>& G, const VR<R>& U, const Xf
       int o = k * S;
       R rlo = ld(U.rhob + (k - 1)) + ld(X.rho + (o - S + c)), rhi = ld(U.rhob + (k)) + ld(X.rho + (o + c));
       R rif = HO ? vint_iface(U, X.rho, U.rhob, k, c, S, G.nv) : ld(U.wlo + (k)) * rlo + ld(U.whi + (k)) * rhi;
-      T.qvr[o + c] = rif * Kd * apply7(wl, nb, T.vr + o) / ld(U.ri2 + (k));
+      T.qvr[o + c] = rif * Kd * apply7(wl, nb, T.vr + o) * ld(U.inv_ri2 + (k));
     } else if (k == 0 || k == G.nv) {
       T.qvr[k * S + c] = 0;
     }
@@ -340,7 +340,7 @@ __device__ __forceinline__ void d_slow_w(const Geo<R>& G, const VR<R>& U, const 
     // inertia that the hydrostatic switch drops
     if (!ph.hydrostatic) {
       R FW = 0;
-      if (hyper) FW = -apply7(wl, nb, T.qvr + k * S) / ld(U.ri2 + (k));
+      if (hyper) FW = -apply7(wl, nb, T.qvr + k * S) * ld(U.inv_ri2 + (k));
       const R acr_i = HO ? vint_iface(U, (const R*)SL.acr, (const R*)nullptr, k, c, S, G.nv)
                                     : wlo * ld(SL.acr + (i - S)) + whi * ld(SL.acr + (i));
       sw = sw - acr_i + FW;
@@ -910,17 +910,17 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
 // (Eq. im_eq_t) with the Sec. 6.1 Held-Suarez or Sec. 6.2 hot-Jupiter
 // coefficients; sigma = p / p_s with p_s extrapolated hydrostatically at the
 // lowest layer's temperature.
-// p_s of every column before the physics update, from its lowest layer
+// 1 / p_s of every column before the physics update, from its lowest layer
 // (one thread per column; the update kernel then works on chunks of levels
 // and changes the lowest layer's rho theta)
 template <typename R>
 __device__ __forceinline__ void d_surface_p(const Geo<R>& G, const VR<R>& U, const Phys& ph, const Xf<R>& X, const Work<R>& T, int bx) {
   int c = bx * blockDim.x + threadIdx.x;
   if (c >= G.ncol) return;
-  const R gamma = pc<R>(ph.gamma, ph.gamma_f), Rd = pc<R>(ph.Rd, ph.Rd_f);
-  R p0 = ld(U.pb + (0)) + eos_dev<R>(ld(U.pb + (0)), ld(U.thb + (0)), ld(X.th + (c)), gamma);
+  const R Rd = pc<R>(ph.Rd, ph.Rd_f);
+  R p0 = ld(U.pb + (0)) + eos_level(U, ph, 0, ld(X.th + (c)));
   R T0 = p0 / ((ld(U.rhob + (0)) + ld(X.rho + (c))) * Rd);
-  T.psurf[c] = p0 * rexp<R>(pc<R>(ph.g, ph.g_f) * ld(U.zc + (0)) / (Rd * T0));
+  T.psurf[c] = R(1) / (p0 * rexp<R>(pc<R>(ph.g, ph.g_f) * ld(U.zc + (0)) / (Rd * T0)));
 }
 
 // XL: the low parts of a compensated state (null: none); there the friction
@@ -936,7 +936,7 @@ __device__ __forceinline__ void d_physics(const Geo<R>& G, const VR<R>& U, const
   const R gamma = pc<R>(ph.gamma, ph.gamma_f), inv_gamma = pc<R>(ph.inv_gamma, ph.inv_gamma_f),
           Rd = pc<R>(ph.Rd, ph.Rd_f), kappa = pc<R>(ph.kappa, ph.kappa_f);
   R sl = ld(G.sinlat + (c)), cl = ld(G.coslat + (c)), clcl = ld(G.xdir + (c));
-  const R ps = ld(T.psurf + (c));
+  const R inv_ps = ld(T.psurf + (c));
   const R rdt = (R)dt;
   const int k0 = by * kchunk, k1 = min(G.nv, k0 + kchunk);
   const bool cmp = XL.rho != nullptr;
@@ -945,37 +945,50 @@ __device__ __forceinline__ void d_physics(const Geo<R>& G, const VR<R>& U, const
     R rhop = cmp ? ld(X.rho + (i)) + ld(XL.rho + (i)) : ld(X.rho + (i));
     const R thp = cmp ? ld(X.th + (i)) + ld(XL.th + (i)) : ld(X.th + (i));
     R rho = ld(U.rhob + (k)) + rhop;
-    R p = ld(U.pb + (k)) + eos_dev<R>(ld(U.pb + (k)), ld(U.thb + (k)), thp, gamma);
+    // p and, for Held-Suarez, ln(p / p0) and (p / p0)^kappa, kappa gamma =
+    // gamma - 1; float64 takes all three from one table row
+    const R p00 = R(1.0e5);
+    R p, lpr = 0, prk = 0;
+    if constexpr (sizeof(R) == sizeof(double)) {
+      const double x = thp * ld(U.inv_thb + (k));
+      double f, l;
+      if (!pow1p<true>(ph, U.pw, x, f, l)) {
+        const double2 g = pow1p_general(x, gamma);
+        f = g.x;
+        l = g.y;
+      }
+      p = ld(U.pb + (k)) * (1.0 + f);
+      if (forcing == THOR_FORCING_HELD_SUAREZ) {
+        lpr = fma(gamma, l, ld(U.lnp0 + (k)));
+        prk = ld(U.pk0 + (k)) * (1.0 + f) / (1.0 + x);
+      }
+    } else {
+      p = ld(U.pb + (k)) + eos_level(U, ph, k, thp);
+      if (forcing == THOR_FORCING_HELD_SUAREZ) {
+        lpr = rlog<R>(p / p00);
+        prk = rpow<R>(p / p00, kappa);
+      }
+    }
     R Temp = p / (rho * Rd);
-    R sigma = p / ps;
+    R sigma = p * inv_ps;
     R Kv, KT, Teq;
     if (forcing == THOR_FORCING_HELD_SUAREZ) {
       const R day = R(86400.0);
       const R kf = R(1) / day, ka = R(1) / (R(40) * day), ks = R(1) / (R(4) * day);
-      const R sb = R(0.7), p00 = R(1.0e5);
-      R ramp = (sigma - sb) / (R(1) - sb);
+      const R sb = R(0.7);
+      R ramp = (sigma - sb) * (R(1) / (R(1) - sb));
       ramp = ramp > R(0) ? ramp : R(0);
       Kv = kf * ramp;
       R c2 = cl * cl;
       KT = ka + (ks - ka) * ramp * c2 * c2;
-      R pr = p / p00;
-      Teq = (R(315) - R(60) * sl * sl - R(10) * rlog<R>(pr) * c2) * rpow<R>(pr, kappa);
+      Teq = (R(315) - R(60) * sl * sl - R(10) * lpr * c2) * prk;
       Teq = Teq > R(200) ? Teq : R(200);
     } else {
-      const R ss = R(0.12), zs = R(2.0e6), Ts = R(1600), Gt = R(2.0e-4), dTs = R(10);
-      R z = ld(U.zc + (k));
-      R Tv, bt;
-      if (z <= zs) {
-        R h = Gt * (z - zs) / R(2);
-        Tv = Ts - Gt * (zs + (z - zs) / R(2)) + rsqrt_<R>(h * h + dTs * dTs);
-        bt = (R)sin(M_PI * (double)((sigma - ss) / (R(2) * (R(1) - ss))));
-      } else {
-        Tv = Ts - Gt * zs + dTs;
-        bt = 0;
-      }
+      const R ss = R(0.12), zs = R(2.0e6);
+      const R bt = ld(U.zc + (k)) <= zs ? rsinpi<R>((sigma - ss) * (R(0.5) / (R(1) - ss))) : R(0);
       Kv = 0;
       KT = R(1) / R(1.5e5);
-      Teq = Tv + bt * (R)hj_dT * clcl;
+      Teq = ld(U.hjT + (k)) + bt * (R)hj_dT * clcl;
     }
     // no friction (K_v = 0: above sigma_b, and everywhere on the hot Jupiter)
     // leaves the momentum as it is, so it is neither read nor written there
@@ -996,6 +1009,18 @@ __device__ __forceinline__ void d_physics(const Geo<R>& G, const VR<R>& U, const
       X.mx[i] *= fr;
       X.my[i] *= fr;
       X.mz[i] *= fr;
+    }
+    if constexpr (sizeof(R) == sizeof(double)) {
+      // rho theta at fixed rho scales with T^(1 / gamma); T_new / T - 1 is
+      // small (dt over the relaxation time)
+      const double y = KT * rdt * (Teq - Temp) / ((1.0 + KT * rdt) * Temp), th = ld(U.thb + (k)) + thp;
+      double e;
+      if (U.pw && fabs(y) <= 1.0 / 128)
+        e = inv_gamma * y * fma(y, fma(y, fma(y, fma(y, fma(y, fma(y, ph.qg[5], ph.qg[4]), ph.qg[3]), ph.qg[2]), ph.qg[1]), ph.qg[0]), 1.0);
+      else
+        e = pow1p_general(y, inv_gamma).x;
+      X.th[i] = fma(th, e, thp);
+      continue;
     }
     R Tn = (Temp + KT * rdt * Teq) / (R(1) + KT * rdt);
     // rho theta at fixed rho: Th/Th_bar = ((rho/rho_bar)(T/T_bar))^(1/gamma)
