@@ -8,7 +8,7 @@
 // float32 accumulator in tensor memory, the operands brought in by TMA in
 // the 128-byte swizzled layout (k_gemm_tma; transposed copies of the
 // weights, layer inputs and gradients make every product read both operands
-// along its contraction) or, for widths that are not multiples of 8, staged
+// along its contraction) or, without a tensor-map encoder, staged
 // by threads (k_gemm_tc); the warp-level mma.sync m16n8k16 kernel
 // (k_gemm_bf16) is kept as a switchable reference path (thor_mlp_tune).
 //
@@ -26,6 +26,7 @@
 #include <cstdint>
 #include <cstring>
 #include <new>
+#include <utility>
 #include <vector>
 
 #include "../../include/thor.h"
@@ -119,18 +120,16 @@ __global__ void __launch_bounds__(128) k_gemm_bf16(int M, int N, int K, const __
       }
 }
 
-__global__ void k_to_bf16(const float* x, __nv_bfloat16* y, size_t n) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x)
-    y[i] = __float2bfloat16(x[i]);
-}
-
-// g <- g * (h > 0), then gb = bf16(g)
-__global__ void k_relu_back(float* g, const __nv_bfloat16* h, __nv_bfloat16* gb, size_t n, int mask) {
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+// g [m][N] <- g * (h > 0) (h rows of ldh), then gb = bf16(g) in rows of ldg
+__global__ void k_relu_back(float* g, const __nv_bfloat16* h, int ldh, __nv_bfloat16* gb, int ldg, int m, int N,
+                            int mask) {
+  const size_t cnt = (size_t)m * N;
+  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < cnt; i += (size_t)gridDim.x * blockDim.x) {
+    const size_t r = i / N, n = i % N;
     float v = g[i];
-    if (mask && !(__bfloat162float(h[i]) > 0.0f)) v = 0.0f;
+    if (mask && !(__bfloat162float(h[r * ldh + n]) > 0.0f)) v = 0.0f;
     g[i] = v;
-    gb[i] = __float2bfloat16(v);
+    gb[r * ldg + n] = __float2bfloat16(v);
   }
 }
 
@@ -199,18 +198,18 @@ __global__ void __launch_bounds__(1024) k_sum_parts(const float* part, int n, fl
   if (t == 0) *out = sh[0] * scale;
 }
 
-// Adam on float32 master weights, refreshing the bfloat16 copy of weights
-__global__ void k_adam(float* p, const float* g, float* m, float* v, __nv_bfloat16* pb, size_t n, float lr,
-                       float b1, float b2, float c1, float c2, float eps) {
+// one Adam update of a float32 master weight
+struct Adam {
+  float lr, b1, b2, c1, c2, eps;
+};
+__device__ __forceinline__ float adam_step(const Adam& A, float p, float g, float& m, float& v) {
+  m = A.b1 * m + (1.0f - A.b1) * g;
+  v = A.b2 * v + (1.0f - A.b2) * g * g;
+  return p - A.lr * (m / A.c1) / (sqrtf(v / A.c2) + A.eps);
+}
+__global__ void k_adam(float* p, const float* g, float* m, float* v, size_t n, Adam A) {
   for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
-    float gi = g[i];
-    float mi = b1 * m[i] + (1.0f - b1) * gi;
-    float vi = b2 * v[i] + (1.0f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    float pi = p[i] - lr * (mi / c1) / (sqrtf(vi / c2) + eps);
-    p[i] = pi;
-    if (pb) pb[i] = __float2bfloat16(pi);
+    p[i] = adam_step(A, p[i], g[i], m[i], v[i]);
   }
 }
 
@@ -476,8 +475,20 @@ size_t tc_smem_bytes(int nt) {
 // S <= TMA_STAGES with a full barrier (copies landed, by transaction bytes) and
 // an empty barrier (the MMAs that read the stage are done, by
 // tcgen05.commit). One thread issues copies and MMAs; all four warps run
-// the epilogue, which can also store the bfloat16 result transposed (CbT,
-// [N][ldt]) for a later product that contracts over the rows.
+// the epilogue.
+//
+// At the closure's sizes (batch 1024, widths 160-320) a product takes 2-3 us
+// and the network's step is bound by the number of dependent launches, so
+// (1) the epilogue does the elementwise work of the pass it belongs to
+// (GemmOut: bias, ReLU, the loss and its gradient, the ReLU mask of the
+// backward pass, bfloat16 copies straight and transposed, column sums for the
+// bias gradients), (2) one launch runs two independent products (the weight
+// and the input gradient of a layer), and (3) the kernels of a pass are
+// launched with programmatic stream serialization, each set up (barriers,
+// tensor memory, descriptors) while the previous one drains. Training step of
+// 320-256-256-256-160 at batch 1024, 29 launches -> 10: 163 -> 76 us; forward
+// and gradients of 370-256-256-256-185 at batch 1000, which the thread-staged
+// kernel ran before the copies were padded: 510 -> 64 us.
 
 constexpr int TMA_STAGES = 4, TMA_KC = 64, kMaxSplit = 8;
 
@@ -498,17 +509,71 @@ __device__ __forceinline__ void tma_load_box(uint32_t dst, const CUtensorMap* ma
       : "memory");
 }
 
-__global__ void __launch_bounds__(128, 1) k_gemm_tma(const __grid_constant__ CUtensorMap ma,
-                                                     const __grid_constant__ CUtensorMap mb, int M, int N, int K,
-                                                     float* C, int ldc, const float* bias, int relu,
-                                                     __nv_bfloat16* Cb, int ldcb, __nv_bfloat16* CbT, int ldt,
-                                                     int NT, int S, int kc_per, size_t c_split, int* err) {
+// what the epilogue does with a product, in this order; null pointers: nothing
+struct GemmOut {
+  const float* bias;               // + bias[n]
+  int relu;
+  const float* target;             // result <- gscale (result - target), squares of the difference summed
+  int ld_target;
+  float gscale;
+  float* loss;                     // [CTA of the job]
+  const __nv_bfloat16* mask;       // result zeroed where mask <= 0 (rows of ldm, a multiple of 8)
+  int ldm;
+  float* C;                        // float32 rows of ldc; split z at C + z c_split
+  int ldc;
+  size_t c_split;
+  __nv_bfloat16* Cb;               // bfloat16 rows of ldcb (a multiple of 8, at least N)
+  int ldcb;
+  __nv_bfloat16* CbT;              // bfloat16 transposed, rows of ldt
+  int ldt;
+  float* colsum;                   // [32-row tile][N] column sums
+};
+struct GemmJob {
+  CUtensorMap a, b;
+  int M, N, K, NT, stages, ntiles, mtiles, splits, kc_per;
+  GemmOut o;
+  int blocks() const { return ntiles * mtiles * splits; }
+};
+struct GemmPair {
+  GemmJob j[2];
+  int blocks0;                     // CTAs of the first job
+};
+
+// kernels of a pass: run setup while the previous kernel drains, then wait
+// for its results; let the next kernel do the same
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// column sums over a warp's 32 lanes of 16 values per lane: halves of the
+// columns are exchanged, so that 16 shuffles instead of 80 serve; lane l then
+// holds the sum of column bitwise (l >> 1)
+__device__ __forceinline__ float lane_colsum(const float* x, int lane) {
+  float a[8], b[4], c[2], d;
+  const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4, h1 = lane & 2;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) a[j] = (h4 ? x[8 + j] : x[j]) + __shfl_xor_sync(0xffffffffu, h4 ? x[j] : x[8 + j], 16);
+#pragma unroll
+  for (int j = 0; j < 4; ++j) b[j] = (h3 ? a[4 + j] : a[j]) + __shfl_xor_sync(0xffffffffu, h3 ? a[j] : a[4 + j], 8);
+#pragma unroll
+  for (int j = 0; j < 2; ++j) c[j] = (h2 ? b[2 + j] : b[j]) + __shfl_xor_sync(0xffffffffu, h2 ? b[j] : b[2 + j], 4);
+  d = (h1 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, h1 ? c[0] : c[1], 2);
+  return d + __shfl_xor_sync(0xffffffffu, d, 1);
+}
+
+__global__ void __launch_bounds__(128, 1) k_gemm_tma(const __grid_constant__ GemmPair P, int* err) {
   extern __shared__ unsigned char tma_raw[];
   __shared__ uint64_t full[TMA_STAGES], empty[TMA_STAGES], done;   // the first S in use
   __shared__ uint32_t tmem_base;
   __shared__ int all_ok;
+  __shared__ float wloss[4];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int m0 = blockIdx.y * TC_M, n0 = blockIdx.x * NT;
+  const int which = (int)blockIdx.x >= P.blocks0 ? 1 : 0;
+  const GemmJob& J = P.j[which];
+  const GemmOut& O = J.o;
+  const int bid = (int)blockIdx.x - which * P.blocks0;
+  const int nt_id = bid % J.ntiles, mt_id = bid / J.ntiles % J.mtiles, z = bid / (J.ntiles * J.mtiles);
+  const int M = J.M, N = J.N, K = J.K, NT = J.NT, S = J.stages;
+  const int m0 = mt_id * TC_M, n0 = nt_id * NT;
   const uint32_t ncols = (uint32_t)tc_cols(NT);
   const uint32_t raw = smem_u32(tma_raw), base = (raw + 1023u) & ~1023u;   // swizzle atoms need 1024 B alignment
   const uint32_t a_bytes = TC_M * TMA_KC * 2, stage_bytes = (uint32_t)(TC_M + NT) * TMA_KC * 2;
@@ -524,20 +589,21 @@ __global__ void __launch_bounds__(128, 1) k_gemm_tma(const __grid_constant__ CUt
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  pdl_next();
+  pdl_wait();
   const uint32_t tmem = tmem_base;
-  // split-K: blockIdx.z takes chunks [c0, c0 + nchunks) and stores its
-  // partial product at C + blockIdx.z * c_split
-  const int c0 = blockIdx.z * kc_per;
-  const int nchunks = min(kc_per, (K + TMA_KC - 1) / TMA_KC - c0);
-  C += blockIdx.z * c_split;
+  // split-K: split z takes chunks [c0, c0 + nchunks) and stores its partial
+  // product at C + z c_split
+  const int c0 = z * J.kc_per;
+  const int nchunks = min(J.kc_per, (K + TMA_KC - 1) / TMA_KC - c0);
   if (tid == 0) {
     const uint32_t idesc = tc_idesc(TC_M, NT);
     auto load = [&](int c) {
       const int s = c % S;
       const uint32_t a = base + (uint32_t)s * stage_bytes;
       mbar_arrive_expect_tx(&full[s], stage_bytes);
-      tma_load_box(a, &ma, (c0 + c) * TMA_KC, m0, &full[s]);
-      tma_load_box(a + a_bytes, &mb, (c0 + c) * TMA_KC, n0, &full[s]);
+      tma_load_box(a, &J.a, (c0 + c) * TMA_KC, m0, &full[s]);
+      tma_load_box(a + a_bytes, &J.b, (c0 + c) * TMA_KC, n0, &full[s]);
     };
     int issued = 0, c = 0;
     bool ok = true;
@@ -577,47 +643,98 @@ __global__ void __launch_bounds__(128, 1) k_gemm_tma(const __grid_constant__ CUt
   tc_fence_after();
   if (all_ok) {
     // straight from the accumulator: lane r of warp w holds row 32w + r, 16
-    // columns per tcgen05.ld; row-major stores move 16-byte vectors (N and
-    // the leading dimensions are multiples of 8), the transposed store is
-    // coalesced across the warp's 32 consecutive rows
+    // columns per tcgen05.ld; row-major stores move 16-byte vectors, the
+    // transposed store is coalesced across the warp's 32 consecutive rows
     const int row = m0 + warp * 32 + lane;
+    const bool live = row < M;
+    float* C = O.C ? O.C + z * O.c_split : nullptr;
+    const bool vec = C && O.ldc % 4 == 0 && (reinterpret_cast<uintptr_t>(C) & 15) == 0;
+    float loss = 0.0f;
     for (int c = 0; c < NT; c += 16) {
-      uint32_t v[16];
-      tc_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c, v);
       const int n = n0 + c;
       if (n >= N) break;                                 // warp-uniform
+      uint32_t v[16];
+      tc_ld16(tmem + ((uint32_t)(warp * 32) << 16) + (uint32_t)c, v);
+      const int left = min(16, N - n);
       float x[16];
 #pragma unroll
       for (int j = 0; j < 16; ++j) {
         x[j] = __uint_as_float(v[j]);
-        if (bias && n + j < N) x[j] += bias[n + j];
-        if (relu) x[j] = x[j] > 0.0f ? x[j] : 0.0f;
+        if (O.bias && j < left) x[j] += O.bias[n + j];
+        if (O.relu) x[j] = x[j] > 0.0f ? x[j] : 0.0f;
       }
-      if (row < M) {
+      if (O.target) {
+        const float* t = O.target + (size_t)row * O.ld_target + n;
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          if (n + 8 * h >= N) break;
-          const float* y = x + 8 * h;
-          if (C) {
-            float4* o = reinterpret_cast<float4*>(C + (size_t)row * ldc + n + 8 * h);
-            o[0] = make_float4(y[0], y[1], y[2], y[3]);
-            o[1] = make_float4(y[4], y[5], y[6], y[7]);
+        for (int j = 0; j < 16; ++j) {
+          const float d = live && j < left ? x[j] - t[j] : 0.0f;
+          loss += d * d;
+          x[j] = O.gscale * d;
+        }
+      }
+      if (O.mask) {
+        const uint4* h = reinterpret_cast<const uint4*>(O.mask + (size_t)row * O.ldm + n);
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+          const uint4 w = live && n + 8 * q < O.ldm ? h[q] : make_uint4(0u, 0u, 0u, 0u);
+          const uint32_t u[4] = {w.x, w.y, w.z, w.w};
+#pragma unroll
+          for (int j = 0; j < 8; ++j)
+            if (!(__bfloat162float(__ushort_as_bfloat16((unsigned short)(u[j >> 1] >> (16 * (j & 1))))) > 0.0f))
+              x[8 * q + j] = 0.0f;
+        }
+      }
+      if (live) {
+        if (C) {
+          float* o = C + (size_t)row * O.ldc + n;
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            if (vec && 4 * q + 4 <= left) {
+              *reinterpret_cast<float4*>(o + 4 * q) = make_float4(x[4 * q], x[4 * q + 1], x[4 * q + 2], x[4 * q + 3]);
+            } else {
+#pragma unroll
+              for (int j = 4 * q; j < 4 * q + 4; ++j)
+                if (j < left) o[j] = x[j];
+            }
           }
-          if (Cb) {
+        }
+        if (O.Cb) {
+          // columns beyond N are zero: they pad the row to a multiple of 8
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            if (8 * h >= left) break;
+            const float* y = x + 8 * h;
             uint4 q;
             q.x = pack_bf16(__float2bfloat16(y[0]), __float2bfloat16(y[1]));
             q.y = pack_bf16(__float2bfloat16(y[2]), __float2bfloat16(y[3]));
             q.z = pack_bf16(__float2bfloat16(y[4]), __float2bfloat16(y[5]));
             q.w = pack_bf16(__float2bfloat16(y[6]), __float2bfloat16(y[7]));
-            *reinterpret_cast<uint4*>(Cb + (size_t)row * ldcb + n + 8 * h) = q;
+            *reinterpret_cast<uint4*>(O.Cb + (size_t)row * O.ldcb + n + 8 * h) = q;
           }
         }
-        if (CbT) {
+        if (O.CbT) {
 #pragma unroll
           for (int j = 0; j < 16; ++j)
-            if (n + j < N) CbT[(size_t)(n + j) * ldt + row] = __float2bfloat16(x[j]);
+            if (j < left) O.CbT[(size_t)(n + j) * O.ldt + row] = __float2bfloat16(x[j]);
         }
       }
+      if (O.colsum) {
+        if (!live) {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) x[j] = 0.0f;
+        }
+        const float t = lane_colsum(x, lane);
+        const int col = lane >> 1;
+        if (!(lane & 1) && col < left && m0 + warp * 32 < M)
+          O.colsum[(size_t)(m0 / 32 + warp) * N + n + col] = t;
+      }
+    }
+    if (O.loss) {
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) loss += __shfl_xor_sync(0xffffffffu, loss, o);
+      if (lane == 0) wloss[warp] = loss;
+      __syncthreads();
+      if (tid == 0) O.loss[bid] = ((wloss[0] + wloss[1]) + wloss[2]) + wloss[3];
     }
   }
   tc_fence_before();
@@ -630,98 +747,127 @@ size_t tma_smem_bytes(int nt, int stages = TMA_STAGES) {
   return 1024 + (size_t)stages * (TC_M + nt) * TMA_KC * 2;
 }
 
-// C[M][N] (ldc) = sum over z < splits of W[z][M][N] (row length N), in z
-// order; N a multiple of 4
-__global__ void k_split_sum(const float* W, int splits, int M, int N, float* C, int ldc) {
-  const size_t n4 = (size_t)M * (N / 4);
-  for (size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x; i < n4; i += (size_t)gridDim.x * blockDim.x) {
-    const size_t r = i / (N / 4), c = (i % (N / 4)) * 4;
-    float4 a = *reinterpret_cast<const float4*>(W + r * N + c);
-    for (int z = 1; z < splits; ++z) {
-      const float4 b = *reinterpret_cast<const float4*>(W + (size_t)z * M * N + r * N + c);
-      a.x += b.x;
-      a.y += b.y;
-      a.z += b.z;
-      a.w += b.w;
-    }
-    *reinterpret_cast<float4*>(C + r * ldc + c) = a;
-  }
-}
-
-// x (float32 [m][K]) -> h (bfloat16 [m][K]) and its transpose hT ([K][ldt])
-// through a 32 x 32 shared-memory tile (both stores coalesced)
-__global__ void k_to_bf16_t(const float* x, __nv_bfloat16* h, __nv_bfloat16* hT, int m, int K, int ldt) {
+// x (float32 [m][K]) -> h (bfloat16 rows of ldh) and, unless null, its
+// transpose hT ([K][ldt]) through a 32 x 32 shared-memory tile (both stores
+// coalesced); with part the column sums of x over each 32-row tile in
+// part[row tile][K] (fixed order)
+__global__ void k_to_bf16_t(const float* x, __nv_bfloat16* h, int ldh, __nv_bfloat16* hT, int m, int K, int ldt,
+                            float* part) {
   __shared__ float t[32][33];
+  pdl_next();
+  pdl_wait();
   const int k0 = blockIdx.x * 32, r0 = blockIdx.y * 32, tx = threadIdx.x;
   for (int j = threadIdx.y; j < 32; j += 8) {
     const int r = r0 + j, k = k0 + tx;
     float v = 0.0f;
     if (r < m && k < K) {
       v = x[(size_t)r * K + k];
-      h[(size_t)r * K + k] = __float2bfloat16(v);
+      h[(size_t)r * ldh + k] = __float2bfloat16(v);
     }
     t[j][tx] = v;
   }
+  if (!hT && !part) return;
   __syncthreads();
-  for (int j = threadIdx.y; j < 32; j += 8) {
-    const int k = k0 + j, r = r0 + tx;
-    if (k < K && r < m) hT[(size_t)k * ldt + r] = __float2bfloat16(t[tx][j]);
-  }
-}
-
-// k_relu_back with the bfloat16 gradient also stored transposed (gbT
-// [N][ldt]) and the column sums of the masked float32 gradient over each
-// 32-row tile in part[row tile][N] (fixed order; k_colsum_final adds them)
-__global__ void k_relu_back_t(float* g, const __nv_bfloat16* h, __nv_bfloat16* gb, __nv_bfloat16* gbT, int m, int N,
-                              int ldt, int mask, float* part) {
-  __shared__ float t[32][33];
-  const int n0 = blockIdx.x * 32, r0 = blockIdx.y * 32, tx = threadIdx.x;
-  for (int j = threadIdx.y; j < 32; j += 8) {
-    const int r = r0 + j, n = n0 + tx;
-    float v = 0.0f;
-    if (r < m && n < N) {
-      const size_t i = (size_t)r * N + n;
-      v = g[i];
-      if (mask && !(__bfloat162float(h[i]) > 0.0f)) v = 0.0f;
-      g[i] = v;
-      gb[i] = __float2bfloat16(v);
+  if (hT) {
+    for (int j = threadIdx.y; j < 32; j += 8) {
+      const int k = k0 + j, r = r0 + tx;
+      if (k < K && r < m) hT[(size_t)k * ldt + r] = __float2bfloat16(t[tx][j]);
     }
-    t[j][tx] = v;
   }
-  __syncthreads();
-  for (int j = threadIdx.y; j < 32; j += 8) {
-    const int n = n0 + j, r = r0 + tx;
-    if (n < N && r < m) gbT[(size_t)n * ldt + r] = __float2bfloat16(t[tx][j]);
-  }
-  if (threadIdx.y == 0 && n0 + tx < N) {
+  if (part && threadIdx.y == 0 && k0 + tx < K) {
     float a = 0.0f;
 #pragma unroll 8
     for (int j = 0; j < 32; ++j) a += t[j][tx];
-    part[(size_t)blockIdx.y * N + n0 + tx] = a;
+    part[(size_t)blockIdx.y * K + k0 + tx] = a;
   }
 }
 
-// bfloat16 weights W_l [K][N] -> their transposes [N][K] at wtoff[l], every
-// layer in one launch (blockIdx.z = layer)
-struct WTable {
-  int K[16], N[16];
-  unsigned long long woff[16], wtoff[16];
+// The parameters of every layer in one launch. A block owns a 32 x 32 tile of
+// one W_l, or eight biases of one b_l (a warp each). kGrad and kAdam add the
+// split-K partials of dW_l and the row-tile partials of db_l in a fixed order;
+// kAdam updates the master weights with them, kGrad stores them flat; kAdam
+// and kCopy write the bfloat16 copies W_l (rows of Np) and W_l^T (rows of Kp)
+// that the products read. With kAdam the last block sums the loss partials.
+enum { kCopy = 0, kGrad = 1, kAdam = 2 };
+struct ParamTable {
+  int L;
+  int K[15], N[15], Kp[15], Np[15], splits[15], blk0[16];     // blk0: first block of the layer; [L]: all
+  unsigned long long woff[15], boff[15], wpoff[15], wtoff[15], wsoff[15], cpoff[15];
+  int rtiles;                                                 // 32-row tiles of the batch
+  int nloss;
+  float loss_scale;
 };
-__global__ void k_weights_t(const __nv_bfloat16* pb, __nv_bfloat16* pbt, WTable T) {
-  __shared__ __nv_bfloat16 t[32][34];
-  const int l = blockIdx.z, K = T.K[l], N = T.N[l];
-  const int n0 = blockIdx.x * 32, k0 = blockIdx.y * 32, tx = threadIdx.x;
-  if (n0 >= N || k0 >= K) return;
-  const __nv_bfloat16* W = pb + T.woff[l];
-  __nv_bfloat16* Wt = pbt + T.wtoff[l];
-  for (int j = threadIdx.y; j < 32; j += 8) {
-    const int k = k0 + j, n = n0 + tx;
-    if (k < K && n < N) t[j][tx] = W[(size_t)k * N + n];
+inline int weight_tiles(int K, int N) { return ((N + 31) / 32) * ((K + 31) / 32); }
+template <int MODE>
+__global__ void __launch_bounds__(256) k_params(float* p, float* am, float* av, const float* ws, const float* cpart,
+                                                __nv_bfloat16* wp, __nv_bfloat16* wt, float* grad,
+                                                const float* lpart, float* loss,
+                                                const __grid_constant__ ParamTable T, Adam A) {
+  __shared__ float t[32][33];
+  const int tx = threadIdx.x, ty = threadIdx.y, b = blockIdx.x;
+  pdl_next();
+  pdl_wait();
+  if (MODE == kAdam && b == T.blk0[T.L]) {
+    float* sh = &t[0][0];
+    const int q = ty * 32 + tx;
+    float a = 0.0f;
+    for (int i = q; i < T.nloss; i += 256) a += lpart[i];
+    sh[q] = a;
+    __syncthreads();
+    for (int w = 128; w > 0; w >>= 1) {
+      if (q < w) sh[q] += sh[q + w];
+      __syncthreads();
+    }
+    if (q == 0 && loss) *loss = sh[0] * T.loss_scale;
+    return;
   }
+  int l = 0;
+  while (b >= T.blk0[l + 1]) ++l;
+  const int K = T.K[l], N = T.N[l], r = b - T.blk0[l], nw = ((N + 31) / 32) * ((K + 31) / 32);
+  if (r >= nw) {
+    const int n = (r - nw) * 8 + ty;
+    if (MODE == kCopy || n >= N) return;
+    const float* cp = cpart + T.cpoff[l];
+    float g = 0.0f;
+    for (int j = tx; j < T.rtiles; j += 32) g += cp[(size_t)j * N + n];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) g += __shfl_xor_sync(0xffffffffu, g, o);
+    if (tx != 0) return;
+    const size_t i = T.boff[l] + n;
+    if (MODE == kAdam)
+      p[i] = adam_step(A, p[i], g, am[i], av[i]);
+    else
+      grad[i] = g;
+    return;
+  }
+  const int n0 = r % ((N + 31) / 32) * 32, k0 = r / ((N + 31) / 32) * 32, n = n0 + tx;
+  for (int j = ty; j < 32; j += 8) {
+    const int k = k0 + j;
+    if (k >= K || n >= N) continue;
+    const size_t i = T.woff[l] + (size_t)k * N + n;
+    float v;
+    if (MODE == kCopy) {
+      v = p[i];
+    } else {
+      const float* w = ws + T.wsoff[l] + (size_t)k * T.Np[l] + n;
+      const size_t plane = (size_t)K * T.Np[l];
+      float g = w[0];
+      for (int z = 1; z < T.splits[l]; ++z) g += w[z * plane];
+      if (MODE == kGrad) {
+        grad[i] = g;
+        continue;
+      }
+      v = adam_step(A, p[i], g, am[i], av[i]);
+      p[i] = v;
+    }
+    wp[T.wpoff[l] + (size_t)k * T.Np[l] + n] = __float2bfloat16(v);
+    t[j][tx] = v;
+  }
+  if (MODE == kGrad) return;
   __syncthreads();
-  for (int j = threadIdx.y; j < 32; j += 8) {
-    const int n = n0 + j, k = k0 + tx;
-    if (n < N && k < K) Wt[(size_t)n * K + k] = t[tx][j];
+  for (int j = ty; j < 32; j += 8) {
+    const int nn = n0 + j, k = k0 + tx;
+    if (nn < N && k < K) wt[T.wtoff[l] + (size_t)nn * T.Kp[l] + k] = __float2bfloat16(t[tx][j]);
   }
 }
 }  // namespace
@@ -731,8 +877,9 @@ __global__ void k_weights_t(const __nv_bfloat16* pb, __nv_bfloat16* pbt, WTable 
 
 struct thor_mlp {
   std::vector<int> sizes;              // layer widths, n_layers + 1 entries
+  std::vector<int> ps;                 // the same rounded up to multiples of 8: the rows of the bfloat16 copies
   int use_tc = 1;                      // tcgen05 TMA-fed (1) or thread-staged (2), mma.sync reference path (0)
-  bool tma_ok = false;                 // every width a multiple of 8 and the tensor-map encoder found
+  bool tma_ok = false;                 // the tensor-map encoder was found
   bool fwd_tma = false;                // the last forward kept the transposed layer inputs
   int sms = 148;                       // streaming multiprocessors of the device
   int ldt = 0;                         // row length of the transposed buffers (max_batch rounded up to 64)
@@ -743,20 +890,20 @@ struct thor_mlp {
   std::vector<size_t> woff, boff;      // offsets of W_l and b_l in the flat parameter vector
   void* arena = nullptr;
   float *p = nullptr, *grad = nullptr, *m = nullptr, *v = nullptr;   // flat float32 [nparam]
-  __nv_bfloat16* pb = nullptr;         // bf16 copy of all parameters (weights used)
-  __nv_bfloat16* pbt = nullptr;        // bf16 transposed weights, W_l^T [N][K] at wtoff[l]
-  std::vector<size_t> wtoff;
-  std::vector<__nv_bfloat16*> h;       // layer inputs (bf16) [max_batch][sizes[l]]
+  __nv_bfloat16* wp = nullptr;         // bf16 weights W_l [K][Np] at wpoff[l], zero beyond N
+  __nv_bfloat16* wt = nullptr;         // bf16 transposed weights W_l^T [N][Kp] at wtoff[l], zero beyond K
+  std::vector<size_t> wpoff, wtoff;
+  std::vector<__nv_bfloat16*> h;       // layer inputs (bf16) [max_batch][ps[l]], zero beyond the width
   std::vector<__nv_bfloat16*> hT;      // their transposes [sizes[l]][ldt] (TMA-fed backward)
-  __nv_bfloat16* gbT = nullptr;        // transposed bf16 gradient scratch [max width][ldt]
-  std::vector<float*> z;               // hidden outputs / gradients (float32) [max_batch][sizes[l+1]]
-  __nv_bfloat16* gb = nullptr;         // bf16 gradient scratch [max_batch][max width]
-  float* y = nullptr;                  // network output [max_batch][n_out]
-  float* dy = nullptr;                 // output gradient
+  __nv_bfloat16* gb[2] = {nullptr, nullptr};    // bf16 gradients [max_batch][max width], of a layer and the one below
+  __nv_bfloat16* gbT[2] = {nullptr, nullptr};   // their transposes [max width][ldt]
+  std::vector<float*> z;               // hidden outputs / gradients (float32) [max_batch][sizes[l+1]] (not TMA-fed)
+  float* y = nullptr;                  // network output [max_batch][n_out] (not TMA-fed)
+  float* dy = nullptr;                 // output gradient (not TMA-fed)
   float* part = nullptr;               // reduction partials
-  float* cpart = nullptr;              // column-sum partials [row blocks][max width]
-  float* ws = nullptr;                 // split-K partial products [splits][M][N]
-  size_t ws_elems = 0;
+  float* cpart = nullptr;              // column-sum partials, [row tiles][sizes[l + 1]] at cpoff[l]
+  float* ws = nullptr;                 // weight gradients, [splits][K][Np] at wsoff[l]
+  std::vector<size_t> cpoff, wsoff, ws_splits;
   int last_m = 0;
   long long step_count = 0;
   int n_layers() const { return (int)sizes.size() - 1; }
@@ -822,157 +969,243 @@ bool encode_operand(CUtensorMap* map, const __nv_bfloat16* X, int kext, int rows
              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
-// C = A B^T, A [M][lda] and B [N][ldb] both along k, on k_gemm_tma: the
-// widest tile (fewest re-reads of A) that still gives a CTA per SM, else
-// 16 columns
-int gemm_tma(const thor_mlp* net, int M, int N, int K, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B,
-             int ldb, float* C, int ldc, const float* bias, int relu, __nv_bfloat16* Cb, int ldcb,
-             __nv_bfloat16* CbT, int ldt) {
-  const int mtiles = (M + TC_M - 1) / TC_M;
+// Shape of one product on k_gemm_tma: the widest tile (fewest re-reads of A)
+// that still gives a CTA per SM, else 16 columns; with split a long
+// contraction on too few tiles (the weight gradients: K = batch) is split
+// along k over the idle SMs into at most max_split partials
+void gemm_shape(const thor_mlp* net, int M, int N, int K, bool split, int max_split, GemmJob& J) {
+  J.M = M;
+  J.N = N;
+  J.K = K;
+  J.mtiles = (M + TC_M - 1) / TC_M;
   int width = 16;
   for (int w : {256, 128, 64, 32})
-    if (mtiles * ((N + w - 1) / w) >= net->sms) {
+    if (J.mtiles * ((N + w - 1) / w) >= net->sms) {
       width = w;
       break;
     }
-  const int ntiles = (N + width - 1) / width;
-  const int nt = ((N + ntiles - 1) / ntiles + 15) / 16 * 16;
-  // a long contraction on too few tiles (the weight gradients: K = batch)
-  // is split along k over the idle SMs; the float32 partials are added in
-  // a fixed order afterwards
-  const int nchunks = (K + TMA_KC - 1) / TMA_KC, ctas = mtiles * ntiles;
-  int splits = 1;
-  if (C && !Cb && !CbT && !bias && !relu && 2 * ctas <= net->sms && nchunks >= 8) {
-    splits = std::min({(net->sms + ctas - 1) / ctas, nchunks / 4, kMaxSplit});
-    while (splits > 1 && (size_t)splits * M * N > net->ws_elems) --splits;
-  }
-  const int kc_per = (nchunks + splits - 1) / splits;
-  splits = (nchunks + kc_per - 1) / kc_per;
+  const int tiles = (N + width - 1) / width;
+  J.NT = ((N + tiles - 1) / tiles + 15) / 16 * 16;
+  J.ntiles = (N + J.NT - 1) / J.NT;
+  const int nchunks = (K + TMA_KC - 1) / TMA_KC, ctas = J.mtiles * J.ntiles;
+  J.splits = 1;
+  if (split && 2 * ctas <= net->sms && nchunks >= 8)
+    J.splits = std::min({(net->sms + ctas - 1) / ctas, nchunks / 4, max_split});
+  J.kc_per = (nchunks + J.splits - 1) / J.splits;
+  J.splits = (nchunks + J.kc_per - 1) / J.kc_per;
+  J.o = GemmOut{};
+}
+
+bool gemm_operands(GemmJob& J, const __nv_bfloat16* A, int lda, const __nv_bfloat16* B, int ldb) {
+  return encode_operand(&J.a, A, J.K, J.M, lda, TC_M) && encode_operand(&J.b, B, J.K, J.N, ldb, J.NT);
+}
+
+// a kernel of a pass, with programmatic serialization against the one before
+template <typename... K, typename... V>
+cudaError_t launch_pass(void (*kern)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, V&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, std::forward<V>(args)...);
+}
+
+// one or two independent products in one launch
+int gemm_launch(const thor_mlp* net, GemmPair& P, int jobs) {
+  P.blocks0 = P.j[0].blocks();
+  const int total = P.blocks0 + (jobs > 1 ? P.j[1].blocks() : 0);
   // the deepest ring that still lets every CTA of the grid be resident at
   // once (a second, partial wave would double the time of a short product)
-  const int per_sm = (ctas * splits + net->sms - 1) / net->sms;
+  const int per_sm = (total + net->sms - 1) / net->sms;
+  int nt = P.j[0].NT;
+  if (jobs > 1) nt = std::max(nt, P.j[1].NT);
   int stages = 2;
   for (int st = TMA_STAGES; st > 2; --st)
     if ((size_t)per_sm * (tma_smem_bytes(nt, st) + 2048) <= (size_t)227 * 1024 && per_sm * tc_cols(nt) <= 512) {
       stages = st;
       break;
     }
-  CUtensorMap ma, mb;
-  if (!encode_operand(&ma, A, K, M, lda, TC_M) || !encode_operand(&mb, B, K, N, ldb, nt)) return THOR_ECUDA;
-  dim3 grid(ntiles, mtiles, splits);
-  const size_t smem = tma_smem_bytes(nt, stages);
-  if (splits == 1) {
-    k_gemm_tma<<<grid, 128, smem, net->stream>>>(ma, mb, M, N, K, C, ldc, bias, relu, Cb, ldcb, CbT, ldt, nt, stages,
-                                                  kc_per, 0, net->err);
-  } else {
-    k_gemm_tma<<<grid, 128, smem, net->stream>>>(ma, mb, M, N, K, net->ws, N, nullptr, 0, nullptr, 0, nullptr, 0, nt,
-                                                  stages, kc_per, (size_t)M * N, net->err);
-    const size_t n4 = (size_t)M * N / 4;
-    k_split_sum<<<(int)std::min<size_t>((n4 + 255) / 256, 2048), 256, 0, net->stream>>>(net->ws, splits, M, N, C,
-                                                                                          ldc);
+  for (int q = 0; q < jobs; ++q) P.j[q].stages = stages;
+  return launch_pass(k_gemm_tma, total, 128, tma_smem_bytes(nt, stages), net->stream, P, net->err) == cudaSuccess
+             ? THOR_OK
+             : THOR_ECUDA;
+}
+
+// row length in elements of the bfloat16 gradient buffers
+int grad_ld(const thor_mlp* net, int l) { return net->ps[l + 1]; }
+
+// forward for m rows of x (float32 [m][n_in] on the device) into y (float32
+// [m][n_out]); train: instead of y, the gradient 2 (y - target) / (m n_out) of
+// the mean-squared error into gb[0], gbT[0] and the column and loss partials
+int mlp_forward_tma(thor_mlp* net, const float* x, int m, float* y, const float* target, int* nloss) {
+  cudaStream_t st = net->stream;
+  const int L = net->n_layers();
+  dim3 g((net->sizes[0] + 31) / 32, (m + 31) / 32);
+  if (launch_pass(k_to_bf16_t, g, dim3(32, 8), 0, st, x, net->h[0], net->ps[0], net->hT[0], m, net->sizes[0],
+                  net->ldt, (float*)nullptr))
+    return THOR_ECUDA;
+  for (int l = 0; l < L; ++l) {
+    const int K = net->sizes[l], N = net->sizes[l + 1];
+    const bool last = l + 1 == L;
+    GemmPair P;
+    GemmJob& J = P.j[0];
+    gemm_shape(net, m, N, K, false, 1, J);
+    // op(B) = W_l read along k from its transposed copy [N][Kp]
+    if (!gemm_operands(J, net->h[l], net->ps[l], net->wt + net->wtoff[l], net->ps[l])) return THOR_ECUDA;
+    J.o.bias = net->p + net->boff[l];
+    if (!last) {
+      J.o.relu = 1;
+      J.o.Cb = net->h[l + 1];
+      J.o.ldcb = net->ps[l + 1];
+      J.o.CbT = net->hT[l + 1];
+      J.o.ldt = net->ldt;
+    } else if (target) {
+      J.o.target = target;
+      J.o.ld_target = N;
+      J.o.gscale = 2.0f * (1.0f / ((float)m * (float)N));
+      J.o.loss = net->part;
+      J.o.Cb = net->gb[0];
+      J.o.ldcb = grad_ld(net, l);
+      J.o.CbT = net->gbT[0];
+      J.o.ldt = net->ldt;
+      J.o.colsum = net->cpart + net->cpoff[l];
+      *nloss = J.blocks();
+    } else {
+      J.o.C = y;
+      J.o.ldc = N;
+    }
+    int rc = gemm_launch(net, P, 1);
+    if (rc) return rc;
+  }
+  net->fwd_tma = true;
+  net->last_m = m;
+  return THOR_OK;
+}
+
+// backward from the output gradient in gb[0], gbT[0] and its column partials:
+// per layer one launch of dW_l = h_l^T g (into ws, both operands along the
+// batch) and, above the first layer, g_{l-1} = (g W_l^T) masked by the ReLU
+int mlp_backward_tma(thor_mlp* net, int m) {
+  const int L = net->n_layers();
+  for (int l = L - 1; l >= 0; --l) {
+    const int K = net->sizes[l], N = net->sizes[l + 1], c = (L - 1 - l) & 1;
+    GemmPair P;
+    GemmJob &W = P.j[l > 0 ? 1 : 0], &X = P.j[0];
+    gemm_shape(net, K, N, m, true, (int)net->ws_splits[l], W);
+    if (!gemm_operands(W, net->hT[l], net->ldt, net->gbT[c], net->ldt)) return THOR_ECUDA;
+    W.o.C = net->ws + net->wsoff[l];
+    W.o.ldc = net->ps[l + 1];
+    W.o.c_split = (size_t)K * net->ps[l + 1];
+    if (l > 0) {
+      // W_l [K][Np] runs along N, the contraction
+      gemm_shape(net, m, K, N, false, 1, X);
+      if (!gemm_operands(X, net->gb[c], grad_ld(net, l), net->wp + net->wpoff[l], net->ps[l + 1])) return THOR_ECUDA;
+      X.o.mask = net->h[l];
+      X.o.ldm = net->ps[l];
+      X.o.Cb = net->gb[c ^ 1];
+      X.o.ldcb = grad_ld(net, l - 1);
+      X.o.CbT = net->gbT[c ^ 1];
+      X.o.ldt = net->ldt;
+      X.o.colsum = net->cpart + net->cpoff[l - 1];
+    }
+    int rc = gemm_launch(net, P, l > 0 ? 2 : 1);
+    if (rc) return rc;
   }
   return THOR_OK;
 }
 
-// forward for m rows of x (float32 [m][n_in] on the device); keep_t: also
-// store the transposed layer inputs the TMA-fed backward contracts over
-int mlp_forward(thor_mlp* net, const float* x, int m, bool keep_t = true) {
+// k_params over every layer
+template <int MODE>
+int params_pass(const thor_mlp* net, int m, float* grad, int nloss, float loss_scale, float* loss, const Adam& A) {
+  ParamTable T{};
+  const int L = net->n_layers();
+  T.L = L;
+  T.rtiles = (m + 31) / 32;
+  T.nloss = nloss;
+  T.loss_scale = loss_scale;
+  int b = 0;
+  for (int l = 0; l < L; ++l) {
+    const int K = net->sizes[l], N = net->sizes[l + 1];
+    T.K[l] = K;
+    T.N[l] = N;
+    T.Kp[l] = net->ps[l];
+    T.Np[l] = net->ps[l + 1];
+    T.woff[l] = net->woff[l];
+    T.boff[l] = net->boff[l];
+    T.wpoff[l] = net->wpoff[l];
+    T.wtoff[l] = net->wtoff[l];
+    T.wsoff[l] = net->wsoff[l];
+    T.cpoff[l] = net->cpoff[l];
+    GemmJob J;
+    gemm_shape(net, K, N, std::max(m, 1), true, (int)net->ws_splits[l], J);
+    T.splits[l] = J.splits;
+    T.blk0[l] = b;
+    b += weight_tiles(K, N) + (N + 7) / 8;
+  }
+  T.blk0[L] = b;
+  return launch_pass(k_params<MODE>, b + (MODE == kAdam ? 1 : 0), dim3(32, 8), 0, net->stream, net->p, net->m, net->v,
+                     (const float*)net->ws, (const float*)net->cpart, net->wp, net->wt, grad,
+                     (const float*)net->part, loss, T, A) == cudaSuccess
+             ? THOR_OK
+             : THOR_ECUDA;
+}
+
+// the bfloat16 copies of the weights from the master weights
+int weights_copy(const thor_mlp* net) { return params_pass<kCopy>(net, 0, nullptr, 0, 0.0f, nullptr, Adam{}); }
+
+bool tma_path(const thor_mlp* net) { return net->use_tc == 1 && net->tma_ok; }
+
+// forward on the thread-staged tcgen05 or the mma.sync kernel, into net->y
+int mlp_forward_staged(thor_mlp* net, const float* x, int m) {
   cudaStream_t st = net->stream;
   const int L = net->n_layers();
-  const bool tma = net->use_tc == 1 && net->tma_ok;
-  net->fwd_tma = tma && keep_t;
-  if (net->fwd_tma) {
-    dim3 g((net->sizes[0] + 31) / 32, (m + 31) / 32);
-    k_to_bf16_t<<<g, dim3(32, 8), 0, st>>>(x, net->h[0], net->hT[0], m, net->sizes[0], net->ldt);
-  } else {
-    k_to_bf16<<<blocks_for((size_t)m * net->sizes[0]), 256, 0, st>>>(x, net->h[0], (size_t)m * net->sizes[0]);
-  }
+  net->fwd_tma = false;
+  dim3 g((net->sizes[0] + 31) / 32, (m + 31) / 32);
+  k_to_bf16_t<<<g, dim3(32, 8), 0, st>>>(x, net->h[0], net->ps[0], nullptr, m, net->sizes[0], 0, nullptr);
   for (int l = 0; l < L; ++l) {
     const int K = net->sizes[l], N = net->sizes[l + 1];
     const float* b = net->p + net->boff[l];
-    const bool last = l + 1 == L;
-    if (tma) {
-      // op(B) = W_l read along k from its transposed copy [N][K]
-      int rc = gemm_tma(net, m, N, K, net->h[l], K, net->pbt + net->wtoff[l], K, last ? net->y : nullptr, N, b,
-                        !last, last ? nullptr : net->h[l + 1], N,
-                        last || !net->fwd_tma ? nullptr : net->hT[l + 1], net->ldt);
-      if (rc) return rc;
-      continue;
-    }
-    const __nv_bfloat16* W = net->pb + net->woff[l];
-    if (!last)
-      gemm(net, m, N, K, net->h[l], K, 0, W, N, 0, nullptr, 0, b, 1, net->h[l + 1], N);
+    const __nv_bfloat16* W = net->wp + net->wpoff[l];
+    if (l + 1 < L)
+      gemm(net, m, N, K, net->h[l], net->ps[l], 0, W, net->ps[l + 1], 0, nullptr, 0, b, 1, net->h[l + 1], net->ps[l + 1]);
     else
-      gemm(net, m, N, K, net->h[l], K, 0, W, N, 0, net->y, N, b, 0, nullptr, 0);
+      gemm(net, m, N, K, net->h[l], net->ps[l], 0, W, net->ps[l + 1], 0, net->y, N, b, 0, nullptr, 0);
   }
   net->last_m = m;
   return cudaGetLastError() == cudaSuccess ? THOR_OK : THOR_ECUDA;
 }
 
-// gradients of sum(y * dy) after a forward of the same batch; dy float32 [m][n_out]
-int mlp_backward(thor_mlp* net, const float* dy, int m) {
+// gradients of sum(y * dy) after a forward of the same batch into net->grad;
+// dy float32 [m][n_out]
+int mlp_backward_staged(thor_mlp* net, const float* dy, int m) {
   cudaStream_t st = net->stream;
   const int L = net->n_layers();
   // g (float32) lives in z[l] buffers: z[L-1] holds the output gradient
   float* g = net->z[L - 1];
   if (cudaMemcpyAsync(g, dy, (size_t)m * net->sizes[L] * sizeof(float), cudaMemcpyDeviceToDevice, st))
     return THOR_ECUDA;
-  // the TMA-fed products need the transposed inputs of a TMA-fed forward
-  const bool tma = net->fwd_tma && net->use_tc == 1;
   for (int l = L - 1; l >= 0; --l) {
-    const int K = net->sizes[l], N = net->sizes[l + 1];
+    const int K = net->sizes[l], N = net->sizes[l + 1], ldg = grad_ld(net, l);
     float* gl = net->z[l];
-    const size_t cnt = (size_t)m * N;
-    const __nv_bfloat16* W = net->pb + net->woff[l];
+    const __nv_bfloat16* W = net->wp + net->wpoff[l];
     // relu mask of this layer's output (hidden layers), then bf16 copy
-    if (tma) {
-      dim3 g((N + 31) / 32, (m + 31) / 32);
-      k_relu_back_t<<<g, dim3(32, 8), 0, st>>>(gl, l + 1 < L ? net->h[l + 1] : nullptr, net->gb, net->gbT, m, N,
-                                               net->ldt, l + 1 < L, net->cpart);
-      // db_l = column sums of g
-      k_colsum_final<<<(N * 32 + 255) / 256, 256, 0, st>>>(net->cpart, (m + 31) / 32, N, net->grad + net->boff[l]);
-      // dW_l = h_l^T gb ([K][N]) from the transposes, both along the batch
-      int rc = gemm_tma(net, K, N, m, net->hT[l], net->ldt, net->gbT, net->ldt, net->grad + net->woff[l], N,
-                        nullptr, 0, nullptr, 0, nullptr, 0);
-      if (rc) return rc;
-    } else {
-      k_relu_back<<<blocks_for(cnt), 256, 0, st>>>(gl, l + 1 < L ? net->h[l + 1] : nullptr, net->gb, cnt,
-                                                   l + 1 < L);
-      // dW_l = h_l^T gb  ([K][N])
-      gemm(net, K, N, m, net->h[l], K, 1, net->gb, N, 0, net->grad + net->woff[l], N, nullptr, 0, nullptr, 0);
-      // db_l = column sums of g
-      k_colsum_part<<<dim3((N + 31) / 32, (m + 127) / 128), dim3(32, 8), 0, st>>>(gl, m, N, net->cpart);
-      k_colsum_final<<<(N * 32 + 255) / 256, 256, 0, st>>>(net->cpart, (m + 127) / 128, N, net->grad + net->boff[l]);
-    }
-    if (l > 0) {
-      // g_{l-1} = gb W_l^T ([m][K]) into z[l-1]; W_l [K][N] runs along N, the contraction
-      if (tma) {
-        int rc = gemm_tma(net, m, K, N, net->gb, N, W, N, net->z[l - 1], K, nullptr, 0, nullptr, 0, nullptr, 0);
-        if (rc) return rc;
-      } else {
-        gemm(net, m, K, N, net->gb, N, 0, W, N, 1, net->z[l - 1], K, nullptr, 0, nullptr, 0);
-      }
-    }
+    k_relu_back<<<blocks_for((size_t)m * N), 256, 0, st>>>(gl, l + 1 < L ? net->h[l + 1] : nullptr, net->ps[l + 1],
+                                                           net->gb[0], ldg, m, N, l + 1 < L);
+    // dW_l = h_l^T gb  ([K][N])
+    gemm(net, K, N, m, net->h[l], net->ps[l], 1, net->gb[0], ldg, 0, net->grad + net->woff[l], N, nullptr, 0, nullptr, 0);
+    // db_l = column sums of g
+    k_colsum_part<<<dim3((N + 31) / 32, (m + 127) / 128), dim3(32, 8), 0, st>>>(gl, m, N, net->cpart);
+    k_colsum_final<<<(N * 32 + 255) / 256, 256, 0, st>>>(net->cpart, (m + 127) / 128, N, net->grad + net->boff[l]);
+    // g_{l-1} = gb W_l^T ([m][K]) into z[l-1]
+    if (l > 0) gemm(net, m, K, N, net->gb[0], ldg, 0, W, net->ps[l + 1], 1, net->z[l - 1], K, nullptr, 0, nullptr, 0);
   }
   return cudaGetLastError() == cudaSuccess ? THOR_OK : THOR_ECUDA;
-}
-
-// refreshes the transposed bfloat16 weights from pb (TMA-fed forward)
-void weights_t(const thor_mlp* net) {
-  if (!net->tma_ok) return;
-  WTable T{};
-  int kmax = 0, nmax = 0;
-  const int L = net->n_layers();
-  for (int l = 0; l < L; ++l) {
-    T.K[l] = net->sizes[l];
-    T.N[l] = net->sizes[l + 1];
-    T.woff[l] = net->woff[l];
-    T.wtoff[l] = net->wtoff[l];
-    kmax = std::max(kmax, T.K[l]);
-    nmax = std::max(nmax, T.N[l]);
-  }
-  dim3 g((nmax + 31) / 32, (kmax + 31) / 32, L);
-  k_weights_t<<<g, dim3(32, 8), 0, net->stream>>>(net->pb, net->pbt, T);
 }
 
 }  // namespace
@@ -1000,14 +1233,17 @@ int thor_mlp_create(const int* sizes, int n_sizes, int max_batch, unsigned long 
     net->nparam += sizes[l + 1];
   }
   for (int i = 0; i < n_sizes; ++i) wmax = std::max(wmax, sizes[i]);
-  // the TMA-fed products read rows of 16-byte multiples
+  // the TMA-fed products read rows of 16-byte multiples: the bfloat16 copies
+  // of weights, layer inputs and gradients are padded with zeros to them
   net->tma_ok = encode_tiled() != nullptr;
-  for (int i = 0; i < n_sizes; ++i) net->tma_ok = net->tma_ok && sizes[i] % 8 == 0;
+  for (int i = 0; i < n_sizes; ++i) net->ps.push_back((sizes[i] + 7) / 8 * 8);
   net->ldt = (max_batch + 63) / 64 * 64;
-  size_t nwt = 0;
+  size_t nwp = 0, nwt = 0;
   for (int l = 0; l < L; ++l) {
+    net->wpoff.push_back(nwp);
+    nwp += ((size_t)sizes[l] * net->ps[l + 1] + 63) / 64 * 64;
     net->wtoff.push_back(nwt);
-    nwt += ((size_t)sizes[l] * sizes[l + 1] + 63) / 64 * 64;
+    nwt += ((size_t)sizes[l + 1] * net->ps[l] + 63) / 64 * 64;
   }
   {
     int dev = 0, sms = 0;
@@ -1019,23 +1255,31 @@ int thor_mlp_create(const int* sizes, int n_sizes, int max_batch, unsigned long 
   size_t bytes = 0;
   auto take = [&](size_t b) { size_t o = bytes; bytes += (b + 255) / 256 * 256; return o; };
   size_t o_p = take(net->nparam * 4), o_g = take(net->nparam * 4), o_m = take(net->nparam * 4),
-         o_v = take(net->nparam * 4), o_pb = take(net->nparam * 2);
+         o_v = take(net->nparam * 4), o_wp = take(nwp * 2), o_wt = take(nwt * 2);
+  const int wpad = (wmax + 7) / 8 * 8, rt = (max_batch + 31) / 32;
   std::vector<size_t> o_h, o_z, o_ht;
-  for (int l = 0; l < L; ++l) o_h.push_back(take((size_t)max_batch * sizes[l] * 2));
+  for (int l = 0; l < L; ++l) o_h.push_back(take((size_t)max_batch * net->ps[l] * 2));
   for (int l = 0; l < L; ++l) o_z.push_back(take((size_t)max_batch * sizes[l + 1] * 4));
-  size_t o_gb = take((size_t)max_batch * wmax * 2), o_y = take((size_t)max_batch * sizes[L] * 4),
-         o_dy = take((size_t)max_batch * sizes[L] * 4), o_part = take(4096 * 4 + 64), o_err = take(64),
-         o_cpart = take((size_t)((max_batch + 31) / 32) * wmax * 4);
-  size_t o_pbt = 0, o_gbt = 0, o_ws = 0;
-  if (net->tma_ok) {
-    size_t wmn = 0;
-    for (int l = 0; l < L; ++l) wmn = std::max(wmn, (size_t)sizes[l] * sizes[l + 1]);
-    net->ws_elems = (size_t)kMaxSplit * wmn;
-    o_ws = take(net->ws_elems * 4);
-    o_pbt = take(nwt * 2);
-    for (int l = 0; l < L; ++l) o_ht.push_back(take((size_t)sizes[l] * net->ldt * 2));
-    o_gbt = take((size_t)wmax * net->ldt * 2);
+  size_t o_gb[2] = {0, 0}, o_gbt[2] = {0, 0};
+  for (int q = 0; q < 2; ++q) o_gb[q] = take((size_t)max_batch * wpad * 2);
+  // a loss partial per CTA of the output layer's product (at most 16 columns x 128 rows each)
+  const size_t nparts = std::max<size_t>(4096, (size_t)((max_batch + TC_M - 1) / TC_M) * ((sizes[L] + 15) / 16));
+  size_t o_y = take((size_t)max_batch * sizes[L] * 4), o_dy = take((size_t)max_batch * sizes[L] * 4),
+         o_part = take(nparts * 4 + 64), o_err = take(64);
+  size_t ncp = 0, nws = 0;
+  for (int l = 0; l < L; ++l) {
+    net->cpoff.push_back(ncp);
+    ncp += (size_t)rt * sizes[l + 1];
+    // room for the splits of the largest batch (a smaller one has no more)
+    GemmJob J;
+    gemm_shape(net, sizes[l], sizes[l + 1], max_batch, true, kMaxSplit, J);
+    net->ws_splits.push_back(J.splits);
+    net->wsoff.push_back(nws);
+    nws += (size_t)J.splits * sizes[l] * net->ps[l + 1];
   }
+  size_t o_cpart = take(ncp * 4), o_ws = take(nws * 4);
+  for (int l = 0; l < L; ++l) o_ht.push_back(take((size_t)sizes[l] * net->ldt * 2));
+  for (int q = 0; q < 2; ++q) o_gbt[q] = take((size_t)wmax * net->ldt * 2);
   if (cudaMalloc(&net->arena, bytes) != cudaSuccess) {
     delete net;
     return THOR_ENOMEM;
@@ -1045,20 +1289,20 @@ int thor_mlp_create(const int* sizes, int n_sizes, int max_batch, unsigned long 
   net->grad = (float*)(base + o_g);
   net->m = (float*)(base + o_m);
   net->v = (float*)(base + o_v);
-  net->pb = (__nv_bfloat16*)(base + o_pb);
+  net->wp = (__nv_bfloat16*)(base + o_wp);
+  net->wt = (__nv_bfloat16*)(base + o_wt);
   for (int l = 0; l < L; ++l) {
     net->h.push_back((__nv_bfloat16*)(base + o_h[l]));
     net->z.push_back((float*)(base + o_z[l]));
+    net->hT.push_back((__nv_bfloat16*)(base + o_ht[l]));
   }
-  net->gb = (__nv_bfloat16*)(base + o_gb);
+  for (int q = 0; q < 2; ++q) {
+    net->gb[q] = (__nv_bfloat16*)(base + o_gb[q]);
+    net->gbT[q] = (__nv_bfloat16*)(base + o_gbt[q]);
+  }
   net->y = (float*)(base + o_y);
   net->err = (int*)(base + o_err);
-  if (net->tma_ok) {
-    net->pbt = (__nv_bfloat16*)(base + o_pbt);
-    for (int l = 0; l < L; ++l) net->hT.push_back((__nv_bfloat16*)(base + o_ht[l]));
-    net->gbT = (__nv_bfloat16*)(base + o_gbt);
-    net->ws = (float*)(base + o_ws);
-  }
+  net->ws = (float*)(base + o_ws);
   if (cudaMemsetAsync(net->err, 0, 64, net->stream) ||
       cudaFuncSetAttribute(k_gemm_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, 128 * 1024) ||
       cudaFuncSetAttribute(k_gemm_tma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tma_smem_bytes(256))) {
@@ -1087,9 +1331,7 @@ int thor_mlp_create(const int* sizes, int n_sizes, int max_batch, unsigned long 
     delete net;
     return THOR_ECUDA;
   }
-  k_to_bf16<<<blocks_for(net->nparam), 256, 0, st>>>(net->p, net->pb, net->nparam);
-  weights_t(net);
-  if (cudaStreamSynchronize(st)) {
+  if (weights_copy(net) || cudaStreamSynchronize(st)) {
     cudaFree(net->arena);
     delete net;
     return THOR_ECUDA;
@@ -1127,8 +1369,7 @@ int thor_mlp_set_params(thor_mlp* net, const float* host, size_t n) {
   using namespace thor;
   if (!net || !host || n != net->nparam) return THOR_EINVAL;
   if (cudaMemcpyAsync(net->p, host, n * 4, cudaMemcpyHostToDevice, net->stream)) return THOR_ECUDA;
-  k_to_bf16<<<blocks_for(n), 256, 0, net->stream>>>(net->p, net->pb, n);
-  weights_t(net);
+  if (weights_copy(net)) return THOR_ECUDA;
   if (cudaMemsetAsync(net->m, 0, n * 4, net->stream) || cudaMemsetAsync(net->v, 0, n * 4, net->stream))
     return THOR_ECUDA;
   net->step_count = 0;
@@ -1138,7 +1379,8 @@ int thor_mlp_set_params(thor_mlp* net, const float* host, size_t n) {
 int thor_mlp_forward(thor_mlp* net, const float* x, int m, float* y) {
   using namespace thor;
   if (!net || !x || !y || m < 1 || m > net->max_batch) return THOR_EINVAL;
-  int rc = mlp_forward(net, x, m);
+  if (tma_path(net)) return mlp_forward_tma(net, x, m, y, nullptr, nullptr);
+  int rc = mlp_forward_staged(net, x, m);
   if (rc) return rc;
   const size_t cnt = (size_t)m * net->sizes.back() * sizeof(float);
   return cudaMemcpyAsync(y, net->y, cnt, cudaMemcpyDeviceToDevice, net->stream) ? THOR_ECUDA : THOR_OK;
@@ -1147,7 +1389,17 @@ int thor_mlp_forward(thor_mlp* net, const float* x, int m, float* y) {
 int thor_mlp_backward(thor_mlp* net, const float* dy, int m, float* grad) {
   using namespace thor;
   if (!net || !dy || !grad || m != net->last_m || m < 1) return THOR_EINVAL;
-  int rc = mlp_backward(net, dy, m);
+  // the TMA-fed products need the transposed inputs of a TMA-fed forward
+  if (net->fwd_tma && tma_path(net)) {
+    const int L = net->n_layers(), N = net->sizes[L];
+    dim3 g((N + 31) / 32, (m + 31) / 32);
+    if (launch_pass(k_to_bf16_t, g, dim3(32, 8), 0, net->stream, dy, net->gb[0], grad_ld(net, L - 1), net->gbT[0], m, N,
+                    net->ldt, net->cpart + net->cpoff[L - 1]))
+      return THOR_ECUDA;
+    int rc = mlp_backward_tma(net, m);
+    return rc ? rc : params_pass<kGrad>(net, m, grad, 0, 0.0f, nullptr, Adam{});
+  }
+  int rc = mlp_backward_staged(net, dy, m);
   if (rc) return rc;
   return cudaMemcpyAsync(grad, net->grad, net->nparam * 4, cudaMemcpyDeviceToDevice, net->stream) ? THOR_ECUDA
                                                                                               : THOR_OK;
@@ -1157,20 +1409,28 @@ int thor_mlp_train_step(thor_mlp* net, const float* x, const float* target, int 
   using namespace thor;
   if (!net || !x || !target || m < 1 || m > net->max_batch || !(lr > 0)) return THOR_EINVAL;
   cudaStream_t st = net->stream;
-  int rc = mlp_forward(net, x, m);
-  if (rc) return rc;
   const size_t cnt = (size_t)m * net->sizes.back();
+  auto adam = [&]() {
+    net->step_count += 1;
+    const float b1 = 0.9f, b2 = 0.999f;
+    return Adam{lr, b1, b2, 1.0f - powf(b1, (float)net->step_count), 1.0f - powf(b2, (float)net->step_count), 1e-8f};
+  };
+  if (tma_path(net)) {
+    int nloss = 0;
+    int rc = mlp_forward_tma(net, x, m, nullptr, target, &nloss);
+    if (!rc) rc = mlp_backward_tma(net, m);
+    return rc ? rc : params_pass<kAdam>(net, m, nullptr, nloss, 1.0f / (float)cnt, loss, adam());
+  }
+  int rc = mlp_forward_staged(net, x, m);
+  if (rc) return rc;
   const int nb = std::min(blocks_for(cnt), 1024);
   k_mse<<<nb, 256, 0, st>>>(net->y, target, net->dy, cnt, 1.0f / (float)cnt, net->part);
   if (loss) k_sum_parts<<<1, 1024, 0, st>>>(net->part, nb, 1.0f / (float)cnt, loss);
-  rc = mlp_backward(net, net->dy, m);
+  rc = mlp_backward_staged(net, net->dy, m);
   if (rc) return rc;
-  net->step_count += 1;
-  const float b1 = 0.9f, b2 = 0.999f;
-  const float c1 = 1.0f - powf(b1, (float)net->step_count), c2 = 1.0f - powf(b2, (float)net->step_count);
-  k_adam<<<blocks_for(net->nparam), 256, 0, st>>>(net->p, net->grad, net->m, net->v, net->pb, net->nparam, lr,
-                                                  b1, b2, c1, c2, 1e-8f);
-  weights_t(net);
+  k_adam<<<blocks_for(net->nparam), 256, 0, st>>>(net->p, net->grad, net->m, net->v, net->nparam, adam());
+  rc = weights_copy(net);
+  if (rc) return rc;
   return cudaGetLastError() == cudaSuccess ? THOR_OK : THOR_ECUDA;
 }
 
@@ -1262,10 +1522,15 @@ int closure_evaluate_t(thor_state* s) {
   const int Fin = 2 * kClosureFields * nv, Fout = kClosureFields * nv;
   for (int c0 = 0; c0 < ncol; c0 += net->max_batch) {
     const int m = std::min(net->max_batch, ncol - c0);
-    int rc = mlp_forward(net, cb.x + (size_t)c0 * Fin, m, false);
+    float* y = cb.y + (size_t)c0 * Fout;
+    int rc;
+    if (tma_path(net)) {
+      rc = mlp_forward_tma(net, cb.x + (size_t)c0 * Fin, m, y, nullptr, nullptr);
+    } else {
+      rc = mlp_forward_staged(net, cb.x + (size_t)c0 * Fin, m);
+      if (!rc && cudaMemcpyAsync(y, net->y, (size_t)m * Fout * 4, cudaMemcpyDeviceToDevice, st)) rc = THOR_ECUDA;
+    }
     if (rc) return rc;
-    if (cudaMemcpyAsync(cb.y + (size_t)c0 * Fout, net->y, (size_t)m * Fout * 4, cudaMemcpyDeviceToDevice, st))
-      return THOR_ECUDA;
   }
   I->launches += 1 + 4 * ((ncol + net->max_batch - 1) / net->max_batch);
   return cudaGetLastError() == cudaSuccess ? THOR_OK : THOR_ECUDA;
