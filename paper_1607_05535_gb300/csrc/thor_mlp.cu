@@ -1208,6 +1208,31 @@ int mlp_backward_staged(thor_mlp* net, const float* dy, int m) {
   return cudaGetLastError() == cudaSuccess ? THOR_OK : THOR_ECUDA;
 }
 
+// y = MLP(x) for any number of rows through two scratch buffers of m rows x
+// the widest layer, without the network's own batch buffers (inference)
+int mlp_infer(thor_mlp* net, int m, float* y, __nv_bfloat16* const buf[2]) {
+  const int L = net->n_layers();
+  for (int l = 0; l < L; ++l) {
+    const int K = net->sizes[l], N = net->sizes[l + 1];
+    GemmPair P;
+    GemmJob& J = P.j[0];
+    gemm_shape(net, m, N, K, false, 1, J);
+    if (!gemm_operands(J, buf[l & 1], net->ps[l], net->wt + net->wtoff[l], net->ps[l])) return THOR_ECUDA;
+    J.o.bias = net->p + net->boff[l];
+    if (l + 1 < L) {
+      J.o.relu = 1;
+      J.o.Cb = buf[(l & 1) ^ 1];
+      J.o.ldcb = net->ps[l + 1];
+    } else {
+      J.o.C = y;
+      J.o.ldc = N;
+    }
+    int rc = gemm_launch(net, P, 1);
+    if (rc) return rc;
+  }
+  return THOR_OK;
+}
+
 }  // namespace
 }  // namespace thor
 
@@ -1462,51 +1487,112 @@ __device__ __forceinline__ R* closure_field_rw(const Xf<R>& X, int f) {
 // that field over the neighbours of c minus its value at c (the neighbour
 // anomaly carries the horizontal-curvature signal without the cancellation
 // that bfloat16 inputs would suffer if centre and mean were given apart);
-// normalised by (x - mean) / std per feature
+// normalised by (x - mean) / std per feature. Into float32 rows of F, or (Y =
+// __nv_bfloat16) straight into the network's input rows of ldx.
+//
+// The planes run along the columns, the features along the levels: a block
+// owns 32 columns x 32 levels of one field and turns them in shared memory,
+// so that both sides move whole lines (one thread per column wrote every
+// value to a line of its own). Sums over neighbours: float64 for
+// float64 states; for float states the differences a(n) - a(c) as TwoSum
+// pairs on the float32 pipes, about 48 bits, rounded once.
 template <typename R>
-__global__ void k_features(Geo<R> G, Xf<R> X, const float* mean, const float* std, float* x) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  const int k = blockIdx.y;
-  if (c >= G.ncol) return;
-  const int S = G.colp, nv = G.nv, F = 2 * kClosureFields * nv;
-  int nb[6], nn = 0;
-  for (int j = 0; j < 6; ++j) {
-    const int q = G.nbr[j * S + c];
-    if (q != c) nb[nn++] = q;
+struct NbrMean {
+  R c, s = 0, e = 0;
+  __device__ void add(R a);
+  __device__ float anomaly(int nn) const;
+};
+template <>
+__device__ __forceinline__ void NbrMean<double>::add(double a) { s += a; }
+template <>
+__device__ __forceinline__ float NbrMean<double>::anomaly(int nn) const { return (float)(s / nn - c); }
+template <>
+__device__ __forceinline__ void NbrMean<float>::add(float a) {
+  float d, d1, t, t1;
+  two_sum(a, -c, d, d1);
+  two_sum(s, d, t, t1);
+  s = t;
+  e += d1 + t1;
+}
+template <>
+__device__ __forceinline__ float NbrMean<float>::anomaly(int nn) const { return (s + e) / (float)nn; }
+__device__ __forceinline__ void feature_store(float* x, float v) { *x = v; }
+__device__ __forceinline__ void feature_store(__nv_bfloat16* x, float v) { *x = __float2bfloat16(v); }
+
+template <typename R, typename Y>
+__global__ void __launch_bounds__(256) k_features(Geo<R> G, Xf<R> X, const float* mean, const float* std, Y* x, int ldx) {
+  __shared__ float tv[32][33], ta[32][33];
+  const int S = G.colp, nv = G.nv, tx = threadIdx.x, ty = threadIdx.y;
+  const int c0 = blockIdx.x * 32, c = c0 + tx, k0 = blockIdx.y * 32, f = blockIdx.z;
+  if (c < G.ncol) {
+    int nb[6], nn = 0;
+#pragma unroll
+    for (int j = 0; j < 6; ++j) {
+      nb[j] = ld(G.nbr + j * S + c);
+      nn += nb[j] != c;
+    }
+    for (int j = ty; j < 32 && k0 + j < nv; j += 8) {
+      const R* a = closure_field(X, f) + (size_t)(k0 + j) * S;
+      NbrMean<R> m{ld(a + c)};
+#pragma unroll
+      for (int q = 0; q < 6; ++q)
+        if (nb[q] != c) m.add(ld(a + nb[q]));
+      tv[j][tx] = (float)m.c;
+      ta[j][tx] = m.anomaly(nn);
+    }
   }
-  for (int f = 0; f < kClosureFields; ++f) {
-    const R* a = closure_field(X, f) + (size_t)k * S;
-    const int j0 = f * nv + k, j1 = kClosureFields * nv + f * nv + k;
-    double s = 0.0;
-    for (int j = 0; j < nn; ++j) s += (double)a[nb[j]];
-    x[(size_t)c * F + j0] = ((float)a[c] - mean[j0]) / std[j0];
-    x[(size_t)c * F + j1] = ((float)(s / nn - (double)a[c]) - mean[j1]) / std[j1];
+  __syncthreads();
+  const int k = k0 + tx;
+  if (k >= nv) return;
+  const int j0 = f * nv + k, j1 = kClosureFields * nv + j0;
+  const float m0 = mean[j0], s0 = std[j0], m1 = mean[j1], s1 = std[j1];
+  for (int j = ty; j < 32 && c0 + j < G.ncol; j += 8) {
+    Y* row = x + (size_t)(c0 + j) * ldx;
+    feature_store(row + j0, (tv[tx][j] - m0) / s0);
+    feature_store(row + j1, (ta[tx][j] - m1) / s1);
   }
 }
 
 // field += span (y * out_std + out_mean); the momentum correction is projected
-// onto the tangent plane like every horizontal-momentum update
+// onto the tangent plane like every horizontal-momentum update. Blocks of 32
+// columns x 32 levels, the network's rows turned in shared memory as above.
 template <typename R>
-__global__ void k_apply(Geo<R> G, Xf<R> X, const float* y, const float* omean, const float* ostd, float span) {
-  const int c = blockIdx.x * blockDim.x + threadIdx.x;
-  const int k = blockIdx.y;
+__global__ void __launch_bounds__(256) k_apply(Geo<R> G, Xf<R> X, const float* y, const float* omean,
+                                               const float* ostd, float span) {
+  __shared__ float t[kClosureFields][32][33];
+  const int S = G.colp, nv = G.nv, F = kClosureFields * nv, tx = threadIdx.x, ty = threadIdx.y;
+  const int c0 = blockIdx.x * 32, k0 = blockIdx.y * 32;
+  if (k0 + tx < nv) {
+#pragma unroll
+    for (int f = 0; f < kClosureFields; ++f) {
+      const int q = f * nv + k0 + tx;
+      const float sd = ostd[q], mn = omean[q];
+      for (int j = ty; j < 32 && c0 + j < G.ncol; j += 8) t[f][j][tx] = y[(size_t)(c0 + j) * F + q] * sd + mn;
+    }
+  }
+  __syncthreads();
+  const int c = c0 + tx;
   if (c >= G.ncol) return;
-  const int S = G.colp, nv = G.nv, F = kClosureFields * nv;
-  const size_t i = (size_t)k * S + c;
-  float t[kClosureFields];
-  for (int f = 0; f < kClosureFields; ++f) {
-    const int j = f * nv + k;
-    t[f] = y[(size_t)c * F + j] * ostd[j] + omean[j];
-  }
   const float rx = (float)G.rhat[c], ry = (float)G.rhat[S + c], rz = (float)G.rhat[2 * S + c];
-  const float d = t[1] * rx + t[2] * ry + t[3] * rz;
-  t[1] -= d * rx;
-  t[2] -= d * ry;
-  t[3] -= d * rz;
-  for (int f = 0; f < kClosureFields; ++f) {
-    R* a = closure_field_rw(X, f);
-    a[i] = a[i] + (R)(span * t[f]);
+  for (int j = ty; j < 32 && k0 + j < nv; j += 8) {
+    const size_t i = (size_t)(k0 + j) * S + c;
+    float u[kClosureFields];
+#pragma unroll
+    for (int f = 0; f < kClosureFields; ++f) u[f] = t[f][tx][j];
+    const float d = u[1] * rx + u[2] * ry + u[3] * rz;
+    u[1] -= d * rx;
+    u[2] -= d * ry;
+    u[3] -= d * rz;
+#pragma unroll
+    for (int f = 0; f < kClosureFields; ++f) {
+      R* a = closure_field_rw(X, f);
+      a[i] = a[i] + (R)(span * u[f]);
+    }
   }
+}
+template <typename R>
+dim3 turn_grid(const Impl<R>* I, int fields) {
+  return dim3((I->G.ncol + 31) / 32, (I->G.nv + 31) / 32, fields);
 }
 
 // tau_hat = MLP(features of the current state), kept in the binding's y buffer
@@ -1517,22 +1603,29 @@ int closure_evaluate_t(thor_state* s) {
   thor_mlp* net = cb.net;
   cudaStream_t st = I->stream;
   const int ncol = I->G.ncol, nv = I->G.nv;
-  dim3 grid((ncol + 127) / 128, nv);
-  k_features<R><<<grid, 128, 0, st>>>(I->G, I->Xt, cb.in_mean, cb.in_std, cb.x);
   const int Fin = 2 * kClosureFields * nv, Fout = kClosureFields * nv;
+  if (tma_path(net)) {
+    // features straight into the network's bfloat16 input rows, all columns
+    // in one pass of the network through the binding's own buffers, the
+    // output in place (10242 columns: 27 us; a pass of max_batch columns at a
+    // time with float32 features and a copy of the output took about 390)
+    k_features<R, __nv_bfloat16><<<turn_grid(I, kClosureFields), dim3(32, 8), 0, st>>>(
+        I->G, I->Xt, cb.in_mean, cb.in_std, static_cast<__nv_bfloat16*>(cb.act[0]), net->ps[0]);
+    __nv_bfloat16* const act[2] = {static_cast<__nv_bfloat16*>(cb.act[0]), static_cast<__nv_bfloat16*>(cb.act[1])};
+    const int rc = mlp_infer(net, ncol, cb.y, act);
+    if (rc) return rc;
+    I->launches += 1 + net->n_layers();
+    return cudaGetLastError() == cudaSuccess ? THOR_OK : THOR_ECUDA;
+  }
+  k_features<R, float><<<turn_grid(I, kClosureFields), dim3(32, 8), 0, st>>>(I->G, I->Xt, cb.in_mean, cb.in_std, cb.x, Fin);
   for (int c0 = 0; c0 < ncol; c0 += net->max_batch) {
     const int m = std::min(net->max_batch, ncol - c0);
-    float* y = cb.y + (size_t)c0 * Fout;
-    int rc;
-    if (tma_path(net)) {
-      rc = mlp_forward_tma(net, cb.x + (size_t)c0 * Fin, m, y, nullptr, nullptr);
-    } else {
-      rc = mlp_forward_staged(net, cb.x + (size_t)c0 * Fin, m);
-      if (!rc && cudaMemcpyAsync(y, net->y, (size_t)m * Fout * 4, cudaMemcpyDeviceToDevice, st)) rc = THOR_ECUDA;
-    }
+    int rc = mlp_forward_staged(net, cb.x + (size_t)c0 * Fin, m);
     if (rc) return rc;
+    if (cudaMemcpyAsync(cb.y + (size_t)c0 * Fout, net->y, (size_t)m * Fout * 4, cudaMemcpyDeviceToDevice, st))
+      return THOR_ECUDA;
   }
-  I->launches += 1 + 4 * ((ncol + net->max_batch - 1) / net->max_batch);
+  I->launches += 1 + (1 + net->n_layers()) * ((ncol + net->max_batch - 1) / net->max_batch);
   return cudaGetLastError() == cudaSuccess ? THOR_OK : THOR_ECUDA;
 }
 
@@ -1540,8 +1633,7 @@ template <typename R>
 int closure_correct_t(thor_state* s, double span) {
   Impl<R>* I = static_cast<Impl<R>*>(s->impl.get());
   ClosureBinding& cb = s->closure;
-  dim3 grid((I->G.ncol + 127) / 128, I->G.nv);
-  k_apply<R><<<grid, 128, 0, I->stream>>>(I->G, I->Xt, cb.y, cb.out_mean, cb.out_std, (float)span);
+  k_apply<R><<<turn_grid(I, 1), dim3(32, 8), 0, I->stream>>>(I->G, I->Xt, cb.y, cb.out_mean, cb.out_std, (float)span);
   I->launches += 1;
   return cudaGetLastError() == cudaSuccess ? THOR_OK : THOR_ECUDA;
 }
@@ -1607,6 +1699,8 @@ int closure_large_step(thor_state* s, int n_small, double dt) {
 void closure_release(thor_state* s) {
   if (s->closure.x) cudaFree(s->closure.x);
   if (s->closure.y) cudaFree(s->closure.y);
+  for (void* a : s->closure.act)
+    if (a) cudaFree(a);
   s->closure = ClosureBinding();
 }
 
@@ -1617,8 +1711,8 @@ template <typename R>
 int features_t(thor_state* s, const float* mean, const float* std, float* x) {
   using namespace thor;
   Impl<R>* I = static_cast<Impl<R>*>(s->impl.get());
-  dim3 grid((I->G.ncol + 127) / 128, I->G.nv);
-  k_features<R><<<grid, 128, 0, I->stream>>>(I->G, I->Xt, mean, std, x);
+  k_features<R, float><<<turn_grid(I, kClosureFields), dim3(32, 8), 0, I->stream>>>(I->G, I->Xt, mean, std, x,
+                                                                                 2 * kClosureFields * I->G.nv);
   I->launches += 1;
   return cudaGetLastError() == cudaSuccess ? THOR_OK : THOR_ECUDA;
 }
@@ -1685,9 +1779,16 @@ int thor_closure_attach(thor_state* s, thor_mlp* net, const float* in_mean, cons
   cb.out_mean = out_mean;
   cb.out_std = out_std;
   cb.period = period;
-  if (cudaMalloc(&cb.x, (size_t)ncol * 2 * kClosureFields * nv * 4) ||
-      cudaMalloc(&cb.y, (size_t)ncol * kClosureFields * nv * 4)) {
-    if (cb.x) cudaFree(cb.x);
+  // network buffers for every column: x and y, and two of the widest layer
+  int wmax = 0;
+  for (int l = 0; l < net->n_layers(); ++l) wmax = std::max(wmax, net->ps[l]);
+  const size_t act = (size_t)ncol * wmax * sizeof(__nv_bfloat16);
+  bool ok = !cudaMalloc(&cb.x, (size_t)ncol * 2 * kClosureFields * nv * 4) &&
+            !cudaMalloc(&cb.y, (size_t)ncol * kClosureFields * nv * 4);
+  for (int q = 0; q < 2 && ok && net->tma_ok; ++q) ok = !cudaMalloc(&cb.act[q], act);
+  if (!ok) {
+    s->closure = cb;
+    closure_release(s);
     return THOR_ENOMEM;
   }
   net->stream = s->impl->stream;            // the closure runs on the state's stream

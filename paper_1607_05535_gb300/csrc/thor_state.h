@@ -17,6 +17,7 @@ struct ClosureBinding {
   thor_mlp* net = nullptr;
   const float *in_mean = nullptr, *in_std = nullptr, *out_mean = nullptr, *out_std = nullptr;
   float *x = nullptr, *y = nullptr;   // per-state feature / output buffers
+  void* act[2] = {nullptr, nullptr};  // bfloat16 layer inputs of every column (two of the widest layer)
   int period = 1;                     // large steps per closure window
   long long counter = 0;              // large steps since attach
 };
