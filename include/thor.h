@@ -281,9 +281,10 @@ int thor_launch_count(const thor_state* state, long long* count);
 
 /* Launch-shape knobs (no passage of the paper: the paper's K20 kernels use
  * fixed 2-D blocks of 256 threads, Sec. 5); the results do not depend on them.
- * THOR_TUNE_KCHUNK: levels each thread of the stencil kernels walks (1..256,
- * default 2); fewer levels mean more threads in flight, more levels fewer
- * reloads of the per-column weights.
+ * THOR_TUNE_KCHUNK: levels each thread of the stencil kernels walks (1..256;
+ * the default, 1 to 3, follows from the state's cells and precision); fewer
+ * levels mean more threads in flight, more levels fewer reloads of the
+ * per-column weights.
  * THOR_TUNE_GRAPH: 1 (default) replays a captured CUDA graph of one large
  * step on a non-default stream (re-captured when dt, n_small or the chunk
  * change; never while thor_profile records); 0 launches kernel by kernel.
@@ -400,8 +401,9 @@ int thor_zonal_read_w(thor_state* state, int nlat, double* out, size_t n, long l
  * levels, on two streams (graph branches), joined before the column solve:
  * the levels of a horizontal stencil do not depend on each other, and one
  * chain's kernels fill the SMs the other's leave idle while they start and
- * drain. Default 1 (g6 x 32 large step 1.477 -> 1.426 ms at 4 levels per
- * thread); the same numbers either way (tested bit for bit). */
+ * drain. Default 1 for states large enough to gain from it (from 800 000
+ * cells in THOR_MIXED, 200 000 in THOR_FP64), else 0; the same numbers either
+ * way (tested bit for bit). */
 
 /* Launch-shape autotuner (an extension; the paper fixes no launch shapes).
  * Times `steps` large steps of (n_small, dt) for every levels-per-thread

@@ -561,6 +561,34 @@ int Impl<R>::set_compensated(int on) {
   return THOR_OK;
 }
 
+// Launch shape by size (thor_tune and the autotuner change it; the numbers do
+// not depend on it). Large-step times on a GB300 in us, 128-column blocks:
+//  - levels per thread. Float: few cells want every level as a thread, many
+//    want the stencil weights shared by more levels (1 / 2 / 3 levels:
+//    7.7 k cells 168 / 203 / 240, 77 k 253 / 280 / 313, 123 k 216 / 241 / 271,
+//    379 k 453 / 414 / 458, 492 k 521 / 498 / 506, 1.31 M 1461 / 1290 / 1248).
+//    Float64 is bound by its pipe, and more threads balance it better (51 k
+//    430 / 483 / 537, 328 k 1560 / 1640 / 1690, 1.31 M 6084 / 6087 / 6128).
+//  - the stencils in two level halves on two streams: where one kernel fills
+//    the chip several times over (1.31 M float 1263 -> 1248, float64 6156 ->
+//    6066; 328 k float64 1599 -> 1566), elsewhere they cost (379 k 414 -> 432).
+//  - few cells, float: one shared-memory carveout for every kernel. The staged
+//    solve wants more shared memory than the stencils, and an SM changes the
+//    split only when idle, twice a small step (77 k 253 -> 220, 123 k 216 ->
+//    211; larger grids lose more L1 than they gain, 1.31 M 1263 -> 1319).
+//  - at most a block per SM, float: each kernel starts beside the one before
+//    it (7.7 k 166 -> 152; with more blocks the early ones take the room of
+//    the running ones, 77 k 220 -> 235).
+template <typename R>
+void Impl<R>::shape() {
+  const long long cells = (long long)G.ncol * G.nv;
+  const bool f32 = sizeof(R) == sizeof(float), few = cells < 200000;
+  kchunk = !f32 || few ? 1 : cells < 800000 ? 2 : 3;
+  level_split = cells >= (f32 ? 800000 : 200000);
+  carveout = f32 && few ? 50 : -1;
+  overlap = f32 && few && (long long)((G.ncol + block - 1) / block) * G.nv <= 152;
+}
+
 template Impl<double>::~Impl();
 template Impl<float>::~Impl();
 template int Impl<double>::get(int, double*, size_t);
@@ -571,6 +599,8 @@ template int Impl<double>::diag(double*, long long*);
 template int Impl<double>::set_compensated(int);
 template int Impl<float>::set_compensated(int);
 template int Impl<float>::diag(double*, long long*);
+template void Impl<double>::shape();
+template void Impl<float>::shape();
 
 namespace {
 
@@ -767,6 +797,7 @@ int make_impl(thor_grid* grid, const thor_planet& pl, const thor_init& in, cudaS
   I->forcing = in.forcing;
   I->hj_dT = in.hj_dT;
   I->diff_D = pl.diff_D;
+  I->shape();
   double dbar = std::sqrt(2.0 * M_PI / 5.0) * pl.radius / std::pow(2.0, h.glevel);
   I->dbar4 = dbar * dbar * dbar * dbar;
   Carver dry{nullptr};

@@ -81,6 +81,15 @@ struct Member {
   int* err;                        // the state's device error flag
 };
 
+// How a state's kernels are launched (Impl::shape). after: overlap the start
+// with the kernel before it on the stream (pdl_wait), only where that kernel is
+// the one dependency. carveout: shared memory share of the SM's L1, -1 the
+// driver's choice per kernel.
+struct LaunchHint {
+  bool after = false;
+  int carveout = -1;
+};
+
 // device buffer of the energy fixer and budget: two diagnostics reductions
 // (kDiagBlocks + 1 rows of 8 each), dT in float64, dT in the storage type
 constexpr size_t kFixBufBytes = (size_t)(2 * (512 + 1) * 8 + 2) * sizeof(double);
@@ -112,6 +121,8 @@ struct ImplBase {
   int block = kBlock;                  // threads (columns) per block of the stencil kernels
   int solve_tma = 1;                   // TMA-staged column solve where available
   int level_split = 1;                 // small-step stencils in two level halves on two streams
+  int overlap = 0;                     // start kernels while the one before drains (pdl_wait)
+  int carveout = -1;                   // LaunchHint::carveout of every kernel of the step
   int rk_stages = 3;                   // RK3 stages a large step runs (THOR_TUNE_RK_STAGES; tests)
   int* dev_err = nullptr;              // device flag: 1 = a bounded device wait timed out
   // energy fixer and budget (thor_tune THOR_TUNE_ENERGY_FIXER / THOR_TUNE_BUDGET)
@@ -217,6 +228,7 @@ struct Impl : ImplBase {
   void reset_graph() override { drop_graph(); }
   ~Impl() override;
   void launch_2d(int nplanes, int kchunk, dim3& grid) const;
+  void shape();                    // the defaults of the launch shape for this size
   int large_step(double dt, int n_small);
   // CUDA graph of one large step, replayed while (dt, n_small, kchunk) stay
   // the same; used on a non-default stream when no profiling is recorded
@@ -238,7 +250,7 @@ struct Impl : ImplBase {
   // the state's stream) and its copy (on the side stream)
   cudaEvent_t ev_x[4] = {nullptr, nullptr, nullptr, nullptr};
   int build_solve_maps();
-  cudaError_t launch_solve_tma(dim3 grid, int stage, const Xf<R>& Xo, const Xf<R>& XsL, const Xf<R>& XoL,
+  cudaError_t launch_solve_tma(LaunchHint hint, dim3 grid, int stage, const Xf<R>& Xo, const Xf<R>& XsL, const Xf<R>& XoL,
                                double dtau, int want_div, int last);
   long long graph_launches = 0;
   void drop_graph() {

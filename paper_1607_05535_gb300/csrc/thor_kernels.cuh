@@ -353,6 +353,22 @@ __device__ __forceinline__ T ld(const T* p) { return __ldg(p); }
 // be loaded evict-first and the perturbations kept evict-last, so that the
 // second set has the better chance of staying in L2 (the first alone is
 // what pays at that size). Hints change where a line lives, never a value.
+// Programmatic dependent launch: a kernel launched with programmatic stream
+// serialization starts while the one before it is still running. It may read
+// what no kernel writes (geometry, weights, level constants), and waits here
+// before everything else; kernels call pdl_next first, so that the next one
+// may start once all their blocks have. Without the launch attribute both do
+// nothing. pdl_wait passes an index through: addresses formed from the result
+// cannot be loaded from before the wait (read-only loads are free to move
+// across a memory clobber, not across the value they depend on).
+__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ int pdl_wait(int v) {
+  int o;
+  asm volatile("griddepcontrol.wait;\n\tmov.b32 %0, %1;" : "=r"(o) : "r"(v) : "memory");
+  return o;
+}
+
 enum { kL2Normal = 0, kL2First = 1, kL2Last = 2 };
 __device__ __forceinline__ uint64_t l2_policy(int prio) {
   uint64_t p;

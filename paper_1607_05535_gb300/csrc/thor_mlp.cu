@@ -539,11 +539,6 @@ struct GemmPair {
   int blocks0;                     // CTAs of the first job
 };
 
-// kernels of a pass: run setup while the previous kernel drains, then wait
-// for its results; let the next kernel do the same
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // column sums over a warp's 32 lanes of 16 values per lane: halves of the
 // columns are exchanged, so that 16 shuffles instead of 80 serve; lane l then
 // holds the sum of column bitwise (l >> 1)

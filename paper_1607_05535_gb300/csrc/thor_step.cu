@@ -29,6 +29,28 @@ cudaError_t launch_k(void (*kern)(K...), dim3 grid, dim3 block, size_t smem, cud
   cfg.stream = st;
   return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
 }
+template <typename... K, typename... A>
+cudaError_t launch_hint(LaunchHint hint, void (*kern)(K...), dim3 grid, dim3 block, size_t smem, cudaStream_t st,
+                        A&&... args) {
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = st;
+  cudaLaunchAttribute at[2];
+  int n = 0;
+  if (hint.after) {
+    at[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[n++].val.programmaticStreamSerializationAllowed = 1;
+  }
+  if (hint.carveout >= 0) {
+    at[n].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+    at[n++].val.sharedMemCarveout = (unsigned)hint.carveout;
+  }
+  cfg.attrs = at;
+  cfg.numAttrs = n;
+  return cudaLaunchKernelEx(&cfg, kern, std::forward<A>(args)...);
+}
 
 // Each step of the method is a device function over one block of columns
 // (block indices passed in); the kernels below run it either for one state
@@ -48,10 +70,11 @@ template <typename R, bool HO = false>
 __device__ __forceinline__ void d_derived(const Geo<R>& G, const VR<R>& U, const Phys& ph, const Xf<R>& X, const Work<R>& T, R* pi, int shallow, int kchunk,
                                           int bx, int by) {
   int c = bx * blockDim.x + threadIdx.x;
+  pdl_next();
   if (c >= G.ncol) return;
-  const int S = G.colp;
   const R gamma = pc<R>(ph.gamma, ph.gamma_f), inv_Rd = pc<R>(ph.inv_Rd, ph.inv_Rd_f);
-  R rx = ld(G.rhat + (c)), ry = ld(G.rhat + (S + c)), rz = ld(G.rhat + (2 * S + c));
+  R rx = ld(G.rhat + (c)), ry = ld(G.rhat + (G.colp + c)), rz = ld(G.rhat + (2 * G.colp + c));
+  const int S = pdl_wait(G.colp);
   int k0 = by * kchunk, k1 = min(G.nv + 1, k0 + kchunk);
 #pragma unroll 2
   for (int k = k0; k < k1; ++k) {
@@ -94,10 +117,11 @@ template <typename R, bool HO = false>
 __device__ __forceinline__ void d_lap1(const Geo<R>& G, const VR<R>& U, const Xf<R>& X, const Work<R>& T, R Kd, int kchunk, int bx, int by,
                                        int kend) {
   int c = bx * blockDim.x + threadIdx.x;
+  pdl_next();
   if (c >= G.ncol) return;
-  const int S = G.colp;
   Nbr7 nb = load_nbr(G, c);
-  W7<R> wl = load_w7(G.wlap, S, c);
+  W7<R> wl = load_w7(G.wlap, G.colp, c);
+  const int S = pdl_wait(G.colp);
   int k0 = by * kchunk, k1 = min(kend, k0 + kchunk);
 #pragma unroll 2
   for (int k = k0; k < k1; ++k) {
@@ -135,19 +159,21 @@ template <typename R, bool SH = false, bool HO = false>
 __device__ __forceinline__ void d_slow(const Geo<R>& G, const VR<R>& U, const Phys& ph, const Xf<R>& X, const Work<R>& T, const Slow<R>& SL, int hyper,
                                             R* d0, int kchunk, int bx, int by, int kend) {
   int c = bx * blockDim.x + threadIdx.x;
+  pdl_next();
   if (c >= G.ncol) return;
-  const int S = G.colp;
+  const int S0 = G.colp;
   Nbr7 nb = load_nbr(G, c);
   // the divergence and Laplacian weights; the gradient of p below is taken
   // with the divergence weights plus the centre correction, unprojected
   // (S_M is projected as a whole)
   W7x3<R> wd;
   W7<R> wl;
-  load_w7x3_lap(G.wdiv, S, c, wd, wl);
-  const R gcx = ld(G.gcor + (c)), gcy = ld(G.gcor + (S + c)), gcz = ld(G.gcor + (2 * S + c));
-  R rx = ld(G.rhat + (c)), ry = ld(G.rhat + (S + c)), rz = ld(G.rhat + (2 * S + c));
-  const R tA = ld(G.tb + (2 * S + c));
+  load_w7x3_lap(G.wdiv, S0, c, wd, wl);
+  const R gcx = ld(G.gcor + (c)), gcy = ld(G.gcor + (S0 + c)), gcz = ld(G.gcor + (2 * S0 + c));
+  R rx = ld(G.rhat + (c)), ry = ld(G.rhat + (S0 + c)), rz = ld(G.rhat + (2 * S0 + c));
+  const R tA = ld(G.tb + (2 * S0 + c));
   const R two_om = pc<R>(ph.two_omega, ph.two_omega_f), Rd = pc<R>(ph.Rd, ph.Rd_f);
+  const int S = pdl_wait(G.colp);
   int k0 = by * kchunk, k1 = min(kend, k0 + kchunk);
   constexpr int kUnroll = sizeof(R) == sizeof(float) ? 2 : 1;   // float64: registers
 #pragma unroll kUnroll
@@ -294,11 +320,12 @@ __device__ __forceinline__ void d_slow_w(const Geo<R>& G, const VR<R>& U, const 
                                          const Pert<R>& P, int hyper, int init, int kchunk, int bx, int by,
                                          const Xf<R>& XtL = Xf<R>{}) {
   int c = bx * blockDim.x + threadIdx.x;
+  pdl_next();
   if (c >= G.ncol) return;
-  const int S = G.colp;
   Nbr7 nb = load_nbr(G, c);
-  W7<R> wl = load_w7(G.wlap, S, c);
-  const Tan<R> tb = load_tan(G.tb, S, c);
+  W7<R> wl = load_w7(G.wlap, G.colp, c);
+  const Tan<R> tb = load_tan(G.tb, G.colp, c);
+  const int S = pdl_wait(G.colp);
   const R g = pc<R>(ph.g, ph.g_f);
   int k0 = by * kchunk, k1 = min(G.nv + 1, k0 + kchunk);
 #pragma unroll 2
@@ -362,9 +389,10 @@ template <typename R>
 __device__ __forceinline__ void d_stage_init(const Geo<R>& G, const VR<R>& U, const Phys& ph, const Xf<R>& Xt, const Xf<R>& X, const R* pi, const Pert<R>& P,
                                              const Xf<R>& XtL, const Xf<R>& XL, int zero, int kchunk, int bx, int by) {
   int c = bx * blockDim.x + threadIdx.x;
+  pdl_next();
   if (c >= G.ncol) return;
-  const int S = G.colp;
-  const Tan<R> tb = load_tan(G.tb, S, c);
+  const Tan<R> tb = load_tan(G.tb, G.colp, c);
+  const int S = pdl_wait(G.colp);
   const bool cmp = XtL.rho != nullptr;
   int k0 = by * kchunk, k1 = min(G.nv + 1, k0 + kchunk);
 #pragma unroll 2
@@ -427,11 +455,12 @@ template <typename R>
 __device__ __forceinline__ void d_ss_lapd(const Geo<R>& G, const VR<R>& U, const Work<R>& T, const R* dsrc, const R* pstar, R Kd,
                                           int kchunk, int bx, int by) {
   int c = bx * blockDim.x + threadIdx.x;
+  pdl_next();
   if (c >= G.ncol) return;
-  const int S = G.colp;
   const uint64_t pk = pol_keep<R>();
   Nbr7 nb = load_nbr(G, c);
-  W7<R> wl = load_w7(G.wlap, S, c);
+  W7<R> wl = load_w7(G.wlap, G.colp, c);
+  const int S = pdl_wait(G.colp);
   int k0 = by * kchunk, k1 = min(G.nv, k0 + kchunk);
 #pragma unroll 2
   for (int k = k0; k < k1; ++k) {
@@ -458,11 +487,12 @@ __device__ __forceinline__ void d_ss_mom(const Geo<R>& G, const VR<R>& U, const 
                                             int divdamp, const Xf<R>& Xs, const Xf<R>& Xo, const Xf<R>& XsL, const Xf<R>& XoL, int last,
                                             int kchunk, int bx, int by) {
   int c = bx * blockDim.x + threadIdx.x;
+  pdl_next();
   if (c >= G.ncol) return;
-  const int S = G.colp;
   const uint64_t ps = pol_stream(), pk = pol_keep<R>();
   Nbr7 nb = load_nbr(G, c);
-  W7x2<R> wg = load_w7x2(G.wg2, S, c);
+  W7x2<R> wg = load_w7x2(G.wg2, G.colp, c);
+  const int S = pdl_wait(G.colp);
   const R* q = divdamp ? T.lp : P.p;
   int k0 = by * kchunk, k1 = min(G.nv, k0 + kchunk);
 #pragma unroll 2
@@ -536,11 +566,12 @@ __device__ __forceinline__ FluxCell<R> flux_cell(const W7x2<R>& wd, const Nbr7& 
 template <typename R>
 __device__ __forceinline__ void d_ss_flux(const Geo<R>& G, const VR<R>& U, const Slow<R>& SL, const Pert<R>& P, const Work<R>& T, R dtau, int kchunk, int bx, int by) {
   int c = bx * blockDim.x + threadIdx.x;
+  pdl_next();
   if (c >= G.ncol) return;
-  const int S = G.colp;
   const uint64_t ps = pol_stream(), pk = pol_keep<R>();
   Nbr7 nb = load_nbr(G, c);
-  W7x2<R> wd = load_w7x2(G.wd2, S, c);
+  W7x2<R> wd = load_w7x2(G.wd2, G.colp, c);
+  const int S = pdl_wait(G.colp);
   int k0 = by * kchunk, k1 = min(G.nv, k0 + kchunk);
 #pragma unroll 2
   for (int k = k0; k < k1; ++k) {
@@ -586,7 +617,8 @@ __device__ __forceinline__ void fac_store(const Fac<R>& F, int i, double inv, do
 template <typename R>
 __device__ __forceinline__ void d_ss_factor(const Geo<R>& G, const VR<R>& U, const Phys& ph, const Slow<R>& SL, const Fac<R>& F,
                                             double dtau, int bx, int by) {
-  const int nv = G.nv, S = G.colp, N = nv - 1;
+  pdl_next();
+  const int nv = G.nv, S = pdl_wait(G.colp), N = nv - 1;
   const int tx = threadIdx.x & 31, half = threadIdx.x >> 5;
   const int c = bx * 32 + tx;
   const bool valid = c < G.ncol;
@@ -739,9 +771,10 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
                                             int want_div, const Xf<R>& Xo, const Xf<R>& XsL, const Xf<R>& XoL, int last, int bx,
                                             int by) {
   extern __shared__ double sm[];
-  const int nv = G.nv, S = G.colp, N = nv - 1;
+  pdl_next();
+  const int nv = G.nv, S = pdl_wait(G.colp), N = nv - 1;
   const int tx = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int c = bx * 32 + tx;
+  const int c = pdl_wait(bx * 32 + tx);
   const bool valid = c < G.ncol;
   const int cs = valid ? c : 0;          // padding lanes read column 0 and store nothing
   double* sdp = sm;                      // [nv + 1][32] d' / f', then W
@@ -915,7 +948,8 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
 // and changes the lowest layer's rho theta)
 template <typename R>
 __device__ __forceinline__ void d_surface_p(const Geo<R>& G, const VR<R>& U, const Phys& ph, const Xf<R>& X, const Work<R>& T, int bx) {
-  int c = bx * blockDim.x + threadIdx.x;
+  pdl_next();
+  const int c = pdl_wait((int)(bx * blockDim.x + threadIdx.x));
   if (c >= G.ncol) return;
   const R Rd = pc<R>(ph.Rd, ph.Rd_f);
   R p0 = ld(U.pb + (0)) + eos_level(U, ph, 0, ld(X.th + (c)));
@@ -930,7 +964,8 @@ __device__ __forceinline__ void d_surface_p(const Geo<R>& G, const VR<R>& U, con
 template <typename R>
 __device__ __forceinline__ void d_physics(const Geo<R>& G, const VR<R>& U, const Phys& ph, const Xf<R>& X, const Xf<R>& XL, const Work<R>& T, int forcing,
                                           double dt, double hj_dT, int kchunk, int bx, int by) {
-  int c = bx * blockDim.x + threadIdx.x;
+  pdl_next();
+  const int c = pdl_wait((int)(bx * blockDim.x + threadIdx.x));
   if (c >= G.ncol) return;
   const int S = G.colp;
   const R gamma = pc<R>(ph.gamma, ph.gamma_f), inv_gamma = pc<R>(ph.inv_gamma, ph.inv_gamma_f),
@@ -1345,7 +1380,6 @@ __device__ __forceinline__ void d_ss_solve_tma(const Geo<float>& G, const VR<flo
   extern __shared__ unsigned char smraw[];
   const int nv = G.nv;
   const int tid = threadIdx.x, tx = tid & 31, warp = tid >> 5;
-  const int c0 = bx * 32, c = c0 + tx;
   unsigned char* base = smraw + ((128u - (smem_u32(smraw) & 127u)) & 127u);
   const SolveSm s = solve_sm(base, nv);
   float2* sx = reinterpret_cast<float2*>(base + solve_stage_bytes(nv));   // [2][32]
@@ -1355,6 +1389,8 @@ __device__ __forceinline__ void d_ss_solve_tma(const Geo<float>& G, const VR<flo
     mbar_init(bar, 1);
     mbar_init_fence();
   }
+  pdl_next();
+  const int c0 = pdl_wait(bx * 32), c = c0 + tx;
   __syncthreads();
   if (tid == 0) solve_issue(s, M, c0, bar, nv, stage0, want_div);
   if (!__syncthreads_and(mbar_wait(bar, 0))) {
@@ -1534,7 +1570,7 @@ static bool raise_smem_limit(K* kernel, int bytes) {
 }
 
 template <typename R>
-int col_kernel_setup(int nv) {
+int col_kernel_setint nv {
   const int bytes = (int)solve_smem_bytes(nv);
   return raise_smem_limit(k_ss_solve<R>, bytes) && raise_smem_limit(ke_ss_solve<R>, bytes) ? 0 : -3;
 }
@@ -1554,11 +1590,13 @@ int Impl<R>::large_step(double dt, int n_small) {
   // level halves of the small-step stencils (THOR_TUNE_LEVEL_SPLIT): levels
   // [0, kc * hc) on the state's stream, [kc * hc, nv) on side2
   const bool lsplit = level_split && side != nullptr && !prof_on && side2 != nullptr && G.nv >= 2 * kc;
+  const bool pdl = overlap && !lsplit && !prof_on && stream != nullptr;
+  auto hint = [&](bool after) { return LaunchHint{after, carveout}; };
   const int nch = (G.nv + kc - 1) / kc, hc = lsplit ? nch / 2 : nch;
   dim3 glo(g2.x, hc), ghi(g2.x, nch - hc);
   const R Kd = (R)(diff_D * dbar4 / dt);
-  auto lapd = [&](cudaStream_t st, const R* dsrc, dim3 g, int klo, int khi) -> cudaError_t {
-    return launch_k(k_ss_lapd<R>, g, bs, 0, st, G, U, T, dsrc, (const R*)P.p, Kd, kc, klo, khi);
+  auto lapd = [&](bool after, cudaStream_t st, const R* dsrc, dim3 g, int klo, int khi) -> cudaError_t {
+    return launch_hint(hint(after), k_ss_lapd<R>, g, bs, 0, st, G, U, T, dsrc, (const R*)P.p, Kd, kc, klo, khi);
   };
   const double dts[3] = {dt / 3.0, dt / n_small, dt / n_small};
   const int nsub[3] = {1, n_small / 2, n_small};
@@ -1597,7 +1635,7 @@ int Impl<R>::large_step(double dt, int n_small) {
     cudaStream_t aux = fork ? side : stream;
     mark(THOR_K_DERIVED, true);
     const bool ho = ph.vorder > 1;
-    chk(launch_k(ho ? k_derived<R, true> : k_derived<R, false>, g2i, bs, 0, stream, G, U, ph, Xs, T, SL.pi, shallow, kc));
+    chk(launch_hint(hint(pdl && s > 0), ho ? k_derived<R, true> : k_derived<R, false>, g2i, bs, 0, stream, G, U, ph, Xs, T, SL.pi, shallow, kc));
     mark(THOR_K_DERIVED, false);
     ++launches;
     if (fork) {
@@ -1605,27 +1643,27 @@ int Impl<R>::large_step(double dt, int n_small) {
       chk(cudaStreamWaitEvent(side, ev_fork, 0));
     }
     mark(THOR_K_STAGE_INIT, true);
-    chk(launch_k(k_stage_init<R>, g2i, bs, 0, aux, G, U, ph, Xt, Xs, (const R*)SL.pi, P, XtL, XsL, (int)(s == 0), kc));
+    chk(launch_hint(hint(false), k_stage_init<R>, g2i, bs, 0, aux, G, U, ph, Xt, Xs, (const R*)SL.pi, P, XtL, XsL, (int)(s == 0), kc));
     mark(THOR_K_STAGE_INIT, false);
     ++launches;
     const bool early_grad = divdamp && s > 0;    // D of X^t is ready before the slow terms
     if (early_grad) {
       mark(THOR_K_SS_LAPD, true);
-      chk(lapd(aux, (const R*)T.dd0, g2, 0, G.nv));
+      chk(lapd(pdl, aux, (const R*)T.dd0, g2, 0, G.nv));
       mark(THOR_K_SS_LAPD, false);
       ++launches;
     }
     if (fork) chk(cudaEventRecord(ev_join0, side));
     if (hyper) {
       mark(THOR_K_LAP1, true);
-      chk(launch_k(ho ? k_lap1<R, true> : k_lap1<R, false>, g2i, bs, 0, stream, G, U, Xs, T, Kd, kc, 0, G.nv + 1));
+      chk(launch_hint(hint(pdl), ho ? k_lap1<R, true> : k_lap1<R, false>, g2i, bs, 0, stream, G, U, Xs, T, Kd, kc, 0, G.nv + 1));
       mark(THOR_K_LAP1, false);
       ++launches;
     }
     mark(THOR_K_SLOW, true);
     auto slow = shallow ? (ho ? k_slow<R, true, true> : k_slow<R, true, false>)
                         : (ho ? k_slow<R, false, true> : k_slow<R, false, false>);
-    chk(launch_k(slow, g2, bs, 0, stream, G, U, ph, Xs, T, SL, hyper,
+    chk(launch_hint(hint(pdl), slow, g2, bs, 0, stream, G, U, ph, Xs, T, SL, hyper,
                  s == 0 && divdamp ? T.dd0 : (R*)nullptr, kc, 0, G.nv));
     mark(THOR_K_SLOW, false);
     ++launches;
@@ -1637,11 +1675,11 @@ int Impl<R>::large_step(double dt, int n_small) {
       chk(cudaStreamWaitEvent(side, ev_fork, 0));
     }
     mark(THOR_K_SLOW_W, true);
-    chk(launch_k(ho ? k_slow_w<R, true> : k_slow_w<R, false>, g2i, bs, 0, aux, G, U, ph, Xt, Xs, T, SL, P, hyper, 0,
+    chk(launch_hint(hint(false), ho ? k_slow_w<R, true> : k_slow_w<R, false>, g2i, bs, 0, aux, G, U, ph, Xt, Xs, T, SL, P, hyper, 0,
                  kc));
     mark(THOR_K_SLOW_W, false);
     mark(THOR_K_SS_FACTOR, true);
-    chk(launch_k(k_ss_factor<R>, gsolve, 64, 0, aux, G, U, ph, SL, F, dts[s]));
+    chk(launch_hint(hint(pdl), k_ss_factor<R>, gsolve, 64, 0, aux, G, U, ph, SL, F, dts[s]));
     mark(THOR_K_SS_FACTOR, false);
     if (fork) {
       chk(cudaEventRecord(ev_join, side));
@@ -1656,16 +1694,16 @@ int Impl<R>::large_step(double dt, int n_small) {
         // D: of X^t in the first small step, then from the previous column step
         if (divdamp && !(j == 0 && early_grad)) {
           mark(THOR_K_SS_LAPD, true);
-          chk(lapd(st, (const R*)(j == 0 ? T.dd0 : T.dd), g, klo, khi));
+          chk(lapd(pdl && j > 0, st, (const R*)(j == 0 ? T.dd0 : T.dd), g, klo, khi));
           mark(THOR_K_SS_LAPD, false);
           ++launches;
         }
         mark(THOR_K_SS_MOM, true);
-        chk(launch_k(last ? k_ss_mom<R, true> : k_ss_mom<R, false>, g, bs, 0, st, G, U, SL, P, T, (R)dts[s],
+        chk(launch_hint(hint(pdl && (j > 0 || (divdamp && !early_grad))), last ? k_ss_mom<R, true> : k_ss_mom<R, false>, g, bs, 0, st, G, U, SL, P, T, (R)dts[s],
                      divdamp, Xs, Xo, XsL, XoL, kc, klo, khi));
         mark(THOR_K_SS_MOM, false);
         mark(THOR_K_SS_FLUX, true);
-        chk(launch_k(k_ss_flux<R>, g, bs, 0, st, G, U, SL, P, T, (R)dts[s], kc, klo, khi));
+        chk(launch_hint(hint(pdl), k_ss_flux<R>, g, bs, 0, st, G, U, SL, P, T, (R)dts[s], kc, klo, khi));
         mark(THOR_K_SS_FLUX, false);
         launches += 2;
       };
@@ -1683,9 +1721,9 @@ int Impl<R>::large_step(double dt, int n_small) {
       if (fork && j == 0) chk(cudaStreamWaitEvent(stream, ev_join, 0));
       mark(THOR_K_SS_SOLVE, true);
       if (staged)
-        chk(launch_solve_tma(gsolve, s, Xo, XsL, XoL, dts[s], want_div, last));
+        chk(launch_solve_tma(hint(pdl && j > 0), gsolve, s, Xo, XsL, XoL, dts[s], want_div, last));
       else
-        chk(launch_k(k_ss_solve<R>, gsolve, 32 * kSolveWarps, solve_smem, stream, G, U, ph, Xs, SL, P, T, F, dts[s],
+        chk(launch_hint(hint(pdl && j > 0), k_ss_solve<R>, gsolve, 32 * kSolveWarps, solve_smem, stream, G, U, ph, Xs, SL, P, T, F, dts[s],
                      want_div, Xo, XsL, XoL, last));
       mark(THOR_K_SS_SOLVE, false);
       ++launches;
@@ -1704,8 +1742,8 @@ int Impl<R>::large_step(double dt, int n_small) {
   }
   if (forcing != 0 && nstages == 3) {
     mark(THOR_K_PHYSICS, true);
-    chk(launch_k(k_surface_p<R>, g1, bs, 0, stream, G, U, ph, Xt, T));
-    chk(launch_k(k_physics<R>, g2, bs, 0, stream, G, U, ph, Xt, XtL, T, forcing, dt, hj_dT, kc));
+    chk(launch_hint(hint(pdl && !energy), k_surface_p<R>, g1, bs, 0, stream, G, U, ph, Xt, T));
+    chk(launch_hint(hint(pdl), k_physics<R>, g2, bs, 0, stream, G, U, ph, Xt, XtL, T, forcing, dt, hj_dT, kc));
     mark(THOR_K_PHYSICS, false);
     launches += 2;
   }
@@ -1727,9 +1765,6 @@ int Impl<R>::anelastic_step(double dt) {
   launch_2d(G.nv + 1, kc, g2i);
   dim3 g1((G.ncol + bs - 1) / bs);
   const R Kd = (R)(diff_D * dbar4 / dt);
-  auto lapd = [&](cudaStream_t st, const R* dsrc, dim3 g, int klo, int khi) -> cudaError_t {
-    return launch_k(k_ss_lapd<R>, g, bs, 0, st, G, U, T, dsrc, (const R*)P.p, Kd, kc, klo, khi);
-  };
   const double dts[3] = {dt / 3.0, dt / 2.0, dt};
   const bool ho = ph.vorder > 1;
   for (int s = 0; s < 3; ++s) {
@@ -1763,13 +1798,13 @@ template int Impl<double>::anelastic_step(double);
 template int Impl<float>::anelastic_step(double);
 
 template <>
-cudaError_t Impl<float>::launch_solve_tma(dim3 grid, int stage, const Xf<float>& Xo, const Xf<float>& XsL,
+cudaError_t Impl<float>::launch_solve_tma(LaunchHint hint, dim3 grid, int stage, const Xf<float>& Xo, const Xf<float>& XsL,
                                           const Xf<float>& XoL, double dtau, int want_div, int last) {
-  return launch_k(k_ss_solve_tma, grid, 32 * kSolveWarps, solve_tma_smem_bytes(G.nv), stream, G, U, ph, *smaps,
+  return launch_hint(hint, k_ss_solve_tma, grid, 32 * kSolveWarps, solve_tma_smem_bytes(G.nv), stream, G, U, ph, *smaps,
                   (int)(stage == 0), stage == 0 ? Xt : Xst, SL, P, T, dtau, want_div, Xo, XsL, XoL, last, dev_err);
 }
 template <>
-cudaError_t Impl<double>::launch_solve_tma(dim3, int, const Xf<double>&, const Xf<double>&, const Xf<double>&,
+cudaError_t Impl<double>::launch_solve_tma(LaunchHint, dim3, int, const Xf<double>&, const Xf<double>&, const Xf<double>&,
                                            double, int, int) {
   return cudaErrorInvalidValue;
 }
