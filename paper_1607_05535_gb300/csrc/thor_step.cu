@@ -1570,7 +1570,7 @@ static bool raise_smem_limit(K* kernel, int bytes) {
 }
 
 template <typename R>
-int col_kernel_setint nv {
+int col_kernel_setup(int nv) {
   const int bytes = (int)solve_smem_bytes(nv);
   return raise_smem_limit(k_ss_solve<R>, bytes) && raise_smem_limit(ke_ss_solve<R>, bytes) ? 0 : -3;
 }
