@@ -245,8 +245,11 @@ int upload_tables(Impl<R>& I, const HostGrid& h, const std::vector<double>* vert
   std::vector<R> wdiv(28 * (size_t)S, 0), wgrad(28 * (size_t)S, 0), wlap(7 * (size_t)S, 0),
       rhat(3 * (size_t)S, 0), gcor(3 * (size_t)S, 0), sl(S, 0), cl(S, 0), clon(S, 0), tb(3 * (size_t)S, 0),
       wg2(14 * (size_t)S, 0), wd2(14 * (size_t)S, 0);
-  // e1 and e2 of the tangent basis at column c (thor_kernels.cuh)
-  auto basis = [&](int c, double e[2][3]) {
+  // e1 and e2 of every column's tangent basis (thor_kernels.cuh)
+  std::vector<double> bas(6 * (size_t)ncol);
+#pragma omp parallel for schedule(static)
+  for (int c = 0; c < ncol; ++c) {
+    double(*e)[3] = reinterpret_cast<double(*)[3]>(&bas[6 * (size_t)c]);
     const double x = h.P[3 * c], y = h.P[3 * c + 1], z = h.P[3 * c + 2], s = z < 0.0 ? -1.0 : 1.0;
     const double X = s * x, Y = s * y, A = -1.0 / (1.0 + std::fabs(z));
     e[0][0] = 1.0 + A * X * X;
@@ -257,24 +260,23 @@ int upload_tables(Impl<R>& I, const HostGrid& h, const std::vector<double>* vert
     tb[c] = (R)X;
     tb[S + c] = (R)Y;
     tb[2 * (size_t)S + c] = (R)A;
-  };
+  }
   std::vector<double> area(S, 0.0);
+#pragma omp parallel for schedule(static)
   for (int c = 0; c < ncol; ++c) {
     for (int j = 0; j < 6; ++j) {
       int q = h.nbr[6 * c + j];
       nbr[(size_t)j * S + c] = q < 0 ? c : q;
     }
-    double own[2][3];
-    basis(c, own);
+    const double* own = &bas[6 * (size_t)c];
     for (int j = 0; j < 7; ++j) {
       const int m = j == 0 || h.nbr[6 * c + j - 1] < 0 ? c : h.nbr[6 * c + j - 1];
-      double there[2][3];
-      basis(m, there);
+      const double* there = &bas[6 * (size_t)m];
       for (int a = 0; a < 2; ++a) {
         double g = 0.0, d = 0.0;
         for (int k = 0; k < 3; ++k) {
-          g += h.w_grad[21 * c + 3 * j + k] * own[a][k];
-          d += h.w_div[21 * c + 3 * j + k] * there[a][k];
+          g += h.w_grad[21 * c + 3 * j + k] * own[3 * a + k];
+          d += h.w_div[21 * c + 3 * j + k] * there[3 * a + k];
         }
         wg2[((size_t)j * S + c) * 2 + a] = (R)g;
         wd2[((size_t)j * S + c) * 2 + a] = (R)d;

@@ -24,7 +24,7 @@ struct EnsBase {
   virtual int step(int n_large, const int* n_small, const double* dt) = 0;
   virtual void drop_graph() = 0;
   long long launches = 0;
-  int kchunk = 2, block = kBlock, use_graph = 1;
+  int kchunk = 2, block = kMaxBlock, use_graph = 1;   // kchunk: make_ens
 };
 
 template <typename R>
@@ -271,12 +271,23 @@ int make_ens(thor_ensemble* E) {
   using namespace thor;
   auto impl = std::make_unique<EnsImpl<R>>();
   impl->stream = E->stream;
+  long long cells = 0;
   for (thor_state* s : E->members) {
     impl->mem.push_back(static_cast<Impl<R>*>(s->impl.get()));
+    cells += (long long)impl->mem.back()->G.ncol * impl->mem.back()->G.nv;
     cudaStream_t ms = s->impl->stream;
     if (ms != E->stream && std::find(impl->streams.begin(), impl->streams.end(), ms) == impl->streams.end())
       impl->streams.push_back(ms);
   }
+  // Levels per thread by size (as Impl::shape, the numbers do not depend on
+  // it), blocks of 256 threads. Large steps in us on a GB300 at 1 / 2 / 3 / 6 / 8
+  // levels: float, 211 k cells 455 / 448 / 477 / 600 / 695, 948 k 1472 / 1361 /
+  // 1293 / 1319 / 1394, 3.9 M 5367 / 4741 / 4468 / 4254 / 4409, 10.7 M 15307 / 13345
+  // / 12485 / 11720 / 11415; float64 (its pipe) 348 k 1911 / 2014 / 2058, 3.0 M the
+  // same at all.
+  const bool f32 = sizeof(R) == sizeof(float);
+  impl->kchunk = !f32 ? (cells < 1000000 ? 1 : 3)
+                      : cells < 500000 ? 2 : cells < 1500000 ? 3 : cells < 5000000 ? 6 : 8;
   if (cudaEventCreateWithFlags(&impl->ev_in, cudaEventDisableTiming) ||
       cudaEventCreateWithFlags(&impl->ev_out, cudaEventDisableTiming))
     return THOR_ECUDA;

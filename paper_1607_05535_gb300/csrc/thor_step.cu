@@ -1428,16 +1428,21 @@ __global__ void __launch_bounds__(32 * kSolveWarps)
 
 // The block's member record is copied to shared memory once, and the device
 // functions read its fields from there as they need them (by reference), so
-// that the record's pointers do not all occupy registers.
+// that the record's pointers do not all occupy registers. The copy (1.3 KB and
+// a barrier) costs a block as much as a level of its stencils, so the stencil
+// blocks hold several level chunks of their columns (threadIdx.y).
 template <typename T>
 __device__ __forceinline__ const T& stage_record(const T* src, T* dst) {
   static_assert(sizeof(T) % 4 == 0, "record of whole words");
   const uint32_t* a = reinterpret_cast<const uint32_t*>(src);
   uint32_t* b = reinterpret_cast<uint32_t*>(dst);
-  for (int w = threadIdx.x; w < (int)(sizeof(T) / 4); w += blockDim.x) b[w] = a[w];
+  for (int w = threadIdx.y * blockDim.x + threadIdx.x; w < (int)(sizeof(T) / 4); w += blockDim.x * blockDim.y) b[w] = a[w];
   __syncthreads();
   return *dst;
 }
+
+// the level chunk of a thread of the stencil kernels
+__device__ __forceinline__ int member_chunk() { return blockIdx.y * blockDim.y + threadIdx.y; }
 
 #define THOR_MEMBER()                                   \
   __shared__ Member<R> a_sm;                            \
@@ -1449,17 +1454,17 @@ template <typename R>
 __global__ void ke_derived(const Member<R>* __restrict__ M, const int2* __restrict__ map, int s, int kchunk) {
   THOR_MEMBER();
   if (a.ph.vorder > 1)
-    d_derived<R, true>(a.G, a.U, a.ph, Xs, a.T, a.SL.pi, a.shallow, kchunk, e.y, blockIdx.y);
+    d_derived<R, true>(a.G, a.U, a.ph, Xs, a.T, a.SL.pi, a.shallow, kchunk, e.y, member_chunk());
   else
-    d_derived<R>(a.G, a.U, a.ph, Xs, a.T, a.SL.pi, a.shallow, kchunk, e.y, blockIdx.y);
+    d_derived<R>(a.G, a.U, a.ph, Xs, a.T, a.SL.pi, a.shallow, kchunk, e.y, member_chunk());
 }
 template <typename R>
 __global__ void ke_lap1(const Member<R>* __restrict__ M, const int2* __restrict__ map, int s, int kchunk) {
   THOR_MEMBER();
   if (a.hyper && a.ph.vorder > 1)
-    d_lap1<R, true>(a.G, a.U, Xs, a.T, a.Kd, kchunk, e.y, blockIdx.y, a.G.nv + 1);
+    d_lap1<R, true>(a.G, a.U, Xs, a.T, a.Kd, kchunk, e.y, member_chunk(), a.G.nv + 1);
   else if (a.hyper)
-    d_lap1<R>(a.G, a.U, Xs, a.T, a.Kd, kchunk, e.y, blockIdx.y, a.G.nv + 1);
+    d_lap1<R>(a.G, a.U, Xs, a.T, a.Kd, kchunk, e.y, member_chunk(), a.G.nv + 1);
 }
 template <typename R>
 __global__ void __launch_bounds__(kMaxBlock, 2)
@@ -1468,22 +1473,22 @@ __global__ void __launch_bounds__(kMaxBlock, 2)
   R* d0 = s == 0 && a.divdamp ? a.T.dd0 : nullptr;
   const bool ho = a.ph.vorder > 1;
   if (a.shallow && ho)
-    d_slow<R, true, true>(a.G, a.U, a.ph, Xs, a.T, a.SL, a.hyper, d0, kchunk, e.y, blockIdx.y, a.G.nv);
+    d_slow<R, true, true>(a.G, a.U, a.ph, Xs, a.T, a.SL, a.hyper, d0, kchunk, e.y, member_chunk(), a.G.nv);
   else if (a.shallow)
-    d_slow<R, true>(a.G, a.U, a.ph, Xs, a.T, a.SL, a.hyper, d0, kchunk, e.y, blockIdx.y, a.G.nv);
+    d_slow<R, true>(a.G, a.U, a.ph, Xs, a.T, a.SL, a.hyper, d0, kchunk, e.y, member_chunk(), a.G.nv);
   else if (ho)
-    d_slow<R, false, true>(a.G, a.U, a.ph, Xs, a.T, a.SL, a.hyper, d0, kchunk, e.y, blockIdx.y, a.G.nv);
+    d_slow<R, false, true>(a.G, a.U, a.ph, Xs, a.T, a.SL, a.hyper, d0, kchunk, e.y, member_chunk(), a.G.nv);
   else
-    d_slow<R, false>(a.G, a.U, a.ph, Xs, a.T, a.SL, a.hyper, d0, kchunk, e.y, blockIdx.y, a.G.nv);
+    d_slow<R, false>(a.G, a.U, a.ph, Xs, a.T, a.SL, a.hyper, d0, kchunk, e.y, member_chunk(), a.G.nv);
 }
 template <typename R>
 __global__ void ke_slow_w(const Member<R>* __restrict__ M, const int2* __restrict__ map, int s, int kchunk) {
   THOR_MEMBER();
   const Xf<R> XtL = s == 0 ? Xf<R>{} : a.XtL;      // stage 0: X^(s) is X^t, pair and all
   if (a.ph.vorder > 1)
-    d_slow_w<R, true>(a.G, a.U, a.ph, a.Xt, Xs, a.T, a.SL, a.P, a.hyper, 1, kchunk, e.y, blockIdx.y, XtL);
+    d_slow_w<R, true>(a.G, a.U, a.ph, a.Xt, Xs, a.T, a.SL, a.P, a.hyper, 1, kchunk, e.y, member_chunk(), XtL);
   else
-    d_slow_w<R>(a.G, a.U, a.ph, a.Xt, Xs, a.T, a.SL, a.P, a.hyper, 1, kchunk, e.y, blockIdx.y, XtL);
+    d_slow_w<R>(a.G, a.U, a.ph, a.Xt, Xs, a.T, a.SL, a.P, a.hyper, 1, kchunk, e.y, member_chunk(), XtL);
 }
 template <typename R>
 __global__ void __launch_bounds__(64)
@@ -1498,7 +1503,7 @@ __global__ void ke_ss_lapd(const Member<R>* __restrict__ M, const int2* __restri
   THOR_MEMBER();
   Geo<R> G = a.G;
   G.nv = khi;
-  if (a.divdamp) d_ss_lapd<R>(G, a.U, a.T, j == 0 ? a.T.dd0 : a.T.dd, a.P.p, a.Kd, kchunk, e.y, blockIdx.y + klo);
+  if (a.divdamp) d_ss_lapd<R>(G, a.U, a.T, j == 0 ? a.T.dd0 : a.T.dd, a.P.p, a.Kd, kchunk, e.y, member_chunk() + klo);
 }
 template <typename R>
 __global__ void ke_ss_mom(const Member<R>* __restrict__ M, const int2* __restrict__ map, int s, int j,
@@ -1508,7 +1513,7 @@ __global__ void ke_ss_mom(const Member<R>* __restrict__ M, const int2* __restric
   G.nv = khi;
   d_ss_mom<R>(G, a.U, a.SL, a.P, a.T, (R)a.dts[s], a.divdamp, Xs, s == 2 ? a.Xt : a.Xst,
               s == 0 ? a.XtL : Xf<R>{}, s == 2 ? a.XtL : Xf<R>{}, j + 1 == a.nsub[s], kchunk, e.y,
-              blockIdx.y + klo);
+              member_chunk() + klo);
 }
 template <typename R>
 __global__ void ke_ss_flux(const Member<R>* __restrict__ M, const int2* __restrict__ map, int s, int kchunk,
@@ -1516,7 +1521,7 @@ __global__ void ke_ss_flux(const Member<R>* __restrict__ M, const int2* __restri
   THOR_MEMBER();
   Geo<R> G = a.G;
   G.nv = khi;
-  d_ss_flux<R>(G, a.U, a.SL, a.P, a.T, (R)a.dts[s], kchunk, e.y, blockIdx.y + klo);
+  d_ss_flux<R>(G, a.U, a.SL, a.P, a.T, (R)a.dts[s], kchunk, e.y, member_chunk() + klo);
 }
 template <typename R>
 __global__ void __launch_bounds__(32 * kSolveWarps)
@@ -1880,32 +1885,36 @@ template <typename R>
 int ensemble_large_step(const EnsPlan<R>& E, cudaStream_t stream, long long* launches) {
   const int kc = E.kchunk, bs = E.block;
   const int yc = (E.nv + kc - 1) / kc, yci = (E.nv + 1 + kc - 1) / kc;
+  // blocks of bs columns x rows level chunks
+  const int rows = max(1, kMaxBlock / bs);
+  const dim3 tb(bs, rows);
+  auto up = [&](int chunks) { return (chunks + rows - 1) / rows; };
   const size_t solve_smem = solve_smem_bytes(E.nv);
   const Member<R>* M = E.M;
   long long n = 0;
   for (int s = 0; s < 3; ++s) {
-    const dim3 g2(E.nblk, yc), g2i(E.nblk, yci);
-    ke_derived<R><<<g2i, bs, 0, stream>>>(M, E.map, s, kc);
+    const dim3 g2(E.nblk, up(yc)), g2i(E.nblk, up(yci));
+    ke_derived<R><<<g2i, tb, 0, stream>>>(M, E.map, s, kc);
     if (E.any_hyper) {
-      ke_lap1<R><<<g2i, bs, 0, stream>>>(M, E.map, s, kc);
+      ke_lap1<R><<<g2i, tb, 0, stream>>>(M, E.map, s, kc);
       ++n;
     }
-    ke_slow<R><<<g2, bs, 0, stream>>>(M, E.map, s, kc);
-    ke_slow_w<R><<<g2i, bs, 0, stream>>>(M, E.map, s, kc);
+    ke_slow<R><<<g2, tb, 0, stream>>>(M, E.map, s, kc);
+    ke_slow_w<R><<<g2i, tb, 0, stream>>>(M, E.map, s, kc);
     ke_ss_factor<R><<<E.nblkc, 64, 0, stream>>>(M, E.mapc, s);
     n += 4;
     for (int j = 0; j < E.maxsub[s]; ++j) {
       const int nb = E.active[s][j], nbc = E.activec[s][j];
       // the stencils over level chunks [c0, c1) on st
       auto stencils = [&](cudaStream_t st, int c0, int c1) {
-        const dim3 a2(nb, c1 - c0);
+        const dim3 a2(nb, up(c1 - c0));
         const int khi = min(E.nv, c1 * kc);
         if (E.any_divdamp) {
-          ke_ss_lapd<R><<<a2, bs, 0, st>>>(M, E.map, s, j, kc, c0, khi);
+          ke_ss_lapd<R><<<a2, tb, 0, st>>>(M, E.map, s, j, kc, c0, khi);
           ++n;
         }
-        ke_ss_mom<R><<<a2, bs, 0, st>>>(M, E.map, s, j, kc, c0, khi);
-        ke_ss_flux<R><<<a2, bs, 0, st>>>(M, E.map, s, kc, c0, khi);
+        ke_ss_mom<R><<<a2, tb, 0, st>>>(M, E.map, s, j, kc, c0, khi);
+        ke_ss_flux<R><<<a2, tb, 0, st>>>(M, E.map, s, kc, c0, khi);
         n += 2;
       };
       if (E.side2 && yc >= 2) {
