@@ -1093,7 +1093,7 @@ int thor_checkpoint_save(thor_state* s, void* buf, size_t bytes) {
   h.ref_hash = s->impl->ref_hash;
   h.closure_steps = s->closure.counter;
   char* p = static_cast<char*>(buf);
-  if (cudaMemcpy(p, &h, sizeof(h), cudaMemcpyDefault)) return THOR_ECUDA;
+  if (cudaMemcpyAsync(p, &h, sizeof(h), cudaMemcpyDefault, s->impl->stream)) return THOR_ECUDA;
   if (s->impl->save_state(p + sizeof(h))) return THOR_ECUDA;
   return cudaStreamSynchronize(s->impl->stream) ? THOR_ECUDA : THOR_OK;
 }
