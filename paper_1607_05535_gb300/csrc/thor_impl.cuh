@@ -55,7 +55,7 @@ struct Pert {
 // each a 2-D map (x = column, y = plane) with a box of 32 columns x all planes
 struct SolveMaps {
   CUtensorMap w, sw, cc, ca, thi, cb, pi, th_t, th_s, dsc, dhm;   // float
-  CUtensorMap q, inv, cf, junction;                             // float64 factors
+  CUtensorMap lo, up, inv, junction;                            // the matrix and its factors (Fac)
 };
 
 // Everything the kernels of one state need, as one record: a device array of

@@ -130,10 +130,13 @@ template <> __device__ __forceinline__ float pc<float>(double, float f) { return
 
 // Factors of the per-stage vertical matrix: planes [nv + 1][colp] (rows
 // 1..nv-1 used) and one plane for the junction of the two sweeps. Per row:
-// the pivot reciprocal, c' (downward sweep) or e' (upward sweep), and q, the
-// off-diagonal entry lo (down) or up (up) times the pivot reciprocal. 8
-// bytes per entry: float64 values for float64 states, double-float pairs
-// (float2) for float-storage states.
+// the pivot reciprocal inv, c' (downward sweep) or e' (upward sweep) in cf, and
+// q, the off-diagonal entry lo (down) or up (up) times inv. float64 states keep
+// all three in float64. Float-storage states keep inv as a double-float pair
+// (float2) and, in the place of q and cf, the entries lo and up themselves:
+// both are floats, q and cf are one double-float product each away (q = lo inv
+// and cf = up inv downwards, the other way round upwards), and a small step
+// reads 4 words a row instead of 6.
 template <typename R>
 struct Fac {
   double *inv, *cf, *junction, *q;
@@ -305,11 +308,15 @@ __device__ __forceinline__ float2 df_fms(float ph, float pl, float2 c, float2 x)
   const float h = __fadd_rn(s, e);
   return make_float2(h, __fsub_rn(e, __fsub_rn(h, s)));
 }
+// r a for a float r, not renormalised
+__device__ __forceinline__ float2 df_product(float r, float2 a) {
+  const float h = __fmul_rn(r, a.x);
+  return make_float2(h, __fmaf_rn(r, a.y, __fmaf_rn(r, a.x, -h)));
+}
 // r inv - q d for a float r: the sweep step of the elimination
 __device__ __forceinline__ float2 df_sweep(float r, float2 inv, float2 q, float2 d) {
-  const float ph = __fmul_rn(r, inv.x);
-  const float pl = __fmaf_rn(r, inv.y, __fmaf_rn(r, inv.x, -ph));
-  return df_fms(ph, pl, q, d);
+  const float2 t = df_product(r, inv);
+  return df_fms(t.x, t.y, q, d);
 }
 // a b, renormalised
 __device__ __forceinline__ float2 df_mul(float2 a, float2 b) {

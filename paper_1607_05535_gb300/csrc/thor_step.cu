@@ -646,8 +646,8 @@ __device__ __forceinline__ void d_ss_factor(const Geo<R>& G, const VR<R>& U, con
     // (the float coefficients are exact pairs), stored as pairs
     __shared__ float2 sj2[2][32];
     float2* Finv = reinterpret_cast<float2*>(F.inv);
-    float2* Fcf = reinterpret_cast<float2*>(F.cf);
-    float2* Fq = reinterpret_cast<float2*>(F.q);
+    float* Flo = reinterpret_cast<float*>(F.q);
+    float* Fup = reinterpret_cast<float*>(F.cf);
     float2 last = make_float2(0.f, 0.f);
     if (half == 0) {
       for (int m = 1; m <= p; ++m) {
@@ -657,8 +657,8 @@ __device__ __forceinline__ void d_ss_factor(const Geo<R>& G, const VR<R>& U, con
         last = df_mul_f(up, inv);
         if (valid) {
           Finv[m * S + c] = inv;
-          Fcf[m * S + c] = last;
-          Fq[m * S + c] = df_mul_f(lo, inv);
+          Flo[m * S + c] = lo;
+          Fup[m * S + c] = up;
         }
       }
     } else {
@@ -669,8 +669,8 @@ __device__ __forceinline__ void d_ss_factor(const Geo<R>& G, const VR<R>& U, con
         last = df_mul_f(lo, inv);
         if (valid) {
           Finv[m * S + c] = inv;
-          Fcf[m * S + c] = last;
-          Fq[m * S + c] = df_mul_f(up, inv);
+          Flo[m * S + c] = lo;
+          Fup[m * S + c] = up;
         }
       }
     }
@@ -793,9 +793,9 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
     // float storage: the elimination in double-float, the same operations
     // in the same order as the staged solve (solve_sweeps); W* (float) over
     // the first word of each row of sdp
-    const float2* Fq = reinterpret_cast<const float2*>(F.q);
+    const float* Flo = reinterpret_cast<const float*>(F.q);
     const float2* Finv = reinterpret_cast<const float2*>(F.inv);
-    const float2* Fcf = reinterpret_cast<const float2*>(F.cf);
+    const float* Fup = reinterpret_cast<const float*>(F.cf);
     float2* dp2 = reinterpret_cast<float2*>(sdp);
     float2* sx2 = reinterpret_cast<float2*>(sx);
     float2* cf2 = reinterpret_cast<float2*>(scf);
@@ -804,8 +804,9 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
 #pragma unroll 4
       for (int m = 1; m <= p; ++m) {
         const int i = m * S + cs;
-        cf2[m * 32 + tx] = Fcf[i];
-        d1 = df_sweep(rhs_r(m), Finv[i], Fq[i], d1);
+        const float2 inv = Finv[i];
+        cf2[m * 32 + tx] = df_mul_f(Fup[i], inv);
+        d1 = df_sweep(rhs_r(m), inv, df_mul_f(Flo[i], inv), d1);
         dp2[m * 32 + tx] = d1;
       }
     } else if (warp == 1) {
@@ -813,8 +814,9 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
 #pragma unroll 4
       for (int m = N; m > p; --m) {
         const int i = m * S + cs;
-        cf2[m * 32 + tx] = Fcf[i];
-        f1 = df_sweep(rhs_r(m), Finv[i], Fq[i], f1);
+        const float2 inv = Finv[i];
+        cf2[m * 32 + tx] = df_mul_f(Flo[i], inv);
+        f1 = df_sweep(rhs_r(m), inv, df_mul_f(Fup[i], inv), f1);
         dp2[m * 32 + tx] = f1;
       }
     }
@@ -1199,37 +1201,48 @@ __global__ void k_physics(Geo<R> G, VR<R> U, Phys ph, Xf<R> X, Xf<R> XL, Work<R>
 // ---------------------------------------------------------------- staged column solve (float storage)
 //
 // The column step of d_ss_solve for 32 columns with eight warps. Thread 0
-// stages the planes of the elimination (W*, S_W, c, a, the scaled
-// off-diagonals q, pivot reciprocals, c'/e', junction factors) into shared
-// memory with one
-// cp.async.bulk.tensor per array, and asks the copy engine to prefetch the
-// planes of the final updates into L2. Warps 0 and 1 then run the two float64
-// sweeps out of shared memory (d' overwrites the pivot reciprocal it has just
-// used); afterwards all eight warps share the levels of Eqs. dens2, pt2 and
-// theta_to_p, whose loads now hit L2. Same operations in the same order as
-// d_ss_solve.
+// stages the planes of the elimination (W*, S_W, c, a, the matrix's
+// off-diagonals, pivot reciprocals, junction factors) into shared memory with
+// one cp.async.bulk.tensor per array, and asks the copy engine to prefetch the
+// planes of the final updates into L2. All warps then prepare the rows, each
+// in its own place: rh_m / piv_m as a double-float product over the pivot
+// reciprocal, q over the two off-diagonals, c'/e' over W* and S_W. Warps 0 and
+// 1 run the two sweeps and the back substitution, one dependent double-float
+// multiply-subtract per row; afterwards all eight warps share the levels of
+// Eqs. dens2, pt2 and theta_to_p, whose loads now hit L2. Same operations in
+// the same order as d_ss_solve.
+// Bound by the memory phases of the blocks resident together (DRAM 39% busy):
+// off-diagonals instead of q and c'/e' pairs are 19 words a cell instead of 21
+// and 34 KB a block instead of 43, six blocks an SM instead of five (40
+// registers, the ensemble's kernel too, which took 64). At g6 x 32 30.8 -> 28.9
+// us; 64-member ensemble's large step 11.2 -> 10.6 ms.
 
 // one column group's planes in shared memory (32 columns)
 struct SolveSm {
   float *w, *sw, *cc, *ca;        // w: W*, then the solved W*
-  double *q, *inv, *cf, *junc;    // inv: the pivot reciprocals, then d' and f'
+  float *lo, *up;                 // then q, split into its two words
+  float2 *inv;                    // then rh / piv, then d' and f'
+  float2 *junc;
+  // q and c'/e' of element o (row * 32 + column) after solve_rows
+  __device__ float2 q(int o) const { return make_float2(lo[o], up[o]); }
+  __device__ float2 cf(int o) const { return make_float2(w[o], sw[o]); }
 };
 __device__ __forceinline__ SolveSm solve_sm(unsigned char* base, int nv) {
   SolveSm s;
   s.w = reinterpret_cast<float*>(base);             // [nv + 1][32]
   s.sw = s.w + (nv + 1) * 32;                       // [nv + 1][32]
-  s.cc = s.sw + (nv + 1) * 32;                      // [nv][32]
+  s.lo = s.sw + (nv + 1) * 32;                      // [nv + 1][32]
+  s.up = s.lo + (nv + 1) * 32;                      // [nv + 1][32]
+  s.cc = s.up + (nv + 1) * 32;                      // [nv][32]
   s.ca = s.cc + nv * 32;                            // [nv][32]
-  s.q = reinterpret_cast<double*>(s.ca + nv * 32);  // [nv + 1][32]
-  s.inv = s.q + (nv + 1) * 32;                      // [nv + 1][32]
-  s.cf = s.inv + (nv + 1) * 32;                     // [nv + 1][32]
-  s.junc = s.cf + (nv + 1) * 32;                    // [32]
+  s.inv = reinterpret_cast<float2*>(s.ca + nv * 32);  // [nv + 1][32]
+  s.junc = s.inv + (nv + 1) * 32;                   // [32]
   return s;
 }
 // bytes of one group's planes (a multiple of 128, so every plane and what
 // follows them starts 128-byte aligned)
 __host__ __device__ __forceinline__ size_t solve_stage_bytes(int nv) {
-  return (size_t)(2 * (nv + 1) + 2 * nv) * 128 + (size_t)(3 * (nv + 1) + 1) * 256;
+  return (size_t)(4 * (nv + 1) + 2 * nv) * 128 + (size_t)(nv + 2) * 256;
 }
 size_t solve_tma_smem_bytes(int nv) { return 128 + solve_stage_bytes(nv) + 2 * 256 + sizeof(uint64_t); }
 
@@ -1239,14 +1252,14 @@ __device__ __forceinline__ void solve_issue(const SolveSm& s, const SolveMaps& M
                                             int stage0, int want_div) {
   const uint32_t fi = (nv + 1) * 128, fc = nv * 128, di = (nv + 1) * 256;
   const uint64_t ps = pol_stream(), pk = pol_keep();
-  mbar_arrive_expect_tx(bar, 2 * fi + 2 * fc + 3 * di + 256);
+  mbar_arrive_expect_tx(bar, 4 * fi + 2 * fc + di + 256);
   tma_load_2d(s.w, &M.w, c0, 0, bar, pk);
   tma_load_2d(s.sw, &M.sw, c0, 0, bar, ps);
   tma_load_2d(s.cc, &M.cc, c0, 0, bar, pk);
   tma_load_2d(s.ca, &M.ca, c0, 0, bar, pk);
-  tma_load_2d(s.q, &M.q, c0, 0, bar, ps);
+  tma_load_2d(s.lo, &M.lo, c0, 0, bar, ps);
+  tma_load_2d(s.up, &M.up, c0, 0, bar, ps);
   tma_load_2d(s.inv, &M.inv, c0, 0, bar, ps);
-  tma_load_2d(s.cf, &M.cf, c0, 0, bar, ps);
   tma_load_2d(s.junc, &M.junction, c0, 0, bar, ps);
   tma_prefetch_2d(&M.thi, c0, 0, ps);
   tma_prefetch_2d(&M.cb, c0, 0, pk);
@@ -1258,30 +1271,42 @@ __device__ __forceinline__ void solve_issue(const SolveSm& s, const SolveMaps& M
   }
 }
 
+// rows m = 1 + warp, + kSolveWarps, ... of one group prepared for the sweeps,
+// each row's results over its own inputs (the rows above read only cc and ca)
+__device__ __forceinline__ void solve_rows(const SolveSm& s, const VR<float>& U, float rdt, float g, float delta,
+                                           int nv, int tx, int warp) {
+  const int N = nv - 1, p = N / 2 > 0 ? N / 2 : 1;
+  for (int m = 1 + warp; m <= N; m += kSolveWarps) {
+    const int o = m * 32 + tx;
+    const float wlo = ld(U.wlo + m), whi = ld(U.whi + m);
+    const float r = delta * s.w[o] + rdt * s.sw[o] - rdt * ld(U.inv_dzc + m) * (s.cc[o] - s.cc[o - 32])
+                    - rdt * g * (wlo * s.ca[o - 32] + whi * s.ca[o]);
+    const float2 inv = s.inv[o];
+    const float lo = s.lo[o], up = s.up[o];
+    const float2 q = df_mul_f(m <= p ? lo : up, inv), cf = df_mul_f(m <= p ? up : lo, inv);
+    s.inv[o] = df_product(r, inv);
+    s.lo[o] = q.x;
+    s.up[o] = q.y;
+    s.w[o] = cf.x;
+    s.sw[o] = cf.y;
+  }
+}
+
 // the two sweeps of one group, sweep 0 (rows 1..p, downwards) or 1 (rows
 // nv-1..p+1, upwards) by one warp each, then the junction rows and the back
 // substitution; the solved W* over s.w. The elimination runs in
-// double-float on the float32 pipes (the factors arrive as double-float
-// pairs). The two warps meet at named barrier 1.
-__device__ __forceinline__ void solve_sweeps(const SolveSm& s, float2* sx, const VR<float>& U, float rdt, float g,
-                                             float delta, int nv, int tx, int sweep) {
+// double-float on the float32 pipes. The two warps meet at named barrier 1.
+__device__ __forceinline__ void solve_sweeps(const SolveSm& s, float2* sx, int nv, int tx, int sweep) {
   const int N = nv - 1, p = N / 2 > 0 ? N / 2 : 1;
-  auto rhs = [&](int m) {
-    const int o = m * 32 + tx;
-    const float wlo = ld(U.wlo + m), whi = ld(U.whi + m);
-    return delta * s.w[o] + rdt * s.sw[o] - rdt * ld(U.inv_dzc + m) * (s.cc[o] - s.cc[o - 32])
-           - rdt * g * (wlo * s.ca[o - 32] + whi * s.ca[o]);
-  };
-  const float2* q = reinterpret_cast<const float2*>(s.q);
-  const float2* cf = reinterpret_cast<const float2*>(s.cf);
-  float2* sdp = reinterpret_cast<float2*>(s.inv);      // d' / f' over the pivot reciprocals
+  float2* sdp = s.inv;                                 // rh / piv, then d' / f'
   float* s_wf = s.w;
   if (sweep == 0) {
     float2 d1 = make_float2(0.f, 0.f);
 #pragma unroll 4
     for (int m = 1; m <= p; ++m) {
       const int o = m * 32 + tx;
-      d1 = df_sweep(rhs(m), sdp[o], q[o], d1);
+      const float2 r = sdp[o];
+      d1 = df_fms(r.x, r.y, s.q(o), d1);
       sdp[o] = d1;
     }
   } else {
@@ -1289,7 +1314,8 @@ __device__ __forceinline__ void solve_sweeps(const SolveSm& s, float2* sx, const
 #pragma unroll 4
     for (int m = N; m > p; --m) {
       const int o = m * 32 + tx;
-      f1 = df_sweep(rhs(m), sdp[o], q[o], f1);
+      const float2 r = sdp[o];
+      f1 = df_fms(r.x, r.y, s.q(o), f1);
       sdp[o] = f1;
     }
   }
@@ -1299,8 +1325,8 @@ __device__ __forceinline__ void solve_sweeps(const SolveSm& s, float2* sx, const
     float2 xp, xq = make_float2(0.f, 0.f);
     if (p < N) {
       const float2 dp_ = sdp[op], fq = sdp[op + 32];
-      xp = df_mul(df_fms(dp_.x, dp_.y, cf[op], fq), reinterpret_cast<const float2*>(s.junc)[tx]);
-      xq = df_fms(fq.x, fq.y, cf[op + 32], xp);
+      xp = df_mul(df_fms(dp_.x, dp_.y, s.cf(op), fq), s.junc[tx]);
+      xq = df_fms(fq.x, fq.y, s.cf(op + 32), xp);
     } else {
       xp = sdp[op];
     }
@@ -1312,18 +1338,20 @@ __device__ __forceinline__ void solve_sweeps(const SolveSm& s, float2* sx, const
     float2 x = sx[tx];
     s_wf[p * 32 + tx] = df_to_float(x);
     for (int m = p - 1; m >= 1; --m) {
-      const float2 d = sdp[m * 32 + tx];
-      x = df_fms(d.x, d.y, cf[m * 32 + tx], x);
-      s_wf[m * 32 + tx] = df_to_float(x);
+      const int o = m * 32 + tx;
+      const float2 d = sdp[o];
+      x = df_fms(d.x, d.y, s.cf(o), x);
+      s_wf[o] = df_to_float(x);
     }
     s_wf[tx] = 0.f;
   } else {
     float2 x = sx[32 + tx];
     if (p < N) s_wf[(p + 1) * 32 + tx] = df_to_float(x);
     for (int m = p + 2; m <= N; ++m) {
-      const float2 d = sdp[m * 32 + tx];
-      x = df_fms(d.x, d.y, cf[m * 32 + tx], x);
-      s_wf[m * 32 + tx] = df_to_float(x);
+      const int o = m * 32 + tx;
+      const float2 d = sdp[o];
+      x = df_fms(d.x, d.y, s.cf(o), x);
+      s_wf[o] = df_to_float(x);
     }
     s_wf[nv * 32 + tx] = 0.f;
   }
@@ -1401,7 +1429,9 @@ __device__ __forceinline__ void d_ss_solve_tma(const Geo<float>& G, const VR<flo
     return;
   }
   const float rdt = (float)dtau, g = ph.g_f;
-  if (warp < 2) solve_sweeps(s, sx, U, rdt, g, ph.delta_f, nv, tx, warp);
+  solve_rows(s, U, rdt, g, ph.delta_f, nv, tx, warp);
+  __syncthreads();
+  if (warp < 2) solve_sweeps(s, sx, nv, tx, warp);
   __syncthreads();
   if (c >= G.ncol) return;
   // the eight warps share the levels of the final updates
@@ -1412,7 +1442,7 @@ __device__ __forceinline__ void d_ss_solve_tma(const Geo<float>& G, const VR<flo
               XoL, last, c, tx, k, pk);
 }
 
-__global__ void __launch_bounds__(32 * kSolveWarps)
+__global__ void __launch_bounds__(32 * kSolveWarps, 6)
     k_ss_solve_tma(Geo<float> G, VR<float> U, Phys ph, const __grid_constant__ SolveMaps M, int stage0,
                    Xf<float> Xs, Slow<float> SL, Pert<float> P, Work<float> T, double dtau, int want_div,
                    Xf<float> Xo, Xf<float> XsL, Xf<float> XoL, int last, int* err) {
@@ -1531,7 +1561,7 @@ __global__ void __launch_bounds__(32 * kSolveWarps)
   d_ss_solve<R>(a.G, a.U, a.ph, Xs, a.SL, a.P, a.T, a.F, a.dts[s], want_div, s == 2 ? a.Xt : a.Xst,
                 s == 0 ? a.XtL : Xf<R>{}, s == 2 ? a.XtL : Xf<R>{}, j + 1 == a.nsub[s], e.y, 0);
 }
-__global__ void __launch_bounds__(32 * kSolveWarps)
+__global__ void __launch_bounds__(32 * kSolveWarps, 6)
     ke_ss_solve_tma(const Member<float>* __restrict__ M, const int2* __restrict__ map, int s, int j) {
   const int2 e = map[blockIdx.x];
   const Member<float>& a = M[e.x];
@@ -1858,9 +1888,9 @@ int Impl<float>::build_solve_maps() {
   make(&map->th_s, Xst.th, nv, false);
   make(&map->dsc, SL.dsc, nv, false);
   make(&map->dhm, T.dhm, nv, false);
-  make(&map->q, F.q, nv + 1, true);
+  make(&map->lo, F.q, nv + 1, false);
+  make(&map->up, F.cf, nv + 1, false);
   make(&map->inv, F.inv, nv + 1, true);
-  make(&map->cf, F.cf, nv + 1, true);
   make(&map->junction, F.junction, 1, true);
   if (!ok) return 0;
   if (!raise_smem_limit(k_ss_solve_tma, (int)smem) || !raise_smem_limit(ke_ss_solve_tma, (int)smem)) return -3;
