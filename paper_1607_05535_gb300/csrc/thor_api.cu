@@ -587,6 +587,7 @@ void Impl<R>::shape() {
   const bool f32 = sizeof(R) == sizeof(float), few = cells < 200000;
   kchunk = !f32 || few ? 1 : cells < 800000 ? 2 : 3;
   level_split = cells >= (f32 ? 800000 : 200000);
+  dense = f32 && cells >= 800000;
   carveout = f32 && few ? 50 : -1;
   overlap = f32 && few && (long long)((G.ncol + block - 1) / block) * G.nv <= 152;
 }

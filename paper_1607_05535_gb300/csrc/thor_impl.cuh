@@ -122,6 +122,7 @@ struct ImplBase {
   int solve_tma = 1;                   // TMA-staged column solve where available
   int level_split = 1;                 // small-step stencils in two level halves on two streams
   int overlap = 0;                     // start kernels while the one before drains (pdl_wait)
+  int dense = 0;                       // slow terms in few registers (k_slow)
   int carveout = -1;                   // LaunchHint::carveout of every kernel of the step
   int rk_stages = 3;                   // RK3 stages a large step runs (THOR_TUNE_RK_STAGES; tests)
   int* dev_err = nullptr;              // device flag: 1 = a bounded device wait timed out

@@ -155,7 +155,9 @@ __device__ __forceinline__ void d_lap1(const Geo<R>& G, const VR<R>& U, const Xf
 // here the traditional Coriolis, 2 Omega sin(lat) r x M on the horizontal
 // momentum only, and the horizontal velocity and w advected without the
 // metric terms the approximation drops)
-template <typename R, bool SH = false, bool HO = false>
+// DENSE: one level at a time in few registers, for more threads in flight
+// (k_slow chooses)
+template <typename R, bool SH = false, bool HO = false, bool DENSE = false>
 __device__ __forceinline__ void d_slow(const Geo<R>& G, const VR<R>& U, const Phys& ph, const Xf<R>& X, const Work<R>& T, const Slow<R>& SL, int hyper,
                                             R* d0, int kchunk, int bx, int by, int kend) {
   int c = bx * blockDim.x + threadIdx.x;
@@ -175,7 +177,7 @@ __device__ __forceinline__ void d_slow(const Geo<R>& G, const VR<R>& U, const Ph
   const R two_om = pc<R>(ph.two_omega, ph.two_omega_f), Rd = pc<R>(ph.Rd, ph.Rd_f);
   const int S = pdl_wait(G.colp);
   int k0 = by * kchunk, k1 = min(kend, k0 + kchunk);
-  constexpr int kUnroll = sizeof(R) == sizeof(float) ? 2 : 1;   // float64: registers
+  constexpr int kUnroll = sizeof(R) == sizeof(float) && !DENSE ? 2 : 1;   // float64: registers
 #pragma unroll kUnroll
   for (int k = k0; k < k1; ++k) {
     const int o = k * S, i = o + c;
@@ -1139,11 +1141,15 @@ template <typename R, bool HO>
 __global__ void k_lap1(Geo<R> G, VR<R> U, Xf<R> X, Work<R> T, R Kd, int kchunk, int klo, int kend) {
   d_lap1<R, HO>(G, U, X, T, Kd, kchunk, blockIdx.x, blockIdx.y + klo, kend);
 }
-template <typename R, bool SH, bool HO>
-__global__ void __launch_bounds__(kMaxBlock, sizeof(R) == sizeof(float) ? 3 : 2)
+// DENSE (float): 64 registers and four blocks of 256 threads an SM, one level
+// at a time, against 80 and three, two levels at a time. Many cells have threads
+// to fill the SMs with (g6 x 32: 64.4 -> 59.3 us, large step 1.202 -> 1.185 ms);
+// with fewer the longer threads cost (g5 x 37 22.7 -> 24.6 us, 406 -> 415 us).
+template <typename R, bool SH, bool HO, bool DENSE>
+__global__ void __launch_bounds__(kMaxBlock, sizeof(R) == sizeof(float) ? (DENSE ? 4 : 3) : 2)
     k_slow(Geo<R> G, VR<R> U, Phys ph, Xf<R> X, Work<R> T, Slow<R> SL, int hyper, R* d0, int kchunk, int klo,
            int kend) {
-  d_slow<R, SH, HO>(G, U, ph, X, T, SL, hyper, d0, kchunk, blockIdx.x, blockIdx.y + klo, kend);
+  d_slow<R, SH, HO, DENSE>(G, U, ph, X, T, SL, hyper, d0, kchunk, blockIdx.x, blockIdx.y + klo, kend);
 }
 template <typename R, bool HO>
 __global__ void k_slow_w(Geo<R> G, VR<R> U, Phys ph, Xf<R> Xt, Xf<R> X, Work<R> T, Slow<R> SL, Pert<R> P, int hyper,
@@ -1612,6 +1618,19 @@ int col_kernel_setup(int nv) {
 template int col_kernel_setup<double>(int);
 template int col_kernel_setup<float>(int);
 
+// the slow-term kernel of a state
+template <typename R, bool DENSE>
+auto slow_kernel(bool shallow, bool ho) {
+  return shallow ? (ho ? k_slow<R, true, true, DENSE> : k_slow<R, true, false, DENSE>)
+                 : (ho ? k_slow<R, false, true, DENSE> : k_slow<R, false, false, DENSE>);
+}
+template <typename R>
+auto slow_kernel(bool shallow, bool ho, bool dense) {
+  if constexpr (sizeof(R) == sizeof(float))
+    if (dense) return slow_kernel<R, true>(shallow, ho);
+  return slow_kernel<R, false>(shallow, ho);
+}
+
 template <typename R>
 int Impl<R>::large_step(double dt, int n_small) {
   const int kc = kchunk, bs = block;
@@ -1696,8 +1715,7 @@ int Impl<R>::large_step(double dt, int n_small) {
       ++launches;
     }
     mark(THOR_K_SLOW, true);
-    auto slow = shallow ? (ho ? k_slow<R, true, true> : k_slow<R, true, false>)
-                        : (ho ? k_slow<R, false, true> : k_slow<R, false, false>);
+    auto slow = slow_kernel<R>(shallow, ho, dense);
     chk(launch_hint(hint(pdl), slow, g2, bs, 0, stream, G, U, ph, Xs, T, SL, hyper,
                  s == 0 && divdamp ? T.dd0 : (R*)nullptr, kc, 0, G.nv));
     mark(THOR_K_SLOW, false);
@@ -1809,8 +1827,7 @@ int Impl<R>::anelastic_step(double dt) {
     if (hyper && launch_k(ho ? k_lap1<R, true> : k_lap1<R, false>, g2i, bs, 0, stream, G, U, Xs, T, Kd, kc, 0,
                           G.nv + 1))
       return -3;
-    auto slow = shallow ? (ho ? k_slow<R, true, true> : k_slow<R, true, false>)
-                        : (ho ? k_slow<R, false, true> : k_slow<R, false, false>);
+    auto slow = slow_kernel<R>(shallow, ho, dense);
     if (launch_k(slow, g2, bs, 0, stream, G, U, ph, Xs, T, SL, hyper, (R*)nullptr, kc, 0, G.nv) ||
         launch_k(ho ? k_slow_w<R, true> : k_slow_w<R, false>, g2i, bs, 0, stream, G, U, ph, Xt, Xs, T, SL, P,
                  hyper, 0, kc))
