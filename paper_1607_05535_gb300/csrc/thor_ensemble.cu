@@ -19,6 +19,9 @@
 
 namespace thor {
 
+template <typename R>
+int column_width();   // thor_step.cu: columns of a block of the column kernels
+
 struct EnsBase {
   virtual ~EnsBase() {}
   virtual int step(int n_large, const int* n_small, const double* dt) = 0;
@@ -90,7 +93,7 @@ struct EnsImpl : EnsBase {
       const Impl<R>* I = mem[i];
       tab[q] = I->member(dt[i], n_small[i]);
       nb[q] = (I->G.ncol + block - 1) / block;
-      nbc[q] = (I->G.ncol + 31) / 32;
+      nbc[q] = (I->G.ncol + column_width<R>() - 1) / column_width<R>();
       for (int b = 0; b < nb[q]; ++b) map.push_back(make_int2(q, b));
       for (int b = 0; b < nbc[q]; ++b) mapc.push_back(make_int2(q, b));
       p.any_hyper |= I->hyper;

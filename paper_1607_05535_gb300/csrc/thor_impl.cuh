@@ -385,7 +385,7 @@ template <typename R>
 struct EnsPlan {
   const Member<R>* M = nullptr;
   const int2* map = nullptr;        // stencil blocks: (member, local block)
-  const int2* mapc = nullptr;       // 32-column blocks of the column kernels
+  const int2* mapc = nullptr;       // blocks of the column kernels (column_width)
   int nv = 0, kchunk = 2, block = kBlock;
   int nblk = 0, nblkc = 0;          // all members
   int maxsub[3] = {0, 0, 0};

@@ -610,15 +610,33 @@ __device__ __forceinline__ void fac_store(const Fac<R>& F, int i, double inv, do
 // the stage. The factorisation is the matrix half of a two-sided Thomas
 // algorithm, in float64 for float64 states and in double-float (df_rcp,
 // df_mul_f: pivot reciprocals to about 2^-46) for float-storage states:
-// warp 0 eliminates rows 1..p downwards
-// (c'_m = up_m / (di_m - lo_m c'_m-1)), warp 1 rows nv-1..p+1 upwards
-// (e'_m = lo_m / (di_m - up_m e'_m+1)); the two warps run on different SM
-// sub-partitions. Stored per row: the pivot reciprocal, c' or e', and q = lo
+// one half of the lanes eliminates rows 1..p downwards
+// (c'_m = up_m / (di_m - lo_m c'_m-1)), the other rows nv-1..p+1 upwards
+// (e'_m = lo_m / (di_m - up_m e'_m+1)). Stored per row: the pivot reciprocal, c' or e', and q = lo
 // or up times the pivot reciprocal; per column: 1 / (1 - c'_p e'_p+1) for the
 // junction rows p, p+1.
+//
+// the matrix row m of column c in the storage type
 template <typename R>
-__device__ __forceinline__ void d_ss_factor(const Geo<R>& G, const VR<R>& U, const Phys& ph, const Slow<R>& SL, const Fac<R>& F,
-                                            double dtau, int bx, int by) {
+__device__ __forceinline__ void matrix_row(const VR<R>& U, const Slow<R>& SL, R g, R dt2, R delta, int nv, int S, int c,
+                                           int m, R& lo, R& di, R& up) {
+  const int i = m * S + c, N = nv - 1;
+  const R pi_lo = ld(SL.pi + (i - S)), pi_hi = ld(SL.pi + i);
+  const R wlo = ld(U.wlo + m), whi = ld(U.whi + m), dtz = dt2 * ld(U.inv_dzc + m);
+  const R ql = ld(U.sq_lo + (m - 1)), qh = ld(U.sq_hi + (m - 1));   // cell m-1
+  const R pl = ld(U.sq_lo + m), ph_ = ld(U.sq_hi + m);              // cell m
+  const R th_m = ld(SL.thi + i);
+  R lower = 0, upper = 0;
+  if (m > 1) lower = (-dtz * pi_lo * ld(SL.thi + (i - S)) + dt2 * g * wlo) * ql;
+  if (m < N) upper = (-dtz * pi_hi * ld(SL.thi + (i + S)) - dt2 * g * whi) * ph_;
+  lo = lower;
+  up = upper;
+  di = delta + dtz * th_m * (pi_hi * pl + pi_lo * qh) - dt2 * g * (wlo * qh - whi * pl);
+}
+
+// float storage: 32 columns a block, one warp for each of the two sweeps
+__device__ __forceinline__ void d_ss_factor(const Geo<float>& G, const VR<float>& U, const Phys& ph,
+                                            const Slow<float>& SL, const Fac<float>& F, double dtau, int bx) {
   pdl_next();
   const int nv = G.nv, S = pdl_wait(G.colp), N = nv - 1;
   const int tx = threadIdx.x & 31, half = threadIdx.x >> 5;
@@ -626,92 +644,103 @@ __device__ __forceinline__ void d_ss_factor(const Geo<R>& G, const VR<R>& U, con
   const bool valid = c < G.ncol;
   const int cs = valid ? c : 0;          // padding lanes compute on column 0 and store nothing
   const int p = N / 2 > 0 ? N / 2 : 1;
-  const R g = pc<R>(ph.g, ph.g_f), dt2 = (R)(dtau * dtau), delta = pc<R>(ph.delta, ph.delta_f);
-  __shared__ double sj[2][32];
-  // the matrix row m in the storage type
-  auto coef_r = [&](int m, R& lo, R& di, R& up) {
-    const int i = m * S + cs;
-    const R pi_lo = ld(SL.pi + (i - S)), pi_hi = ld(SL.pi + i);
-    const R wlo = ld(U.wlo + m), whi = ld(U.whi + m), dtz = dt2 * ld(U.inv_dzc + m);
-    const R ql = ld(U.sq_lo + (m - 1)), qh = ld(U.sq_hi + (m - 1));   // cell m-1
-    const R pl = ld(U.sq_lo + m), ph_ = ld(U.sq_hi + m);              // cell m
-    const R th_m = ld(SL.thi + i);
-    R lower = 0, upper = 0;
-    if (m > 1) lower = (-dtz * pi_lo * ld(SL.thi + (i - S)) + dt2 * g * wlo) * ql;
-    if (m < N) upper = (-dtz * pi_hi * ld(SL.thi + (i + S)) - dt2 * g * whi) * ph_;
-    lo = lower;
-    up = upper;
-    di = delta + dtz * th_m * (pi_hi * pl + pi_lo * qh) - dt2 * g * (wlo * qh - whi * pl);
+  const float g = ph.g_f, dt2 = (float)(dtau * dtau), delta = ph.delta_f;
+  auto coef_r = [&](int m, float& lo, float& di, float& up) {
+    matrix_row<float>(U, SL, g, dt2, delta, nv, S, cs, m, lo, di, up);
   };
-  if constexpr (sizeof(R) == sizeof(float)) {
-    // float storage: the factorisation in double-float on the float32 pipes
-    // (the float coefficients are exact pairs), stored as pairs
-    __shared__ float2 sj2[2][32];
-    float2* Finv = reinterpret_cast<float2*>(F.inv);
-    float* Flo = reinterpret_cast<float*>(F.q);
-    float* Fup = reinterpret_cast<float*>(F.cf);
-    float2 last = make_float2(0.f, 0.f);
-    if (half == 0) {
-      for (int m = 1; m <= p; ++m) {
-        R lo, di, up;
-        coef_r(m, lo, di, up);
-        const float2 inv = df_rcp(df_fms(di, 0.f, make_float2(lo, 0.f), last));
-        last = df_mul_f(up, inv);
-        if (valid) {
-          Finv[m * S + c] = inv;
-          Flo[m * S + c] = lo;
-          Fup[m * S + c] = up;
-        }
-      }
-    } else {
-      for (int m = N; m > p; --m) {
-        R lo, di, up;
-        coef_r(m, lo, di, up);
-        const float2 inv = df_rcp(df_fms(di, 0.f, make_float2(up, 0.f), last));
-        last = df_mul_f(lo, inv);
-        if (valid) {
-          Finv[m * S + c] = inv;
-          Flo[m * S + c] = lo;
-          Fup[m * S + c] = up;
-        }
-      }
-    }
-    sj2[half][tx] = last;    // c'_p (warp 0) and e'_p+1 (warp 1)
-    __syncthreads();
-    if (half == 0 && valid)
-      reinterpret_cast<float2*>(F.junction)[c] =
-          p < N ? df_rcp(df_fms(1.f, 0.f, sj2[0][tx], sj2[1][tx])) : make_float2(1.f, 0.f);
-    return;
-  }
-  auto coef = [&](int m, double& lo, double& di, double& up) {
-    R l, d, u;
-    coef_r(m, l, d, u);
-    lo = l;
-    di = d;
-    up = u;
-  };
-  auto inv_of = [](double den) { return 1.0 / den; };
-  double last = 0.0;
+  // float storage: the factorisation in double-float on the float32 pipes
+  // (the float coefficients are exact pairs), stored as pairs
+  __shared__ float2 sj2[2][32];
+  float2* Finv = reinterpret_cast<float2*>(F.inv);
+  float* Flo = reinterpret_cast<float*>(F.q);
+  float* Fup = reinterpret_cast<float*>(F.cf);
+  float2 last = make_float2(0.f, 0.f);
   if (half == 0) {
     for (int m = 1; m <= p; ++m) {
-      double lo, di, up;
-      coef(m, lo, di, up);
-      const double inv = inv_of(di - lo * last);
-      last = up * inv;
-      if (valid) fac_store(F, m * S + c, inv, last, lo * inv);
+      float lo, di, up;
+      coef_r(m, lo, di, up);
+      const float2 inv = df_rcp(df_fms(di, 0.f, make_float2(lo, 0.f), last));
+      last = df_mul_f(up, inv);
+      if (valid) {
+        Finv[m * S + c] = inv;
+        Flo[m * S + c] = lo;
+        Fup[m * S + c] = up;
+      }
     }
   } else {
     for (int m = N; m > p; --m) {
-      double lo, di, up;
-      coef(m, lo, di, up);
-      const double inv = inv_of(di - up * last);
-      last = lo * inv;
-      if (valid) fac_store(F, m * S + c, inv, last, up * inv);
+      float lo, di, up;
+      coef_r(m, lo, di, up);
+      const float2 inv = df_rcp(df_fms(di, 0.f, make_float2(up, 0.f), last));
+      last = df_mul_f(lo, inv);
+      if (valid) {
+        Finv[m * S + c] = inv;
+        Flo[m * S + c] = lo;
+        Fup[m * S + c] = up;
+      }
     }
   }
-  sj[half][tx] = last;     // c'_p (warp 0) and e'_p+1 (warp 1)
+  sj2[half][tx] = last;    // c'_p (warp 0) and e'_p+1 (warp 1)
   __syncthreads();
-  if (half == 0 && valid) F.junction[c] = p < N ? 1.0 / (1.0 - sj[0][tx] * sj[1][tx]) : 1.0;
+  if (half == 0 && valid)
+    reinterpret_cast<float2*>(F.junction)[c] =
+        p < N ? df_rcp(df_fms(1.f, 0.f, sj2[0][tx], sj2[1][tx])) : make_float2(1.f, 0.f);
+}
+
+// Float64 columns: a block is kCols64 = 16 columns x 16 threads each. The
+// matrix rows (and the solve's right-hand sides and final updates) are shared
+// by all sixteen; lanes 0-15 of one warp then run the downward sweep and lanes
+// 16-31 the upward one, in the same instructions, each over shared memory.
+// A float64 warp instruction holds its sub-partition's pipe for 80 cycles, so
+// what a small grid needs is every SM: 16 columns a block give a g4 grid 161
+// blocks for 152 SMs where 32 gave it 81. The large step against 32 columns a
+// block: g4 x 20 430 -> 411 us, g5 x 32 1577 -> 1507 us, g6 x 32 6085 -> 6132
+// us (there every SM is busy either way). With 64 / 128 / 256 threads a block
+// in both kernels: g4 508 / 438 / 418, g5 1651 / 1554 / 1508, g6 6108 / 6113 /
+// 6142 us.
+constexpr int kCols64 = 16, kThreads64 = 256;
+struct Lane64 {
+  int tx, slot, c, cs;
+  bool valid, sweeps;
+  __device__ Lane64(int bx, int ncol) {
+    tx = threadIdx.x & (kCols64 - 1);
+    slot = threadIdx.x / kCols64;
+    c = bx * kCols64 + tx;
+    valid = c < ncol;
+    cs = valid ? c : 0;                  // padding lanes compute on column 0 and store nothing
+    // the sweeping warp differs from block to block, so that the blocks of an
+    // SM do not all sweep on one sub-partition
+    sweeps = (threadIdx.x >> 5) == ((unsigned)bx * 2654435761u >> 29);
+  }
+};
+
+__device__ __forceinline__ void d_ss_factor(const Geo<double>& G, const VR<double>& U, const Phys& ph,
+                                            const Slow<double>& SL, const Fac<double>& F, double dtau, int bx) {
+  extern __shared__ double sm[];
+  pdl_next();
+  const int nv = G.nv, S = pdl_wait(G.colp), N = nv - 1;
+  const Lane64 L(bx, G.ncol);
+  const int p = N / 2 > 0 ? N / 2 : 1, rows = (nv + 1) * kCols64;
+  double *slo = sm, *sdi = sm + rows, *sup = sm + 2 * rows;      // [nv + 1][kCols64] each
+  for (int m = 1 + L.slot; m <= N; m += kThreads64 / kCols64) {
+    const int o = m * kCols64 + L.tx;
+    matrix_row<double>(U, SL, ph.g, dtau * dtau, ph.delta, nv, S, L.cs, m, slo[o], sdi[o], sup[o]);
+  }
+  __syncthreads();
+  if (!L.sweeps) return;
+  const bool down = (L.slot & 1) == 0;
+  const int len = down ? p : N - p;
+  const double *off = down ? slo : sup, *oth = down ? sup : slo;
+  double last = 0.0;
+  for (int t = 0; t < len; ++t) {
+    const int m = down ? 1 + t : N - t, o = m * kCols64 + L.tx;
+    const double a = off[o], inv = 1.0 / (sdi[o] - a * last);
+    last = oth[o] * inv;
+    if (L.valid) fac_store(F, m * S + L.c, inv, last, a * inv);
+  }
+  __syncwarp();
+  const double e = __shfl_down_sync(0xffffffffu, last, kCols64);     // e'_p+1 beside c'_p
+  if (down && L.valid) F.junction[L.c] = p < N ? 1.0 / (1.0 - last * e) : 1.0;
 }
 
 // End of an RK stage for one cell of the column step: Phi^(s+1) = Phi^(s) +
@@ -741,16 +770,6 @@ __device__ __forceinline__ void stage_end_cell(const Xf<R>& Xs, const Xf<R>& Xo,
 
 constexpr int kSolveWarps = 8;     // warps of a column solve's block
 
-// the solved W* of row o of the direct solve's shared array: a float64
-// value, or for float storage the float in the first word of the row
-template <typename R>
-__device__ __forceinline__ R solved_w(const double* sdp, int o) {
-  if constexpr (sizeof(R) == sizeof(double))
-    return sdp[o];
-  else
-    return reinterpret_cast<const float2*>(sdp)[o].x;
-}
-
 // HE-VI column step, part 3 (every small step). The right-hand side
 //   rh_m = W*_m + dtau S_W,m - dtau/dzc_m (c_m - c_m-1) - dtau g (w- a_m-1 + w+ a_m)
 // goes through the stored factors (d'_m = rh_m / piv_m - q_m d'_m-1
@@ -760,18 +779,37 @@ __device__ __forceinline__ R solved_w(const double* sdp, int o) {
 // x_p+1 = f'_p+1 - e'_p+1 x_p, then back substitution outwards), in float64
 // for float64 states and in double-float for float-storage states; then
 // rho* and Th* follow from Eqs. dens2 and pt2 and p* from the nonlinear Eq.
-// theta_to_p. One block = 32 columns x 8 warps: two of them sweep, all share
-// the levels of the final updates and, in float64, of the right-hand sides
-// (rh_m / piv_m into shared memory before the sweeps, which then hold one
-// multiply-add per row). A float64 warp instruction holds its sub-partition's
-// pipe for 80 cycles, so work on two warps alone takes four times as long on
-// a grid with fewer blocks than SMs: g4 x 20 float64 31.8 -> 17.3 us;
-// at g6 x 32, where the pipe is busy either way, 105.8 -> 105.5 us.
+// theta_to_p.
+//
+// The cell's update with the solved W* at its interfaces (wl, wh):
 template <typename R>
-__device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, const Phys& ph, const Xf<R>& Xs, const Slow<R>& SL,
-                                            const Pert<R>& P, const Work<R>& T, const Fac<R>& F, double dtau,
-                                            int want_div, const Xf<R>& Xo, const Xf<R>& XsL, const Xf<R>& XoL, int last, int bx,
-                                            int by) {
+__device__ __forceinline__ void update_cell(const VR<R>& U, const Phys& ph, const Xf<R>& Xs, const Slow<R>& SL,
+                                            const Pert<R>& P, const Work<R>& T, R rdt, R wl, R wh, int want_div,
+                                            const Xf<R>& Xo, const Xf<R>& XsL, const Xf<R>& XoL, int last, int k, int i,
+                                            int S, int nv) {
+  const R thl = k > 0 ? ld(SL.thi + i) : R(0);
+  const R thh = k + 1 < nv ? ld(SL.thi + (i + S)) : R(0);
+  const R el = ld(U.sq_lo + k), eh = ld(U.sq_hi + k);
+  R th_new = ld(T.cb + i) - rdt * (eh * thh * wh - el * thl * wl);
+  const R rho_new = ld(T.ca + i) - rdt * (eh * wh - el * wl);
+  P.rho[i] = rho_new;
+  P.th[i] = th_new;
+  // p* = EOS(Th^(s) + Th*) - p^(s)
+  P.p[i] = p_pert(ph, ld(SL.pi + i), ld(U.thb + k) + ld(Xs.th + i), th_new);
+  if (k >= 1) P.w[i] = wl;
+  // 3-D divergence of the new total momentum, for the next small step's
+  // divergence damping: D^(s) + div_h M* (from k_ss_flux) + div_v W*
+  if (want_div) T.dd[i] = ld(SL.dsc + i) + ld(T.dhm + i) + (eh * wh - el * wl);
+  if (last) stage_end_cell(Xs, Xo, XsL, XoL, P, rho_new, th_new, wl, k, i, S, nv);
+}
+
+// One block = 32 columns x 8 warps, float storage where the staged solve does
+// not apply: two warps sweep, all share the levels of the final updates.
+__device__ __forceinline__ void d_ss_solve(const Geo<float>& G, const VR<float>& U, const Phys& ph, const Xf<float>& Xs,
+                                            const Slow<float>& SL, const Pert<float>& P, const Work<float>& T,
+                                            const Fac<float>& F, double dtau, int want_div, const Xf<float>& Xo,
+                                            const Xf<float>& XsL, const Xf<float>& XoL, int last, int bx) {
+  using R = float;
   extern __shared__ double sm[];
   pdl_next();
   const int nv = G.nv, S = pdl_wait(G.colp), N = nv - 1;
@@ -791,130 +829,68 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
     return delta * ld(P.w + i) + rdt * ld(SL.sw + i) - rdt * ld(U.inv_dzc + m) * (ld(T.cc + i) - ld(T.cc + (i - S)))
            - rdt * g * (wlo * ld(T.ca + (i - S)) + whi * ld(T.ca + i));
   };
-  if constexpr (sizeof(R) == sizeof(float)) {
-    // float storage: the elimination in double-float, the same operations
-    // in the same order as the staged solve (solve_sweeps); W* (float) over
-    // the first word of each row of sdp
-    const float* Flo = reinterpret_cast<const float*>(F.q);
-    const float2* Finv = reinterpret_cast<const float2*>(F.inv);
-    const float* Fup = reinterpret_cast<const float*>(F.cf);
-    float2* dp2 = reinterpret_cast<float2*>(sdp);
-    float2* sx2 = reinterpret_cast<float2*>(sx);
-    float2* cf2 = reinterpret_cast<float2*>(scf);
-    if (warp == 0) {
-      float2 d1 = make_float2(0.f, 0.f);
+  // float storage: the elimination in double-float, the same operations
+  // in the same order as the staged solve (solve_sweeps); W* (float) over
+  // the first word of each row of sdp
+  const float* Flo = reinterpret_cast<const float*>(F.q);
+  const float2* Finv = reinterpret_cast<const float2*>(F.inv);
+  const float* Fup = reinterpret_cast<const float*>(F.cf);
+  float2* dp2 = reinterpret_cast<float2*>(sdp);
+  float2* sx2 = reinterpret_cast<float2*>(sx);
+  float2* cf2 = reinterpret_cast<float2*>(scf);
+  if (warp == 0) {
+    float2 d1 = make_float2(0.f, 0.f);
 #pragma unroll 4
-      for (int m = 1; m <= p; ++m) {
-        const int i = m * S + cs;
-        const float2 inv = Finv[i];
-        cf2[m * 32 + tx] = df_mul_f(Fup[i], inv);
-        d1 = df_sweep(rhs_r(m), inv, df_mul_f(Flo[i], inv), d1);
-        dp2[m * 32 + tx] = d1;
-      }
-    } else if (warp == 1) {
-      float2 f1 = make_float2(0.f, 0.f);
-#pragma unroll 4
-      for (int m = N; m > p; --m) {
-        const int i = m * S + cs;
-        const float2 inv = Finv[i];
-        cf2[m * 32 + tx] = df_mul_f(Flo[i], inv);
-        f1 = df_sweep(rhs_r(m), inv, df_mul_f(Fup[i], inv), f1);
-        dp2[m * 32 + tx] = f1;
-      }
-    }
-    __syncthreads();
-    if (warp == 0) {
-      float2 xp, xq = make_float2(0.f, 0.f);
-      if (p < N) {
-        const float2 dp_ = dp2[p * 32 + tx], fq = dp2[(p + 1) * 32 + tx];
-        xp = df_mul(df_fms(dp_.x, dp_.y, cf2[p * 32 + tx], fq), reinterpret_cast<const float2*>(F.junction)[cs]);
-        xq = df_fms(fq.x, fq.y, cf2[(p + 1) * 32 + tx], xp);
-      } else {
-        xp = dp2[p * 32 + tx];
-      }
-      sx2[tx] = xp;
-      sx2[32 + tx] = xq;
-    }
-    __syncthreads();
-    if (warp == 0) {
-      float2 x = sx2[tx];
-      dp2[p * 32 + tx] = make_float2(df_to_float(x), 0.f);
-      for (int m = p - 1; m >= 1; --m) {
-        const float2 d = dp2[m * 32 + tx];
-        x = df_fms(d.x, d.y, cf2[m * 32 + tx], x);
-        dp2[m * 32 + tx] = make_float2(df_to_float(x), 0.f);
-      }
-      dp2[tx] = make_float2(0.f, 0.f);             // bottom interface
-    } else if (warp == 1) {
-      float2 x = sx2[32 + tx];
-      if (p < N) dp2[(p + 1) * 32 + tx] = make_float2(df_to_float(x), 0.f);
-      for (int m = p + 2; m <= N; ++m) {
-        const float2 d = dp2[m * 32 + tx];
-        x = df_fms(d.x, d.y, cf2[m * 32 + tx], x);
-        dp2[m * 32 + tx] = make_float2(df_to_float(x), 0.f);
-      }
-      dp2[nv * 32 + tx] = make_float2(0.f, 0.f);    // top interface
-    }
-  } else {
-    // float64 storage: the elimination in float64
-    for (int m = 1 + warp; m <= N; m += kSolveWarps) {
+    for (int m = 1; m <= p; ++m) {
       const int i = m * S + cs;
-      sdp[m * 32 + tx] = rhs_r(m) * ld(F.inv + i);
-      scf[m * 32 + tx] = ld(F.q + i);
+      const float2 inv = Finv[i];
+      cf2[m * 32 + tx] = df_mul_f(Fup[i], inv);
+      d1 = df_sweep(rhs_r(m), inv, df_mul_f(Flo[i], inv), d1);
+      dp2[m * 32 + tx] = d1;
     }
-    __syncthreads();
-    if (warp == 0) {
-      double d1 = 0.0;
+  } else if (warp == 1) {
+    float2 f1 = make_float2(0.f, 0.f);
 #pragma unroll 4
-      for (int m = 1; m <= p; ++m) {
-        const int o = m * 32 + tx;
-        d1 = fma(-scf[o], d1, sdp[o]);
-        sdp[o] = d1;
-        scf[o] = ld(F.cf + (m * S + cs));
-      }
-    } else if (warp == 1) {
-      double f1 = 0.0;
-#pragma unroll 4
-      for (int m = N; m > p; --m) {
-        const int o = m * 32 + tx;
-        f1 = fma(-scf[o], f1, sdp[o]);
-        sdp[o] = f1;
-        scf[o] = ld(F.cf + (m * S + cs));
-      }
+    for (int m = N; m > p; --m) {
+      const int i = m * S + cs;
+      const float2 inv = Finv[i];
+      cf2[m * 32 + tx] = df_mul_f(Flo[i], inv);
+      f1 = df_sweep(rhs_r(m), inv, df_mul_f(Fup[i], inv), f1);
+      dp2[m * 32 + tx] = f1;
     }
-    __syncthreads();
-    if (warp == 0) {
-      double xp, xq = 0.0;
-      if (p < N) {
-        const double cp_ = scf[p * 32 + tx], eq = scf[(p + 1) * 32 + tx];
-        const double dp_ = sdp[p * 32 + tx], fq = sdp[(p + 1) * 32 + tx];
-        xp = (dp_ - cp_ * fq) * ld(F.junction + cs);
-        xq = fq - eq * xp;
-      } else {
-        xp = sdp[p * 32 + tx];
-      }
-      sx[tx] = xp;
-      sx[32 + tx] = xq;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    float2 xp, xq = make_float2(0.f, 0.f);
+    if (p < N) {
+      const float2 dp_ = dp2[p * 32 + tx], fq = dp2[(p + 1) * 32 + tx];
+      xp = df_mul(df_fms(dp_.x, dp_.y, cf2[p * 32 + tx], fq), reinterpret_cast<const float2*>(F.junction)[cs]);
+      xq = df_fms(fq.x, fq.y, cf2[(p + 1) * 32 + tx], xp);
+    } else {
+      xp = dp2[p * 32 + tx];
     }
-    __syncthreads();
-    // back substitution, each warp over its own rows
-    if (warp == 0) {
-      double x = sx[tx];
-      sdp[p * 32 + tx] = x;
-      for (int m = p - 1; m >= 1; --m) {
-        x = sdp[m * 32 + tx] - scf[m * 32 + tx] * x;
-        sdp[m * 32 + tx] = x;
-      }
-      sdp[tx] = 0.0;                 // bottom interface
-    } else if (warp == 1) {
-      double x = sx[32 + tx];
-      if (p < N) sdp[(p + 1) * 32 + tx] = x;
-      for (int m = p + 2; m <= N; ++m) {
-        x = sdp[m * 32 + tx] - scf[m * 32 + tx] * x;
-        sdp[m * 32 + tx] = x;
-      }
-      sdp[nv * 32 + tx] = 0.0;       // top interface
+    sx2[tx] = xp;
+    sx2[32 + tx] = xq;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    float2 x = sx2[tx];
+    dp2[p * 32 + tx] = make_float2(df_to_float(x), 0.f);
+    for (int m = p - 1; m >= 1; --m) {
+      const float2 d = dp2[m * 32 + tx];
+      x = df_fms(d.x, d.y, cf2[m * 32 + tx], x);
+      dp2[m * 32 + tx] = make_float2(df_to_float(x), 0.f);
     }
+    dp2[tx] = make_float2(0.f, 0.f);             // bottom interface
+  } else if (warp == 1) {
+    float2 x = sx2[32 + tx];
+    if (p < N) dp2[(p + 1) * 32 + tx] = make_float2(df_to_float(x), 0.f);
+    for (int m = p + 2; m <= N; ++m) {
+      const float2 d = dp2[m * 32 + tx];
+      x = df_fms(d.x, d.y, cf2[m * 32 + tx], x);
+      dp2[m * 32 + tx] = make_float2(df_to_float(x), 0.f);
+    }
+    dp2[nv * 32 + tx] = make_float2(0.f, 0.f);    // top interface
   }
   __syncthreads();
   // Eqs. dens2, pt2, theta_to_p with the new W*; the warps share the levels
@@ -922,23 +898,74 @@ __device__ __forceinline__ void d_ss_solve(const Geo<R>& G, const VR<R>& U, cons
 #pragma unroll 4
     for (int k = warp; k < nv; k += kSolveWarps) {
       const int i = k * S + c;
-      const R wl = solved_w<R>(sdp, k * 32 + tx), wh = solved_w<R>(sdp, (k + 1) * 32 + tx);
-      const R thl = k > 0 ? ld(SL.thi + i) : R(0);
-      const R thh = k + 1 < nv ? ld(SL.thi + (i + S)) : R(0);
-      const R el = ld(U.sq_lo + k), eh = ld(U.sq_hi + k);
-      R th_new = ld(T.cb + i) - rdt * (eh * thh * wh - el * thl * wl);
-      const R rho_new = ld(T.ca + i) - rdt * (eh * wh - el * wl);
-      P.rho[i] = rho_new;
-      P.th[i] = th_new;
-      // p* = EOS(Th^(s) + Th*) - p^(s)
-      P.p[i] = p_pert(ph, ld(SL.pi + i), ld(U.thb + k) + ld(Xs.th + i), th_new);
-      if (k >= 1) P.w[i] = wl;
-      // 3-D divergence of the new total momentum, for the next small step's
-      // divergence damping: D^(s) + div_h M* (from k_ss_flux) + div_v W*
-      if (want_div) T.dd[i] = ld(SL.dsc + i) + ld(T.dhm + i) + (eh * wh - el * wl);
-      if (last) stage_end_cell(Xs, Xo, XsL, XoL, P, rho_new, th_new, wl, k, i, S, nv);
+      const R wl = dp2[k * 32 + tx].x, wh = dp2[(k + 1) * 32 + tx].x;
+      update_cell<R>(U, ph, Xs, SL, P, T, rdt, wl, wh, want_div, Xo, XsL, XoL, last, k, i, S, nv);
     }
   }
+}
+
+// Float64 storage (the layout of threads as in the float64 factorisation):
+// rh_m / piv_m by all threads, the sweeps and the back substitution one
+// multiply-add per row in one warp, the updates by all threads.
+__device__ __forceinline__ void d_ss_solve(const Geo<double>& G, const VR<double>& U, const Phys& ph,
+                                            const Xf<double>& Xs, const Slow<double>& SL, const Pert<double>& P,
+                                            const Work<double>& T, const Fac<double>& F, double dtau, int want_div,
+                                            const Xf<double>& Xo, const Xf<double>& XsL, const Xf<double>& XoL, int last,
+                                            int bx) {
+  extern __shared__ double sm[];
+  pdl_next();
+  const int nv = G.nv, S = pdl_wait(G.colp), N = nv - 1;
+  const Lane64 L(pdl_wait(bx), G.ncol);
+  const int p = N / 2 > 0 ? N / 2 : 1, rows = (nv + 1) * kCols64;
+  double *sd = sm, *sq = sm + rows;      // [nv + 1][kCols64]: rh / piv, then d' / f', then W; q, then c' / e'
+  const double g = ph.g, delta = ph.delta;
+  for (int m = 1 + L.slot; m <= N; m += kThreads64 / kCols64) {
+    const int i = m * S + L.cs, o = m * kCols64 + L.tx;
+    const double rh = delta * ld(P.w + i) + dtau * ld(SL.sw + i)
+                      - dtau * ld(U.inv_dzc + m) * (ld(T.cc + i) - ld(T.cc + (i - S)))
+                      - dtau * g * (ld(U.wlo + m) * ld(T.ca + (i - S)) + ld(U.whi + m) * ld(T.ca + i));
+    sd[o] = rh * ld(F.inv + i);
+    sq[o] = ld(F.q + i);
+  }
+  __syncthreads();
+  if (L.sweeps) {
+    const bool down = (L.slot & 1) == 0;
+    const int len = down ? p : N - p;
+    double d = 0.0;
+#pragma unroll 4
+    for (int t = 0; t < len; ++t) {
+      const int m = down ? 1 + t : N - t, o = m * kCols64 + L.tx;
+      d = fma(-sq[o], d, sd[o]);
+      sd[o] = d;
+      sq[o] = ld(F.cf + (m * S + L.cs));
+    }
+    __syncwarp();
+    const int op = p * kCols64 + L.tx, oq = op + kCols64;
+    double x = sd[op];
+    if (p < N) {
+      // x_p, x_p+1
+      x = (x - sq[op] * sd[oq]) * ld(F.junction + L.cs);
+      if (!down) x = sd[oq] - sq[oq] * x;
+    }
+    __syncwarp();
+    if (down)
+      sd[op] = x;
+    else if (p < N)
+      sd[oq] = x;
+    const int back = down ? p - 1 : N - p - 1;
+    for (int t = 0; t < back; ++t) {
+      const int m = down ? p - 1 - t : p + 2 + t, o = m * kCols64 + L.tx;
+      x = sd[o] - sq[o] * x;
+      sd[o] = x;
+    }
+    sd[(down ? 0 : nv) * kCols64 + L.tx] = 0.0;       // bottom and top interfaces
+  }
+  __syncthreads();
+  if (!L.valid) return;
+#pragma unroll 2
+  for (int k = L.slot; k < nv; k += kThreads64 / kCols64)
+    update_cell<double>(U, ph, Xs, SL, P, T, dtau, sd[k * kCols64 + L.tx], sd[(k + 1) * kCols64 + L.tx], want_div, Xo,
+                        XsL, XoL, last, k, k * S + L.c, S, nv);
 }
 
 // ---------------------------------------------------------------- physics
@@ -1184,15 +1211,22 @@ __global__ void k_ss_flux(Geo<R> G, VR<R> U, Slow<R> SL, Pert<R> P, Work<R> T, R
   G.nv = khi;
   d_ss_flux<R>(G, U, SL, P, T, dtau, kchunk, blockIdx.x, blockIdx.y + klo);
 }
+// columns and threads of a column kernel's block
 template <typename R>
-__global__ void __launch_bounds__(64) k_ss_factor(Geo<R> G, VR<R> U, Phys ph, Slow<R> SL, Fac<R> F, double dtau) {
-  d_ss_factor<R>(G, U, ph, SL, F, dtau, blockIdx.x, 0);
+constexpr int col_width() { return sizeof(R) == sizeof(double) ? kCols64 : 32; }
+template <typename R>
+constexpr int factor_threads() { return sizeof(R) == sizeof(double) ? kThreads64 : 64; }
+constexpr int solve_threads() { return 32 * kSolveWarps; }
+static_assert(solve_threads() == kThreads64, "one block size for both solves");
+template <typename R>
+__global__ void __launch_bounds__(factor_threads<R>()) k_ss_factor(Geo<R> G, VR<R> U, Phys ph, Slow<R> SL, Fac<R> F, double dtau) {
+  d_ss_factor(G, U, ph, SL, F, dtau, blockIdx.x);
 }
 template <typename R>
 __global__ void __launch_bounds__(32 * kSolveWarps) k_ss_solve(Geo<R> G, VR<R> U, Phys ph, Xf<R> Xs, Slow<R> SL, Pert<R> P,
                                                  Work<R> T, Fac<R> F, double dtau, int want_div, Xf<R> Xo,
                                                  Xf<R> XsL, Xf<R> XoL, int last) {
-  d_ss_solve<R>(G, U, ph, Xs, SL, P, T, F, dtau, want_div, Xo, XsL, XoL, last, blockIdx.x, 0);
+  d_ss_solve(G, U, ph, Xs, SL, P, T, F, dtau, want_div, Xo, XsL, XoL, last, blockIdx.x);
 }
 template <typename R>
 __global__ void k_surface_p(Geo<R> G, VR<R> U, Phys ph, Xf<R> X, Work<R> T) {
@@ -1527,10 +1561,10 @@ __global__ void ke_slow_w(const Member<R>* __restrict__ M, const int2* __restric
     d_slow_w<R>(a.G, a.U, a.ph, a.Xt, Xs, a.T, a.SL, a.P, a.hyper, 1, kchunk, e.y, member_chunk(), XtL);
 }
 template <typename R>
-__global__ void __launch_bounds__(64)
+__global__ void __launch_bounds__(factor_threads<R>())
     ke_ss_factor(const Member<R>* __restrict__ M, const int2* __restrict__ map, int s) {
   THOR_MEMBER();
-  d_ss_factor<R>(a.G, a.U, a.ph, a.SL, a.F, a.dts[s], e.y, 0);
+  d_ss_factor(a.G, a.U, a.ph, a.SL, a.F, a.dts[s], e.y);
 }
 template <typename R>
 // the small-step stencils over levels [kchunk * klo, khi) (as k_ss_*)
@@ -1564,8 +1598,8 @@ __global__ void __launch_bounds__(32 * kSolveWarps)
     ke_ss_solve(const Member<R>* __restrict__ M, const int2* __restrict__ map, int s, int j) {
   THOR_MEMBER();
   const int want_div = a.divdamp && j + 1 < a.nsub[s];
-  d_ss_solve<R>(a.G, a.U, a.ph, Xs, a.SL, a.P, a.T, a.F, a.dts[s], want_div, s == 2 ? a.Xt : a.Xst,
-                s == 0 ? a.XtL : Xf<R>{}, s == 2 ? a.XtL : Xf<R>{}, j + 1 == a.nsub[s], e.y, 0);
+  d_ss_solve(a.G, a.U, a.ph, Xs, a.SL, a.P, a.T, a.F, a.dts[s], want_div, s == 2 ? a.Xt : a.Xst,
+             s == 0 ? a.XtL : Xf<R>{}, s == 2 ? a.XtL : Xf<R>{}, j + 1 == a.nsub[s], e.y);
 }
 __global__ void __launch_bounds__(32 * kSolveWarps, 6)
     ke_ss_solve_tma(const Member<float>* __restrict__ M, const int2* __restrict__ map, int s, int j) {
@@ -1597,7 +1631,18 @@ void Impl<R>::launch_2d(int nplanes, int kchunk, dim3& grid) const {
   grid = dim3((G.ncol + block - 1) / block, (nplanes + kchunk - 1) / kchunk);
 }
 
-size_t solve_smem_bytes(int nv) { return (size_t)(2 * (nv + 1) + 2) * 32 * sizeof(double); }
+template <typename R>
+size_t solve_smem_bytes(int nv) {
+  return (size_t)(2 * (nv + 1) + (sizeof(R) == sizeof(float) ? 2 : 0)) * col_width<R>() * sizeof(double);
+}
+template <typename R>
+size_t factor_smem_bytes(int nv) {
+  return sizeof(R) == sizeof(double) ? (size_t)3 * (nv + 1) * kCols64 * sizeof(double) : 0;
+}
+template <typename R>
+int column_width() { return col_width<R>(); }
+template int column_width<double>();
+template int column_width<float>();
 
 // Raise a kernel's dynamic shared-memory limit to at least bytes, never
 // lower it: states with different level counts share the kernels, and a
@@ -1612,8 +1657,11 @@ static bool raise_smem_limit(K* kernel, int bytes) {
 
 template <typename R>
 int col_kernel_setup(int nv) {
-  const int bytes = (int)solve_smem_bytes(nv);
-  return raise_smem_limit(k_ss_solve<R>, bytes) && raise_smem_limit(ke_ss_solve<R>, bytes) ? 0 : -3;
+  const int bytes = (int)solve_smem_bytes<R>(nv), fbytes = (int)factor_smem_bytes<R>(nv);
+  return raise_smem_limit(k_ss_solve<R>, bytes) && raise_smem_limit(ke_ss_solve<R>, bytes) &&
+                 raise_smem_limit(k_ss_factor<R>, fbytes) && raise_smem_limit(ke_ss_factor<R>, fbytes)
+             ? 0
+             : -3;
 }
 template int col_kernel_setup<double>(int);
 template int col_kernel_setup<float>(int);
@@ -1638,8 +1686,8 @@ int Impl<R>::large_step(double dt, int n_small) {
   launch_2d(G.nv, kc, g2);
   launch_2d(G.nv + 1, kc, g2i);
   dim3 g1((G.ncol + bs - 1) / bs);
-  dim3 gsolve((G.ncol + 31) / 32);
-  const size_t solve_smem = solve_smem_bytes(G.nv);
+  dim3 gsolve((G.ncol + col_width<R>() - 1) / col_width<R>());
+  const size_t solve_smem = solve_smem_bytes<R>(G.nv);
   const bool staged = solve_tma && smaps != nullptr;
   // level halves of the small-step stencils (THOR_TUNE_LEVEL_SPLIT): levels
   // [0, kc * hc) on the state's stream, [kc * hc, nv) on side2
@@ -1732,7 +1780,7 @@ int Impl<R>::large_step(double dt, int n_small) {
                  kc));
     mark(THOR_K_SLOW_W, false);
     mark(THOR_K_SS_FACTOR, true);
-    chk(launch_hint(hint(pdl), k_ss_factor<R>, gsolve, 64, 0, aux, G, U, ph, SL, F, dts[s]));
+    chk(launch_hint(hint(pdl), k_ss_factor<R>, gsolve, factor_threads<R>(), factor_smem_bytes<R>(G.nv), aux, G, U, ph, SL, F, dts[s]));
     mark(THOR_K_SS_FACTOR, false);
     if (fork) {
       chk(cudaEventRecord(ev_join, side));
@@ -1776,7 +1824,7 @@ int Impl<R>::large_step(double dt, int n_small) {
       if (staged)
         chk(launch_solve_tma(hint(pdl && j > 0), gsolve, s, Xo, XsL, XoL, dts[s], want_div, last));
       else
-        chk(launch_hint(hint(pdl && j > 0), k_ss_solve<R>, gsolve, 32 * kSolveWarps, solve_smem, stream, G, U, ph, Xs, SL, P, T, F, dts[s],
+        chk(launch_hint(hint(pdl && j > 0), k_ss_solve<R>, gsolve, solve_threads(), solve_smem, stream, G, U, ph, Xs, SL, P, T, F, dts[s],
                      want_div, Xo, XsL, XoL, last));
       mark(THOR_K_SS_SOLVE, false);
       ++launches;
@@ -1936,7 +1984,7 @@ int ensemble_large_step(const EnsPlan<R>& E, cudaStream_t stream, long long* lau
   const int rows = max(1, kMaxBlock / bs);
   const dim3 tb(bs, rows);
   auto up = [&](int chunks) { return (chunks + rows - 1) / rows; };
-  const size_t solve_smem = solve_smem_bytes(E.nv);
+  const size_t solve_smem = solve_smem_bytes<R>(E.nv);
   const Member<R>* M = E.M;
   long long n = 0;
   for (int s = 0; s < 3; ++s) {
@@ -1948,7 +1996,7 @@ int ensemble_large_step(const EnsPlan<R>& E, cudaStream_t stream, long long* lau
     }
     ke_slow<R><<<g2, tb, 0, stream>>>(M, E.map, s, kc);
     ke_slow_w<R><<<g2i, tb, 0, stream>>>(M, E.map, s, kc);
-    ke_ss_factor<R><<<E.nblkc, 64, 0, stream>>>(M, E.mapc, s);
+    ke_ss_factor<R><<<E.nblkc, factor_threads<R>(), factor_smem_bytes<R>(E.nv), stream>>>(M, E.mapc, s);
     n += 4;
     for (int j = 0; j < E.maxsub[s]; ++j) {
       const int nb = E.active[s][j], nbc = E.activec[s][j];
