@@ -347,7 +347,7 @@ int thor_zonal_read_w(thor_state* state, int nlat, double* out, size_t n, long l
  * kernels, a multiple of 32 in [32, 256] (default 128).
  * THOR_TUNE_SOLVE_TMA: 1 (default) runs the column solve of a THOR_MIXED
  * state with its planes staged into shared memory by TMA bulk-tensor copies
- * (where the staging fits, nv <= 80); 0 runs the direct-load solve. Same
+ * (where the staging fits); 0 runs the direct-load solve. Same
  * arithmetic, same results. A staged copy that has not landed after 2 s ends
  * the kernel with a device error flag; thor_diag (and thor_step with
  * THOR_TUNE_CHECK_FINITE) then return THOR_ETIMEOUT.

@@ -168,9 +168,6 @@ template <> __device__ __forceinline__ float rpow<float>(float x, float y) { ret
 template <typename R> __device__ __forceinline__ R rsinpi(R x);      // sin(pi x)
 template <> __device__ __forceinline__ double rsinpi<double>(double x) { return sinpi(x); }
 template <> __device__ __forceinline__ float rsinpi<float>(float x) { return sinpif(x); }
-template <typename R> __device__ __forceinline__ R rsqrt_(R x);
-template <> __device__ __forceinline__ double rsqrt_<double>(double x) { return sqrt(x); }
-template <> __device__ __forceinline__ float rsqrt_<float>(float x) { return sqrtf(x); }
 
 // a b + c with one rounding, written out where a sum of two products could
 // otherwise be contracted either way (kernels that must agree bit for bit
@@ -428,32 +425,6 @@ __device__ __forceinline__ void st4(double* base, size_t cell, double x, double 
   reinterpret_cast<double2*>(base)[2 * cell] = make_double2(x, y);
   reinterpret_cast<double2*>(base)[2 * cell + 1] = make_double2(z, w);
 }
-// the same with an L2 policy (l2_policy)
-__device__ __forceinline__ Q4<float> ld4h(const float* base, size_t cell, uint64_t pol) {
-  Q4<float> v;
-  asm("ld.global.nc.L2::cache_hint.v4.f32 {%0, %1, %2, %3}, [%4], %5;"
-      : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w)
-      : "l"(base + 4 * cell), "l"(pol));
-  return v;
-}
-__device__ __forceinline__ Q4<double> ld4h(const double* base, size_t cell, uint64_t pol) {
-  Q4<double> v;
-  asm("ld.global.nc.L2::cache_hint.v2.f64 {%0, %1}, [%2], %3;" : "=d"(v.x), "=d"(v.y) : "l"(base + 4 * cell), "l"(pol));
-  asm("ld.global.nc.L2::cache_hint.v2.f64 {%0, %1}, [%2], %3;" : "=d"(v.z), "=d"(v.w) : "l"(base + 4 * cell + 2), "l"(pol));
-  return v;
-}
-__device__ __forceinline__ void st4h(float* base, size_t cell, float x, float y, float z, float w, uint64_t pol) {
-  asm volatile("st.global.L2::cache_hint.v4.f32 [%0], {%1, %2, %3, %4}, %5;" ::"l"(base + 4 * cell), "f"(x), "f"(y),
-               "f"(z), "f"(w), "l"(pol)
-               : "memory");
-}
-__device__ __forceinline__ void st4h(double* base, size_t cell, double x, double y, double z, double w, uint64_t pol) {
-  asm volatile("st.global.L2::cache_hint.v2.f64 [%0], {%1, %2}, %3;" ::"l"(base + 4 * cell), "d"(x), "d"(y), "l"(pol)
-               : "memory");
-  asm volatile("st.global.L2::cache_hint.v2.f64 [%0], {%1, %2}, %3;" ::"l"(base + 4 * cell + 2), "d"(z), "d"(w),
-               "l"(pol)
-               : "memory");
-}
 
 // two values of one cell stored together ([level][colp][2] planes)
 template <typename R>
@@ -553,22 +524,6 @@ __device__ __forceinline__ W7<R> load_w7(const R* w, int colp, int c) {
   for (int j = 0; j < 7; ++j) o.v[j] = ld(w + j * colp + c);
   return o;
 }
-// The 3-vector weights of the seven stencil points of column c, stored
-// packed as [7][colp][4] (x, y, z and a fourth value: for the gradient table
-// the Laplacian weight of the same point, else 0), so that one 16-byte load
-// (two in float64) brings a point's weights.
-template <typename R>
-__device__ __forceinline__ W7x3<R> load_w7x3(const R* w, int colp, int c) {
-  W7x3<R> o;
-#pragma unroll
-  for (int j = 0; j < 7; ++j) {
-    const Q4<R> q = ld4(w, (size_t)j * colp + c);
-    o.x[j] = q.x;
-    o.y[j] = q.y;
-    o.z[j] = q.z;
-  }
-  return o;
-}
 // two-component weights of the seven points, packed [7][colp][2]
 template <typename R>
 struct W7x2 {
@@ -585,7 +540,9 @@ __device__ __forceinline__ W7x2<R> load_w7x2(const R* w, int colp, int c) {
   }
   return o;
 }
-// the gradient weights and, from the same loads, the Laplacian weights
+// The 3-vector weights of the seven stencil points of column c and, from the
+// same loads (one of 16 bytes a point, two in float64), the Laplacian
+// weights: packed [7][colp][4].
 template <typename R>
 __device__ __forceinline__ void load_w7x3_lap(const R* w, int colp, int c, W7x3<R>& g, W7<R>& l) {
 #pragma unroll
@@ -665,49 +622,6 @@ __device__ __forceinline__ Q4<R> apply7x4(const W7<R>& w, const Nbr7& nb, const 
   }
   return s;
 }
-// sum_j w_j . F(n_j) with F given by three planes
-template <typename R>
-__device__ __forceinline__ R div7(const W7x3<R>& w, const Nbr7& nb, const R* fx, const R* fy, const R* fz) {
-  R s = 0;
-#pragma unroll
-  for (int j = 0; j < 7; ++j) {
-    int q = nb.n[j];
-    s += w.x[j] * ld(fx + q) + w.y[j] * ld(fy + q) + w.z[j] * ld(fz + q);
-  }
-  return s;
-}
-// sum_j w_j . (a(n_j) F(n_j))
-template <typename R>
-__device__ __forceinline__ R div7_scaled(const W7x3<R>& w, const Nbr7& nb, const R* a, const R* fx,
-                                         const R* fy, const R* fz) {
-  R s = 0;
-#pragma unroll
-  for (int j = 0; j < 7; ++j) {
-    int q = nb.n[j];
-    R aq = ld(a + q);
-    s += aq * (w.x[j] * ld(fx + q) + w.y[j] * ld(fy + q) + w.z[j] * ld(fz + q));
-  }
-  return s;
-}
-template <typename R>
-__device__ __forceinline__ void grad7(const W7x3<R>& w, const Nbr7& nb, const R* s, R& gx, R& gy, R& gz) {
-  gx = gy = gz = 0;
-#pragma unroll
-  for (int j = 0; j < 7; ++j) {
-    R v = ld(s + nb.n[j]);
-    gx += w.x[j] * v;
-    gy += w.y[j] * v;
-    gz += w.z[j] * v;
-  }
-}
-template <typename R>
-__device__ __forceinline__ void project(R rx, R ry, R rz, R& x, R& y, R& z) {
-  R d = x * rx + y * ry + z * rz;
-  x -= d * rx;
-  y -= d * ry;
-  z -= d * rz;
-}
-
 }  // namespace thor
 
 // ------------------------------------------------------------ TMA staging

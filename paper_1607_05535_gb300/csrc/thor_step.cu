@@ -819,7 +819,7 @@ __device__ __forceinline__ void d_ss_solve(const Geo<float>& G, const VR<float>&
   const int cs = valid ? c : 0;          // padding lanes read column 0 and store nothing
   double* sdp = sm;                      // [nv + 1][32] d' / f', then W
   double* sx = sdp + (nv + 1) * 32;      // [2][32] junction values
-  double* scf = sx + 64;                 // [nv + 1][32] c' / e', fetched during the sweeps (float64: q before)
+  double* scf = sx + 64;                 // [nv + 1][32] c' / e', fetched during the sweeps
   const int p = N / 2 > 0 ? N / 2 : 1;
   const R rdt = (R)dtau, g = pc<R>(ph.g, ph.g_f), delta = pc<R>(ph.delta, ph.delta_f);
 
