@@ -1255,6 +1255,7 @@ void thor_state_destroy(thor_state* s) {
   thor::closure_release(s);
   if (s->impl) cudaStreamSynchronize(s->impl->stream);
   thor::zonal_release(s->zonal);
+  thor::coarse_release(s->coarse);
   delete s;
 }
 

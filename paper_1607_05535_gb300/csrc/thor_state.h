@@ -33,17 +33,27 @@ struct ZonalAcc {
   long long samples = 0;
 };
 
+// scratch of thor_coarse_grain, kept with the coarse state: the fine columns
+// of every coarse column, listed on the device from the caller's map
+struct CoarseWork {
+  void* buf = nullptr;
+  size_t bytes = 0;
+  cudaEvent_t ready = nullptr;        // the fine state's stream, where it is another than the coarse one's
+};
+
 struct thor_state {
   thor_grid* grid = nullptr;
   int precision = THOR_FP64;
   int check_finite = 0;
   ClosureBinding closure;
   ZonalAcc zonal;
+  CoarseWork coarse;
   std::unique_ptr<thor::ImplBase> impl;
 };
 
 namespace thor {
 int closure_large_step(thor_state* s, int n_small, double dt);   // thor_mlp.cu
 void closure_release(thor_state* s);
+void coarse_release(CoarseWork& w);
 void zonal_release(ZonalAcc& z);                                  // thor_climate.cu
 }
