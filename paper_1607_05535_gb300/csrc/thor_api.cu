@@ -189,7 +189,7 @@ void carve(Carver& cv, Impl<R>& I, int ncol, int nv) {
   const double** vi[] = {&I.V.ri, &I.V.dzc, &I.V.wlo, &I.V.whi, &I.V.Rb, &I.V.ri2, &I.V.inv_dzc};
   for (const double** p : vi) *p = cv.take<double>(nv + 1);
   for (const R** p : vr_slots(I.U)) *p = cv.take<R>(nv + 1);
-  I.U.pw = sizeof(R) == sizeof(double) ? cv.take<double>(kPowRows * kPowCols) : nullptr;
+  I.U.pw = cv.take<double>(kPowRows * kPowCols);
   I.U.iw = cv.take<R>(4 * (size_t)(nv + 1));
   I.U.cw = cv.take<R>(4 * (size_t)nv);
   I.U.ij0 = cv.take<int>(nv + 1);

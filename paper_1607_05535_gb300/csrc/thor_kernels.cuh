@@ -63,7 +63,7 @@ struct VR {
   const R *inv_thb, *inv_ri2;      // 1 / thb, 1 / ri2
   // Held-Suarez: ln(pb / p0) and (pb / p0)^kappa, p0 = 1e5 Pa; hot Jupiter: T_vert of the level
   const R *lnp0, *pk0, *hjT;
-  const double* pw;                // pow1p's table (float64 states; null: not valid for this gamma)
+  const double* pw;                // pow1p's table (null: not valid for this gamma)
   // Lagrange interpolation of order k > 1 in the explicit terms (Sec. 2.1):
   // interface m (1..nv-1) from centres ij0[m] + j with weights iw[j][m];
   // centre c from interfaces cj0[c] + j with weights cw[j][c]; j < 4, the

@@ -25,7 +25,9 @@ struct ClosureBinding {
 // zonal band means accumulated over time (thor_zonal_accumulate)
 struct ZonalAcc {
   int nlat = 0;                       // bands (0: nothing allocated)
-  int* band = nullptr;                // [colp] band of every column
+  int* order = nullptr;               // [ncol] columns in the order of their bands
+  void* chunk = nullptr;              // [nchunk] band, first and last + 1 of order
+  int nchunk = 0;
   double* basis = nullptr;            // [6][colp] east and north unit vectors
   double* tmp = nullptr;              // [nv][nlat][9] sums of one state
   double* acc = nullptr;              // [nv][nlat][9] accumulated band means and covariances
