@@ -61,15 +61,17 @@ def step_method_words(n_small):
 # method words: W*, rho*, Theta and p* read and written (8; rho*, Theta, p*
 # read through the flux kernel's a, b, c), S_W, S_rho, S_Theta (3; the
 # latter two through a and b), theta at the interfaces, Pi, W^(s) and p (4).
-# It moves 21: W*, S_W, a, b, c, theta_iface, p', Th^(s), D^(s), div_h M*
-# read (10), the three float64 factor planes (6 words) and rho*, Theta, p*,
-# W*, D written (5). The interface kernel also sets the stage's
-# perturbations, and the last small step of a stage also ends it; the
-# counts below are those of the other small steps.
+# It moves 19: W*, S_W, a, b, c, theta_iface, Pi, Th^(s), D^(s), div_h M*
+# read (10), the factors (off-diagonals 2, pivot reciprocals as pairs 2) and
+# rho*, Theta, p*, W*, D written (5). Horizontal momentum and its slow term
+# count two words in the small step's kernels, which hold them in each
+# column's tangent basis (the rule above counts three). The last small step
+# of a stage also ends it; the counts below are those of the other small
+# steps.
 KERNEL_WORDS = {        # name: (method words, moved words)
-    "derived": (7, 16), "lap1": (6, 14), "slow": (13, 25), "slow_w": (4, 9),
-    "ss_lapd": (1, 4), "ss_mom": (10, 13), "ss_flux": (10, 14), "ss_solve": (15, 21),
-    "ss_factor": (2, 8), "physics": (9, 9), "stage_init": (7, 20),
+    "derived": (7, 18), "lap1": (6, 14), "slow": (13, 22), "slow_w": (4, 9),
+    "ss_lapd": (1, 3), "ss_mom": (7, 7), "ss_flux": (9, 13), "ss_solve": (15, 19),
+    "ss_factor": (2, 6), "physics": (9, 9), "stage_init": (7, 19),
 }
 
 
