@@ -526,7 +526,8 @@ struct GemmOut {
   int ldcb;
   __nv_bfloat16* CbT;              // bfloat16 transposed, rows of ldt
   int ldt;
-  float* colsum;                   // [32-row tile][N] column sums
+  float* colsum;                   // [row tile][N] column sums
+  int rows128;                     // its tiles: 32 rows (rows_colsum), or 128 (tile_colsum)
 };
 struct GemmJob {
   CUtensorMap a, b;
@@ -539,20 +540,46 @@ struct GemmPair {
   int blocks0;                     // CTAs of the first job
 };
 
-// column sums over a warp's 32 lanes of 16 values per lane: halves of the
-// columns are exchanged, so that 16 shuffles instead of 80 serve; lane l then
-// holds the sum of column bitwise (l >> 1)
-__device__ __forceinline__ float lane_colsum(const float* x, int lane) {
-  float a[8], b[4], c[2], d;
-  const bool h4 = lane & 16, h3 = lane & 8, h2 = lane & 4, h1 = lane & 2;
+// column sums over a warp's 32 rows (lane = row, 16 columns each) in rising
+// row order, as the other column sums of the library run, through the warp's
+// own piece of shared memory; lanes 0..15 return the sums. A tree of
+// exchanged halves costs 16 shuffles instead (the training step 70.4 us, this
+// way 70.9), but rounds differently, and Adam's first steps, which divide a
+// gradient by its own size, carry such a difference into the weights.
+__device__ __forceinline__ float rows_colsum(const float* x, float* sm, int lane) {
+  __syncwarp();
 #pragma unroll
-  for (int j = 0; j < 8; ++j) a[j] = (h4 ? x[8 + j] : x[j]) + __shfl_xor_sync(0xffffffffu, h4 ? x[j] : x[8 + j], 16);
+  for (int j = 0; j < 16; ++j) sm[lane * 17 + j] = x[j];
+  __syncwarp();
+  float a = 0.0f;
+  if (lane < 16) {
 #pragma unroll
-  for (int j = 0; j < 4; ++j) b[j] = (h3 ? a[4 + j] : a[j]) + __shfl_xor_sync(0xffffffffu, h3 ? a[j] : a[4 + j], 8);
+    for (int r = 0; r < 32; ++r) a += sm[r * 17 + lane];
+  }
+  return a;
+}
+
+// column sums over the tile's 128 rows in the order of k_colsum_part (eight
+// strided row lanes, then the lanes); every thread of the block comes here,
+// thread t < 16 returns column t's sum
+__device__ __forceinline__ float tile_colsum(const float* x, float* sm, int tid) {
+  float* lanes = sm + 128 * 17;
+  __syncthreads();
 #pragma unroll
-  for (int j = 0; j < 2; ++j) c[j] = (h2 ? b[2 + j] : b[j]) + __shfl_xor_sync(0xffffffffu, h2 ? b[j] : b[2 + j], 4);
-  d = (h1 ? c[1] : c[0]) + __shfl_xor_sync(0xffffffffu, h1 ? c[0] : c[1], 2);
-  return d + __shfl_xor_sync(0xffffffffu, d, 1);
+  for (int j = 0; j < 16; ++j) sm[tid * 17 + j] = x[j];
+  __syncthreads();
+  const int col = tid & 15, ty = tid >> 4;
+  float a = 0.0f;
+#pragma unroll
+  for (int r = 0; r < 16; ++r) a += sm[(ty + 8 * r) * 17 + col];
+  lanes[ty * 17 + col] = a;
+  __syncthreads();
+  a = 0.0f;
+  if (tid < 16) {
+#pragma unroll
+    for (int j = 0; j < 8; ++j) a += lanes[j * 17 + tid];
+  }
+  return a;
 }
 
 __global__ void __launch_bounds__(128, 1) k_gemm_tma(const __grid_constant__ GemmPair P, int* err) {
@@ -718,10 +745,15 @@ __global__ void __launch_bounds__(128, 1) k_gemm_tma(const __grid_constant__ Gem
 #pragma unroll
           for (int j = 0; j < 16; ++j) x[j] = 0.0f;
         }
-        const float t = lane_colsum(x, lane);
-        const int col = lane >> 1;
-        if (!(lane & 1) && col < left && m0 + warp * 32 < M)
-          O.colsum[(size_t)(m0 / 32 + warp) * N + n + col] = t;
+        // the ring's stages are free: every copy has landed and every MMA is done
+        float* cs = reinterpret_cast<float*>(tma_raw + (base - raw));
+        if (O.rows128) {
+          const float t = tile_colsum(x, cs, tid);
+          if (tid < min(left, 16)) O.colsum[(size_t)mt_id * N + n + tid] = t;
+        } else {
+          const float t = rows_colsum(x, cs + warp * 32 * 17, lane);
+          if (lane < left && lane < 16 && m0 + warp * 32 < M) O.colsum[(size_t)(m0 / 32 + warp) * N + n + lane] = t;
+        }
       }
     }
     if (O.loss) {
@@ -744,35 +776,49 @@ size_t tma_smem_bytes(int nt, int stages = TMA_STAGES) {
 
 // x (float32 [m][K]) -> h (bfloat16 rows of ldh) and, unless null, its
 // transpose hT ([K][ldt]) through a 32 x 32 shared-memory tile (both stores
-// coalesced); with part the column sums of x over each 32-row tile in
-// part[row tile][K] (fixed order)
+// coalesced); with part the column sums of x over each row tile of the block,
+// 32 rows (sub = 1, rising rows) or 128 (sub = 4, the order of
+// k_colsum_part), in part[row tile][K]
 __global__ void k_to_bf16_t(const float* x, __nv_bfloat16* h, int ldh, __nv_bfloat16* hT, int m, int K, int ldt,
-                            float* part) {
+                            float* part, int sub) {
   __shared__ float t[32][33];
   pdl_next();
   pdl_wait();
-  const int k0 = blockIdx.x * 32, r0 = blockIdx.y * 32, tx = threadIdx.x;
-  for (int j = threadIdx.y; j < 32; j += 8) {
-    const int r = r0 + j, k = k0 + tx;
-    float v = 0.0f;
-    if (r < m && k < K) {
-      v = x[(size_t)r * K + k];
-      h[(size_t)r * ldh + k] = __float2bfloat16(v);
-    }
-    t[j][tx] = v;
-  }
-  if (!hT && !part) return;
-  __syncthreads();
-  if (hT) {
+  const int k0 = blockIdx.x * 32, tx = threadIdx.x;
+  float lane_sum = 0.0f;
+  for (int s = 0; s < sub; ++s) {
+    const int r0 = ((int)blockIdx.y * sub + s) * 32;
+    if (s > 0) __syncthreads();
     for (int j = threadIdx.y; j < 32; j += 8) {
-      const int k = k0 + j, r = r0 + tx;
-      if (k < K && r < m) hT[(size_t)k * ldt + r] = __float2bfloat16(t[tx][j]);
+      const int r = r0 + j, k = k0 + tx;
+      float v = 0.0f;
+      if (r < m && k < K) {
+        v = x[(size_t)r * K + k];
+        h[(size_t)r * ldh + k] = __float2bfloat16(v);
+      }
+      t[j][tx] = v;
+      lane_sum += v;
+    }
+    if (!hT && !part) continue;
+    __syncthreads();
+    if (hT) {
+      for (int j = threadIdx.y; j < 32; j += 8) {
+        const int k = k0 + j, r = r0 + tx;
+        if (k < K && r < m) hT[(size_t)k * ldt + r] = __float2bfloat16(t[tx][j]);
+      }
     }
   }
-  if (part && threadIdx.y == 0 && k0 + tx < K) {
+  if (!part) return;
+  if (sub > 1) {
+    __syncthreads();
+    t[threadIdx.y][tx] = lane_sum;
+    __syncthreads();
+  }
+  if (threadIdx.y == 0 && k0 + tx < K) {
+    const int n = sub > 1 ? 8 : 32;
     float a = 0.0f;
 #pragma unroll 8
-    for (int j = 0; j < 32; ++j) a += t[j][tx];
+    for (int j = 0; j < n; ++j) a += t[j][tx];
     part[(size_t)blockIdx.y * K + k0 + tx] = a;
   }
 }
@@ -788,7 +834,7 @@ struct ParamTable {
   int L;
   int K[15], N[15], Kp[15], Np[15], splits[15], blk0[16];     // blk0: first block of the layer; [L]: all
   unsigned long long woff[15], boff[15], wpoff[15], wtoff[15], wsoff[15], cpoff[15];
-  int rtiles;                                                 // 32-row tiles of the batch
+  int rtiles;                                                 // row tiles of the batch (column sums)
   int nloss;
   float loss_scale;
 };
@@ -875,6 +921,11 @@ struct thor_mlp {
   std::vector<int> ps;                 // the same rounded up to multiples of 8: the rows of the bfloat16 copies
   int use_tc = 1;                      // tcgen05 TMA-fed (1) or thread-staged (2), mma.sync reference path (0)
   bool tma_ok = false;                 // the tensor-map encoder was found
+  // Every width a multiple of 8. The sums over the batch of other networks
+  // (dW_l, db_l) run in the order of the thread-staged path, dW_l unsplit, so
+  // that a training run gives the same weights on either; forward and backward
+  // of 370-256-256-256-185 at batch 1000: 64 us split, 87 us unsplit.
+  bool aligned = true;
   bool fwd_tma = false;                // the last forward kept the transposed layer inputs
   int sms = 148;                       // streaming multiprocessors of the device
   int ldt = 0;                         // row length of the transposed buffers (max_batch rounded up to 64)
@@ -1043,7 +1094,7 @@ int mlp_forward_tma(thor_mlp* net, const float* x, int m, float* y, const float*
   const int L = net->n_layers();
   dim3 g((net->sizes[0] + 31) / 32, (m + 31) / 32);
   if (launch_pass(k_to_bf16_t, g, dim3(32, 8), 0, st, x, net->h[0], net->ps[0], net->hT[0], m, net->sizes[0],
-                  net->ldt, (float*)nullptr))
+                  net->ldt, (float*)nullptr, 1))
     return THOR_ECUDA;
   for (int l = 0; l < L; ++l) {
     const int K = net->sizes[l], N = net->sizes[l + 1];
@@ -1070,6 +1121,7 @@ int mlp_forward_tma(thor_mlp* net, const float* x, int m, float* y, const float*
       J.o.CbT = net->gbT[0];
       J.o.ldt = net->ldt;
       J.o.colsum = net->cpart + net->cpoff[l];
+      J.o.rows128 = !net->aligned;
       *nloss = J.blocks();
     } else {
       J.o.C = y;
@@ -1092,7 +1144,7 @@ int mlp_backward_tma(thor_mlp* net, int m) {
     const int K = net->sizes[l], N = net->sizes[l + 1], c = (L - 1 - l) & 1;
     GemmPair P;
     GemmJob &W = P.j[l > 0 ? 1 : 0], &X = P.j[0];
-    gemm_shape(net, K, N, m, true, (int)net->ws_splits[l], W);
+    gemm_shape(net, K, N, m, net->aligned, (int)net->ws_splits[l], W);
     if (!gemm_operands(W, net->hT[l], net->ldt, net->gbT[c], net->ldt)) return THOR_ECUDA;
     W.o.C = net->ws + net->wsoff[l];
     W.o.ldc = net->ps[l + 1];
@@ -1108,6 +1160,7 @@ int mlp_backward_tma(thor_mlp* net, int m) {
       X.o.CbT = net->gbT[c ^ 1];
       X.o.ldt = net->ldt;
       X.o.colsum = net->cpart + net->cpoff[l - 1];
+      X.o.rows128 = !net->aligned;
     }
     int rc = gemm_launch(net, P, l > 0 ? 2 : 1);
     if (rc) return rc;
@@ -1121,7 +1174,7 @@ int params_pass(const thor_mlp* net, int m, float* grad, int nloss, float loss_s
   ParamTable T{};
   const int L = net->n_layers();
   T.L = L;
-  T.rtiles = (m + 31) / 32;
+  T.rtiles = net->aligned ? (m + 31) / 32 : (m + 127) / 128;
   T.nloss = nloss;
   T.loss_scale = loss_scale;
   int b = 0;
@@ -1138,7 +1191,7 @@ int params_pass(const thor_mlp* net, int m, float* grad, int nloss, float loss_s
     T.wsoff[l] = net->wsoff[l];
     T.cpoff[l] = net->cpoff[l];
     GemmJob J;
-    gemm_shape(net, K, N, std::max(m, 1), true, (int)net->ws_splits[l], J);
+    gemm_shape(net, K, N, std::max(m, 1), net->aligned, (int)net->ws_splits[l], J);
     T.splits[l] = J.splits;
     T.blk0[l] = b;
     b += weight_tiles(K, N) + (N + 7) / 8;
@@ -1162,7 +1215,7 @@ int mlp_forward_staged(thor_mlp* net, const float* x, int m) {
   const int L = net->n_layers();
   net->fwd_tma = false;
   dim3 g((net->sizes[0] + 31) / 32, (m + 31) / 32);
-  k_to_bf16_t<<<g, dim3(32, 8), 0, st>>>(x, net->h[0], net->ps[0], nullptr, m, net->sizes[0], 0, nullptr);
+  k_to_bf16_t<<<g, dim3(32, 8), 0, st>>>(x, net->h[0], net->ps[0], nullptr, m, net->sizes[0], 0, nullptr, 1);
   for (int l = 0; l < L; ++l) {
     const int K = net->sizes[l], N = net->sizes[l + 1];
     const float* b = net->p + net->boff[l];
@@ -1256,7 +1309,10 @@ int thor_mlp_create(const int* sizes, int n_sizes, int max_batch, unsigned long 
   // the TMA-fed products read rows of 16-byte multiples: the bfloat16 copies
   // of weights, layer inputs and gradients are padded with zeros to them
   net->tma_ok = encode_tiled() != nullptr;
-  for (int i = 0; i < n_sizes; ++i) net->ps.push_back((sizes[i] + 7) / 8 * 8);
+  for (int i = 0; i < n_sizes; ++i) {
+    net->ps.push_back((sizes[i] + 7) / 8 * 8);
+    net->aligned = net->aligned && sizes[i] % 8 == 0;
+  }
   net->ldt = (max_batch + 63) / 64 * 64;
   size_t nwp = 0, nwt = 0;
   for (int l = 0; l < L; ++l) {
@@ -1292,7 +1348,7 @@ int thor_mlp_create(const int* sizes, int n_sizes, int max_batch, unsigned long 
     ncp += (size_t)rt * sizes[l + 1];
     // room for the splits of the largest batch (a smaller one has no more)
     GemmJob J;
-    gemm_shape(net, sizes[l], sizes[l + 1], max_batch, true, kMaxSplit, J);
+    gemm_shape(net, sizes[l], sizes[l + 1], max_batch, net->aligned, kMaxSplit, J);
     net->ws_splits.push_back(J.splits);
     net->wsoff.push_back(nws);
     nws += (size_t)J.splits * sizes[l] * net->ps[l + 1];
@@ -1411,10 +1467,10 @@ int thor_mlp_backward(thor_mlp* net, const float* dy, int m, float* grad) {
   if (!net || !dy || !grad || m != net->last_m || m < 1) return THOR_EINVAL;
   // the TMA-fed products need the transposed inputs of a TMA-fed forward
   if (net->fwd_tma && tma_path(net)) {
-    const int L = net->n_layers(), N = net->sizes[L];
-    dim3 g((N + 31) / 32, (m + 31) / 32);
+    const int L = net->n_layers(), N = net->sizes[L], sub = net->aligned ? 1 : 4;
+    dim3 g((N + 31) / 32, (m + 32 * sub - 1) / (32 * sub));
     if (launch_pass(k_to_bf16_t, g, dim3(32, 8), 0, net->stream, dy, net->gb[0], grad_ld(net, L - 1), net->gbT[0], m, N,
-                    net->ldt, net->cpart + net->cpoff[L - 1]))
+                    net->ldt, net->cpart + net->cpoff[L - 1], sub))
       return THOR_ECUDA;
     int rc = mlp_backward_tma(net, m);
     return rc ? rc : params_pass<kGrad>(net, m, grad, 0, 0.0f, nullptr, Adam{});
