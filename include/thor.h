@@ -541,7 +541,10 @@ int thor_closure_features(thor_state* state, const float* mean, const float* std
  * (n dt) with period = n. thor_step calls that end inside a window carry it
  * over to the next call. The four normalisation arrays are caller-owned
  * device arrays that must stay valid while attached. mlp = NULL detaches
- * (plain method); re-attaching restarts the window count. */
+ * (plain method); re-attaching restarts the window count. One network may
+ * serve several states, on several streams: each evaluates it on its own
+ * stream, and thor_mlp calls run on the stream of the state attached last.
+ * Attaching to a state on another stream waits for the device. */
 int thor_closure_attach(thor_state* state, thor_mlp* mlp, const float* in_mean, const float* in_std,
                         const float* out_mean, const float* out_std, int period);
 

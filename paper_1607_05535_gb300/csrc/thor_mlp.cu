@@ -25,6 +25,8 @@
 #include <cmath>
 #include <cstdint>
 #include <cstring>
+#include <memory>
+#include <mutex>
 #include <new>
 #include <utility>
 #include <vector>
@@ -952,6 +954,12 @@ struct thor_mlp {
   std::vector<size_t> cpoff, wsoff, ws_splits;
   int last_m = 0;
   long long step_count = 0;
+  // States that evaluate the network (thor_closure_attach). stream is that of
+  // the last one attached; the others wait for updated, the event after the
+  // last change of the weights, and a change waits for their reads.
+  std::vector<std::shared_ptr<ClosureUse>> uses;
+  cudaEvent_t updated = nullptr;
+  std::mutex staged;                   // the batch buffers, lent to one state's evaluation at a time
   int n_layers() const { return (int)sizes.size() - 1; }
 };
 
@@ -1063,7 +1071,7 @@ cudaError_t launch_pass(void (*kern)(K...), dim3 grid, dim3 block, size_t smem, 
 }
 
 // one or two independent products in one launch
-int gemm_launch(const thor_mlp* net, GemmPair& P, int jobs) {
+int gemm_launch(const thor_mlp* net, GemmPair& P, int jobs, cudaStream_t st) {
   P.blocks0 = P.j[0].blocks();
   const int total = P.blocks0 + (jobs > 1 ? P.j[1].blocks() : 0);
   // the deepest ring that still lets every CTA of the grid be resident at
@@ -1078,7 +1086,7 @@ int gemm_launch(const thor_mlp* net, GemmPair& P, int jobs) {
       break;
     }
   for (int q = 0; q < jobs; ++q) P.j[q].stages = stages;
-  return launch_pass(k_gemm_tma, total, 128, tma_smem_bytes(nt, stages), net->stream, P, net->err) == cudaSuccess
+  return launch_pass(k_gemm_tma, total, 128, tma_smem_bytes(nt, stages), st, P, net->err) == cudaSuccess
              ? THOR_OK
              : THOR_ECUDA;
 }
@@ -1127,7 +1135,7 @@ int mlp_forward_tma(thor_mlp* net, const float* x, int m, float* y, const float*
       J.o.C = y;
       J.o.ldc = N;
     }
-    int rc = gemm_launch(net, P, 1);
+    int rc = gemm_launch(net, P, 1, st);
     if (rc) return rc;
   }
   net->fwd_tma = true;
@@ -1162,7 +1170,7 @@ int mlp_backward_tma(thor_mlp* net, int m) {
       X.o.colsum = net->cpart + net->cpoff[l - 1];
       X.o.rows128 = !net->aligned;
     }
-    int rc = gemm_launch(net, P, l > 0 ? 2 : 1);
+    int rc = gemm_launch(net, P, l > 0 ? 2 : 1, net->stream);
     if (rc) return rc;
   }
   return THOR_OK;
@@ -1257,8 +1265,9 @@ int mlp_backward_staged(thor_mlp* net, const float* dy, int m) {
 }
 
 // y = MLP(x) for any number of rows through two scratch buffers of m rows x
-// the widest layer, without the network's own batch buffers (inference)
-int mlp_infer(thor_mlp* net, int m, float* y, __nv_bfloat16* const buf[2]) {
+// the widest layer, without the network's own batch buffers (inference), on
+// the caller's stream
+int mlp_infer(const thor_mlp* net, int m, float* y, __nv_bfloat16* const buf[2], cudaStream_t st) {
   const int L = net->n_layers();
   for (int l = 0; l < L; ++l) {
     const int K = net->sizes[l], N = net->sizes[l + 1];
@@ -1275,9 +1284,23 @@ int mlp_infer(thor_mlp* net, int m, float* y, __nv_bfloat16* const buf[2]) {
       J.o.C = y;
       J.o.ldc = N;
     }
-    int rc = gemm_launch(net, P, 1);
+    int rc = gemm_launch(net, P, 1, st);
     if (rc) return rc;
   }
+  return THOR_OK;
+}
+
+// Around a change of the weights on net->stream: after the states that read
+// them on other streams, and before their next evaluation. Nothing where the
+// network serves one stream.
+int weights_begin(const thor_mlp* net) {
+  for (const std::shared_ptr<ClosureUse>& u : net->uses)
+    if (u->stream != net->stream && cudaStreamWaitEvent(net->stream, u->read, 0)) return THOR_ECUDA;
+  return THOR_OK;
+}
+int weights_end(const thor_mlp* net) {
+  for (const std::shared_ptr<ClosureUse>& u : net->uses)
+    if (u->stream != net->stream) return cudaEventRecord(net->updated, net->stream) ? THOR_ECUDA : THOR_OK;
   return THOR_OK;
 }
 
@@ -1444,6 +1467,7 @@ int thor_mlp_tune(thor_mlp* net, int knob, int value) {
 int thor_mlp_set_params(thor_mlp* net, const float* host, size_t n) {
   using namespace thor;
   if (!net || !host || n != net->nparam) return THOR_EINVAL;
+  if (weights_begin(net)) return THOR_ECUDA;
   if (cudaMemcpyAsync(net->p, host, n * 4, cudaMemcpyHostToDevice, net->stream)) return THOR_ECUDA;
   if (weights_copy(net)) return THOR_ECUDA;
   if (cudaMemsetAsync(net->m, 0, n * 4, net->stream) || cudaMemsetAsync(net->v, 0, n * 4, net->stream))
@@ -1495,7 +1519,9 @@ int thor_mlp_train_step(thor_mlp* net, const float* x, const float* target, int 
     int nloss = 0;
     int rc = mlp_forward_tma(net, x, m, nullptr, target, &nloss);
     if (!rc) rc = mlp_backward_tma(net, m);
-    return rc ? rc : params_pass<kAdam>(net, m, nullptr, nloss, 1.0f / (float)cnt, loss, adam());
+    if (!rc) rc = weights_begin(net);
+    if (!rc) rc = params_pass<kAdam>(net, m, nullptr, nloss, 1.0f / (float)cnt, loss, adam());
+    return rc ? rc : weights_end(net);
   }
   int rc = mlp_forward_staged(net, x, m);
   if (rc) return rc;
@@ -1503,9 +1529,11 @@ int thor_mlp_train_step(thor_mlp* net, const float* x, const float* target, int 
   k_mse<<<nb, 256, 0, st>>>(net->y, target, net->dy, cnt, 1.0f / (float)cnt, net->part);
   if (loss) k_sum_parts<<<1, 1024, 0, st>>>(net->part, nb, 1.0f / (float)cnt, loss);
   rc = mlp_backward_staged(net, net->dy, m);
+  if (!rc) rc = weights_begin(net);
   if (rc) return rc;
   k_adam<<<blocks_for(net->nparam), 256, 0, st>>>(net->p, net->grad, net->m, net->v, net->nparam, adam());
   rc = weights_copy(net);
+  if (!rc) rc = weights_end(net);
   if (rc) return rc;
   return cudaGetLastError() == cudaSuccess ? THOR_OK : THOR_ECUDA;
 }
@@ -1513,6 +1541,7 @@ int thor_mlp_train_step(thor_mlp* net, const float* x, const float* target, int 
 void thor_mlp_destroy(thor_mlp* net) {
   if (!net) return;
   if (net->arena) cudaFree(net->arena);
+  if (net->updated) cudaEventDestroy(net->updated);
   delete net;
 }
 
@@ -1655,6 +1684,7 @@ int closure_evaluate_t(thor_state* s) {
   cudaStream_t st = I->stream;
   const int ncol = I->G.ncol, nv = I->G.nv;
   const int Fin = 2 * kClosureFields * nv, Fout = kClosureFields * nv;
+  const bool apart = net->stream != st;      // the network was attached to a state on another stream since
   if (tma_path(net)) {
     // features straight into the network's bfloat16 input rows, all columns
     // in one pass of the network through the binding's own buffers, the
@@ -1663,19 +1693,25 @@ int closure_evaluate_t(thor_state* s) {
     k_features<R, __nv_bfloat16><<<turn_grid(I, kClosureFields), dim3(32, 8), 0, st>>>(
         I->G, I->Xt, cb.in_mean, cb.in_std, static_cast<__nv_bfloat16*>(cb.act[0]), net->ps[0]);
     __nv_bfloat16* const act[2] = {static_cast<__nv_bfloat16*>(cb.act[0]), static_cast<__nv_bfloat16*>(cb.act[1])};
-    const int rc = mlp_infer(net, ncol, cb.y, act);
+    if (apart && cudaStreamWaitEvent(st, net->updated, 0)) return THOR_ECUDA;
+    const int rc = mlp_infer(net, ncol, cb.y, act, st);
     if (rc) return rc;
+    if (apart && cudaEventRecord(cb.use->read, st)) return THOR_ECUDA;
     I->launches += 1 + net->n_layers();
     return cudaGetLastError() == cudaSuccess ? THOR_OK : THOR_ECUDA;
   }
   k_features<R, float><<<turn_grid(I, kClosureFields), dim3(32, 8), 0, st>>>(I->G, I->Xt, cb.in_mean, cb.in_std, cb.x, Fin);
+  // batches through the network's own buffers, hence on the network's stream
+  std::lock_guard<std::mutex> lend(net->staged);
+  if (apart && (cudaEventRecord(cb.use->read, st) || cudaStreamWaitEvent(net->stream, cb.use->read, 0))) return THOR_ECUDA;
   for (int c0 = 0; c0 < ncol; c0 += net->max_batch) {
     const int m = std::min(net->max_batch, ncol - c0);
     int rc = mlp_forward_staged(net, cb.x + (size_t)c0 * Fin, m);
     if (rc) return rc;
-    if (cudaMemcpyAsync(cb.y + (size_t)c0 * Fout, net->y, (size_t)m * Fout * 4, cudaMemcpyDeviceToDevice, st))
+    if (cudaMemcpyAsync(cb.y + (size_t)c0 * Fout, net->y, (size_t)m * Fout * 4, cudaMemcpyDeviceToDevice, net->stream))
       return THOR_ECUDA;
   }
+  if (apart && (cudaEventRecord(net->updated, net->stream) || cudaStreamWaitEvent(st, net->updated, 0))) return THOR_ECUDA;
   I->launches += 1 + (1 + net->n_layers()) * ((ncol + net->max_batch - 1) / net->max_batch);
   return cudaGetLastError() == cudaSuccess ? THOR_OK : THOR_ECUDA;
 }
@@ -1824,6 +1860,7 @@ int closure_large_step(thor_state* s, int n_small, double dt) {
 }
 
 void closure_release(thor_state* s) {
+  if (s->closure.net) cudaStreamSynchronize(s->impl->stream);   // its last evaluation, before the network forgets it
   if (s->closure.x) cudaFree(s->closure.x);
   if (s->closure.y) cudaFree(s->closure.y);
   for (void* a : s->closure.act)
@@ -1935,7 +1972,23 @@ int thor_closure_attach(thor_state* s, thor_mlp* net, const float* in_mean, cons
     closure_release(s);
     return THOR_ENOMEM;
   }
-  net->stream = s->impl->stream;            // the closure runs on the state's stream
+  // The network moves to the state's stream. What is queued on its old one
+  // (training, another state's evaluation) comes first; that stream may be
+  // gone by now, so the wait is for the device.
+  cudaStream_t st = s->impl->stream;
+  cb.use = std::make_shared<ClosureUse>();
+  cb.use->stream = st;
+  if ((net->stream != st && cudaDeviceSynchronize()) || cudaEventCreateWithFlags(&cb.use->read, cudaEventDisableTiming) ||
+      (!net->updated && cudaEventCreateWithFlags(&net->updated, cudaEventDisableTiming))) {
+    s->closure = cb;
+    closure_release(s);
+    return THOR_ECUDA;
+  }
+  net->uses.erase(std::remove_if(net->uses.begin(), net->uses.end(),
+                                 [](const std::shared_ptr<ClosureUse>& u) { return u.use_count() == 1; }),
+                  net->uses.end());
+  net->uses.push_back(cb.use);
+  net->stream = st;
   s->closure = cb;
   return THOR_OK;
 }

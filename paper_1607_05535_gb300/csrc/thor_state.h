@@ -12,9 +12,21 @@ struct thor_grid {
   thor::HostGrid h;
 };
 
+// One state's use of a network, known to both: the state's stream, and an
+// event after the last launch there that reads the network (or, where the
+// evaluation runs on the network's own stream, after its features).
+struct ClosureUse {
+  cudaStream_t stream = nullptr;
+  cudaEvent_t read = nullptr;
+  ~ClosureUse() {
+    if (read) cudaEventDestroy(read);
+  }
+};
+
 // learned closure attached to a state (thor_closure_attach)
 struct ClosureBinding {
   thor_mlp* net = nullptr;
+  std::shared_ptr<ClosureUse> use;
   const float *in_mean = nullptr, *in_std = nullptr, *out_mean = nullptr, *out_std = nullptr;
   float *x = nullptr, *y = nullptr;   // per-state feature / output buffers
   void* act[2] = {nullptr, nullptr};  // bfloat16 layer inputs of every column (two of the widest layer)
