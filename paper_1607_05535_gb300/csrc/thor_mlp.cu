@@ -1746,15 +1746,22 @@ int closure_large_step_t(thor_state* s, int n_small, double dt) {
 // members of a coarse column are counted, each column takes a segment of the
 // list (in any order: only the order within a segment enters the sums), the
 // segments are filled, and sorted by rank so that every sum runs over rising
-// fine columns whatever the atomics' order. bad is set for an index out of
-// range or a coarse column without members; the averaging kernel then leaves
-// the coarse state as it is. Building the lists on the host, with three
+// fine columns whatever the atomics' order. kCgBad is set for an index out of
+// range or a coarse column without members, kCgLong for a column with more
+// than kCgRank members (ranking compares every member with every other); the
+// kernels that follow then do nothing, so a refused map costs no more than its
+// count, and lists with a long segment are built on the host in one pass over the
+// map and averaged in a second launch. Building all lists on the host, with three
 // buffers allocated and freed around it, made the call 260 us at g6 -> g5 x 32;
 // now it is 121 us: 12 us for the map's upload, 20 us for the lists, 67 us for
 // the averages (bound by the float64 pipe, 82% busy: building the doubles on
 // the integer ALU instead of converting gave 68 us) and the read-back.
+// The limit lies between the lengths measured on both sides, g6 x 32 onto
+// coarser grids: longest list 267, 316 us on the device and 411 with the lists
+// from the host; 995, 1292 and 986; 3426, 7050 and 2450.
+constexpr int kCgRank = 512, kCgBad = 1, kCgLong = 2;
 struct CoarseLists {
-  int *map, *count, *start, *cursor, *raw, *member, *state;   // state[0] bad, state[1] list length
+  int *map, *count, *start, *cursor, *raw, *member, *state;   // state[0] kCgBad | kCgLong, state[1] list length
   double* weight;
 };
 
@@ -1763,7 +1770,7 @@ __global__ void k_cg_count(const int* __restrict__ map, int nfine, int ncol, int
   if (f >= nfine) return;
   const int c = map[f];
   if (c < 0 || c >= ncol)
-    state[0] = 1;
+    atomicOr(state, kCgBad);
   else
     atomicAdd(count + c, 1);
 }
@@ -1782,21 +1789,23 @@ __global__ void k_cg_start(const int* __restrict__ count, int ncol, int* start, 
   base = __shfl_sync(0xffffffffu, base, 31);
   if (c >= ncol) return;
   start[c] = cursor[c] = base + sum - n;
-  if (n == 0) state[0] = 1;
+  if (n == 0) atomicOr(state, kCgBad);
+  if (n > kCgRank) atomicOr(state, kCgLong);
 }
 
-__global__ void k_cg_fill(const int* __restrict__ map, int nfine, int ncol, int* cursor, int* raw) {
+__global__ void k_cg_fill(const int* __restrict__ map, int nfine, int ncol, const int* __restrict__ state, int* cursor,
+                          int* raw) {
   const int f = blockIdx.x * blockDim.x + threadIdx.x;
-  if (f >= nfine) return;
+  if (f >= nfine || state[0]) return;
   const int c = map[f];
   if (c >= 0 && c < ncol) raw[atomicAdd(cursor + c, 1)] = f;
 }
 
 // a warp per coarse column: members in rising order, and their weights
 __global__ void k_cg_sort(const int* __restrict__ count, const int* __restrict__ start, int ncol,
-                          const int* __restrict__ raw, const double* __restrict__ area, int* member, double* weight) {
+                          const int* __restrict__ state, const int* __restrict__ raw, const double* __restrict__ area, int* member, double* weight) {
   const int c = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
-  if (c >= ncol) return;
+  if (c >= ncol || state[0]) return;
   const int n = count[c], s = start[c];
   for (int i = lane; i < n; i += 32) {
     const int f = raw[s + i];
@@ -1916,23 +1925,51 @@ int coarse_t(thor_state* fine, thor_state* coarse, const int* map) {
   L.state = L.count + nc;
   L.start = L.state + 2;
   L.cursor = L.start + nc;
+  auto average = [&]() {
+    k_coarse_grain<R><<<dim3((nc + 127) / 128, C->G.nv + 1), 128, 0, st>>>(C->G, F->Xt, F->G.colp, C->Xt, C->XtL, L);
+    return !cudaGetLastError();
+  };
   bool ok = !cudaMemcpyAsync(L.map, map, nf * sizeof(int), cudaMemcpyHostToDevice, st) &&
             !cudaMemsetAsync(L.count, 0, ((size_t)nc + 2) * sizeof(int), st);
-  k_cg_count<<<(nf + 255) / 256, 256, 0, st>>>(L.map, nf, nc, L.count, L.state);
-  k_cg_start<<<(nc + 255) / 256, 256, 0, st>>>(L.count, nc, L.start, L.cursor, L.state);
-  k_cg_fill<<<(nf + 255) / 256, 256, 0, st>>>(L.map, nf, nc, L.cursor, L.raw);
-  // from here on the fine state is read: its tables and fields are complete on its own stream
+  // the fine state's tables and fields are complete on its own stream
   if (F->stream != st) ok = ok && !cudaEventRecord(w.ready, F->stream) && !cudaStreamWaitEvent(st, w.ready, 0);
-  int bad = 0;
+  int state = 0;
   if (ok) {
-    k_cg_sort<<<(nc + 7) / 8, 256, 0, st>>>(L.count, L.start, nc, L.raw, F->G.area, L.member, L.weight);
-    k_coarse_grain<R><<<dim3((nc + 127) / 128, C->G.nv + 1), 128, 0, st>>>(C->G, F->Xt, F->G.colp, C->Xt, C->XtL, L);
+    k_cg_count<<<(nf + 255) / 256, 256, 0, st>>>(L.map, nf, nc, L.count, L.state);
+    k_cg_start<<<(nc + 255) / 256, 256, 0, st>>>(L.count, nc, L.start, L.cursor, L.state);
+    k_cg_fill<<<(nf + 255) / 256, 256, 0, st>>>(L.map, nf, nc, L.state, L.cursor, L.raw);
+    k_cg_sort<<<(nc + 7) / 8, 256, 0, st>>>(L.count, L.start, nc, L.state, L.raw, F->G.area, L.member, L.weight);
+    ok = average() && !cudaMemcpyAsync(&state, L.state, sizeof(int), cudaMemcpyDeviceToHost, st);
     C->launches += 5;
-    ok = !cudaGetLastError() && !cudaMemcpyAsync(&bad, L.state, sizeof(int), cudaMemcpyDeviceToHost, st);
   }
   // on every path: the map is the caller's, and the fine state may change after the call
   if (cudaStreamSynchronize(st) || !ok) return THOR_ECUDA;
-  return bad ? THOR_EINVAL : THOR_OK;
+  if (state & kCgBad) return THOR_EINVAL;
+  if (!(state & kCgLong)) return THOR_OK;
+  // the lists from the host: the same members in the same order
+  std::vector<int> start(nc + 1, 0), count(nc), at(nc), member(nf);
+  std::vector<double> area(nc, 0.0), weight(nf);
+  for (int f = 0; f < nf; ++f) {
+    ++start[map[f] + 1];
+    area[map[f]] += fine->grid->h.area[f];
+  }
+  for (int c = 0; c < nc; ++c) {
+    count[c] = start[c + 1];
+    at[c] = start[c];
+    start[c + 1] += start[c];
+  }
+  for (int f = 0; f < nf; ++f) {
+    const int e = at[map[f]]++;
+    member[e] = f;
+    weight[e] = fine->grid->h.area[f] / area[map[f]];
+  }
+  ok = !cudaMemcpyAsync(L.start, start.data(), nc * sizeof(int), cudaMemcpyHostToDevice, st) &&
+       !cudaMemcpyAsync(L.count, count.data(), nc * sizeof(int), cudaMemcpyHostToDevice, st) &&
+       !cudaMemcpyAsync(L.member, member.data(), nf * sizeof(int), cudaMemcpyHostToDevice, st) &&
+       !cudaMemcpyAsync(L.weight, weight.data(), nf * sizeof(double), cudaMemcpyHostToDevice, st) &&
+       !cudaMemsetAsync(L.state, 0, sizeof(int), st) && average();
+  if (ok) C->launches += 1;
+  return cudaStreamSynchronize(st) || !ok ? THOR_ECUDA : THOR_OK;
 }
 }  // namespace
 
