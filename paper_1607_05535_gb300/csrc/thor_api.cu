@@ -586,9 +586,9 @@ int Impl<R>::set_compensated(int on) {
 //    solve wants more shared memory than the stencils, and an SM changes the
 //    split only when idle, twice a small step (77 k 253 -> 220, 123 k 216 ->
 //    211; larger grids lose more L1 than they gain, 1.31 M 1263 -> 1319).
-//  - at most a block per SM, float: each kernel starts beside the one before
-//    it (7.7 k 166 -> 152; with more blocks the early ones take the room of
-//    the running ones, 77 k 220 -> 235).
+//  - at most a block per SM as launched, float: each kernel starts beside the
+//    one before it (7.7 k 166 -> 152; with more blocks the early ones take the
+//    room of the running ones, 77 k 220 -> 235).
 template <typename R>
 void Impl<R>::shape() {
   const long long cells = (long long)G.ncol * G.nv;
@@ -597,7 +597,9 @@ void Impl<R>::shape() {
   level_split = cells >= (f32 ? 800000 : 200000);
   dense = f32 && cells >= 800000;
   carveout = f32 && few ? 50 : -1;
-  overlap = f32 && few && (long long)((G.ncol + block - 1) / block) * G.nv <= 152;
+  overlap = f32 && few;
+  int dev = 0;
+  if (cudaGetDevice(&dev) || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) sms = 0;
 }
 
 template Impl<double>::~Impl();

@@ -121,7 +121,8 @@ struct ImplBase {
   int block = kBlock;                  // threads (columns) per block of the stencil kernels
   int solve_tma = 1;                   // TMA-staged column solve where available
   int level_split = 1;                 // small-step stencils in two level halves on two streams
-  int overlap = 0;                     // start kernels while the one before drains (pdl_wait)
+  int overlap = 0;                     // start kernels while the one before drains (pdl_wait), grids of at most sms blocks
+  int sms = 0;                         // streaming multiprocessors of the device
   int dense = 0;                       // slow terms in few registers (k_slow)
   int carveout = -1;                   // LaunchHint::carveout of every kernel of the step
   int rk_stages = 3;                   // RK3 stages a large step runs (THOR_TUNE_RK_STAGES; tests)

@@ -1692,7 +1692,7 @@ int Impl<R>::large_step(double dt, int n_small) {
   // level halves of the small-step stencils (THOR_TUNE_LEVEL_SPLIT): levels
   // [0, kc * hc) on the state's stream, [kc * hc, nv) on side2
   const bool lsplit = level_split && side != nullptr && !prof_on && side2 != nullptr && G.nv >= 2 * kc;
-  const bool pdl = overlap && !lsplit && !prof_on && stream != nullptr;
+  const bool pdl = overlap && !lsplit && !prof_on && stream != nullptr && (long long)g2.x * g2.y <= sms;
   auto hint = [&](bool after) { return LaunchHint{after, carveout}; };
   const int nch = (G.nv + kc - 1) / kc, hc = lsplit ? nch / 2 : nch;
   dim3 glo(g2.x, hc), ghi(g2.x, nch - hc);
