@@ -165,9 +165,10 @@ template <> __device__ __forceinline__ float rexp<float>(float x) { return expf(
 template <typename R> __device__ __forceinline__ R rpow(R x, R y);
 template <> __device__ __forceinline__ double rpow<double>(double x, double y) { return pow(x, y); }
 template <> __device__ __forceinline__ float rpow<float>(float x, float y) { return powf(x, y); }
-template <typename R> __device__ __forceinline__ R rsinpi(R x);      // sin(pi x)
-template <> __device__ __forceinline__ double rsinpi<double>(double x) { return sinpi(x); }
-template <> __device__ __forceinline__ float rsinpi<float>(float x) { return sinpif(x); }
+// sin(pi x), in float64 for either type and rounded once: sinpif is off by up
+// to 1 ulp (about 13 float64 instructions a cell: the hot Jupiter's large step
+// at g6 x 32 1.066 -> 1.083 ms)
+template <typename R> __device__ __forceinline__ R rsinpi(R x) { return (R)sinpi((double)x); }
 
 // a b + c with one rounding, written out where a sum of two products could
 // otherwise be contracted either way (kernels that must agree bit for bit

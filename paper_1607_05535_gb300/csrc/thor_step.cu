@@ -1051,7 +1051,7 @@ __device__ __forceinline__ void d_physics(const Geo<R>& G, const VR<R>& U, const
       Teq = Teq > R(200) ? Teq : R(200);
     } else {
       const R ss = R(0.12), zs = R(2.0e6);
-      const R bt = ld(U.zc + (k)) <= zs ? rsinpi<R>((sigma - ss) * (R(0.5) / (R(1) - ss))) : R(0);
+      const R bt = ld(U.zc + (k)) <= zs ? rsinpi<R>((sigma - ss) / (R(2) * (R(1) - ss))) : R(0);
       Kv = 0;
       KT = R(1) / R(1.5e5);
       Teq = ld(U.hjT + (k)) + bt * (R)hj_dT * clcl;
