@@ -1595,7 +1595,11 @@ __device__ __forceinline__ void NbrMean<float>::add(float a) {
   e += d1 + t1;
 }
 template <>
-__device__ __forceinline__ float NbrMean<float>::anomaly(int nn) const { return (s + e) / (float)nn; }
+__device__ __forceinline__ float NbrMean<float>::anomaly(int nn) const {
+  // the quotient of s, corrected by its exact remainder and the low part: one rounding
+  const float n = (float)nn, inv = 1.0f / n, q = s * inv;
+  return q + (fmaf(-q, n, s) + e) * inv;
+}
 __device__ __forceinline__ void feature_store(float* x, float v) { *x = v; }
 __device__ __forceinline__ void feature_store(__nv_bfloat16* x, float v) { *x = __float2bfloat16(v); }
 
