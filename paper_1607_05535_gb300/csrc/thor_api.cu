@@ -152,7 +152,7 @@ void carve(Carver& cv, Impl<R>& I, int ncol, int nv) {
   T.vr = cv.take<R>(F);
   T.qvr = cv.take<R>(F);
   T.wc = cv.take<R>(C);
-  T.psurf = cv.take<R>(S);
+  T.psurf = cv.take<R>(2 * S);
   Slow<R>& SL = I.SL;
   R** sc[] = {&SL.srho, &SL.sth, &SL.dsc, &SL.acr, &SL.pi};
   for (R** p : sc) *p = cv.take<R>(C);

@@ -32,7 +32,7 @@ struct Work {
   R *lp;                           // p* + K_d lap(D): the scalar whose gradient drives M*
   R *ca, *cb, *cc;                 // per-cell parts of the column equations (a, b, c)
   R *dhm;                          // horizontal divergence of the new M*
-  R *psurf;                        // [colp] surface pressure (physics)
+  R *psurf;                        // [2][colp] surface pressure and its reciprocal (physics)
 };
 
 // Slow tendencies and small-step coefficients of a stage

@@ -138,7 +138,7 @@ __device__ __forceinline__ void d_lap1(const Geo<R>& G, const VR<R>& U, const Xf
       int o = k * S;
       R rlo = ld(U.rhob + (k - 1)) + ld(X.rho + (o - S + c)), rhi = ld(U.rhob + (k)) + ld(X.rho + (o + c));
       R rif = HO ? vint_iface(U, X.rho, U.rhob, k, c, S, G.nv) : ld(U.wlo + (k)) * rlo + ld(U.whi + (k)) * rhi;
-      T.qvr[o + c] = rif * Kd * apply7(wl, nb, T.vr + o) * ld(U.inv_ri2 + (k));
+      T.qvr[o + c] = div_by(rif * Kd * apply7(wl, nb, T.vr + o), ld(U.ri2 + (k)), ld(U.inv_ri2 + (k)));
     } else if (k == 0 || k == G.nv) {
       T.qvr[k * S + c] = 0;
     }
@@ -369,7 +369,7 @@ __device__ __forceinline__ void d_slow_w(const Geo<R>& G, const VR<R>& U, const 
     // inertia that the hydrostatic switch drops
     if (!ph.hydrostatic) {
       R FW = 0;
-      if (hyper) FW = -apply7(wl, nb, T.qvr + k * S) * ld(U.inv_ri2 + (k));
+      if (hyper) FW = div_by(-apply7(wl, nb, T.qvr + k * S), ld(U.ri2 + (k)), ld(U.inv_ri2 + (k)));
       const R acr_i = HO ? vint_iface(U, (const R*)SL.acr, (const R*)nullptr, k, c, S, G.nv)
                                     : wlo * ld(SL.acr + (i - S)) + whi * ld(SL.acr + (i));
       sw = sw - acr_i + FW;
@@ -986,7 +986,7 @@ __device__ __forceinline__ void d_ss_solve(const Geo<double>& G, const VR<double
 // (Eq. im_eq_t) with the Sec. 6.1 Held-Suarez or Sec. 6.2 hot-Jupiter
 // coefficients; sigma = p / p_s with p_s extrapolated hydrostatically at the
 // lowest layer's temperature.
-// 1 / p_s of every column before the physics update, from its lowest layer
+// p_s (and 1 / p_s, div_by) of every column before the physics update, from its lowest layer
 // (one thread per column; the update kernel then works on chunks of levels
 // and changes the lowest layer's rho theta)
 template <typename R>
@@ -997,7 +997,9 @@ __device__ __forceinline__ void d_surface_p(const Geo<R>& G, const VR<R>& U, con
   const R Rd = pc<R>(ph.Rd, ph.Rd_f);
   R p0 = ld(U.pb + (0)) + eos_level(U, ph, 0, ld(X.th + (c)));
   R T0 = p0 / ((ld(U.rhob + (0)) + ld(X.rho + (c))) * Rd);
-  T.psurf[c] = R(1) / (p0 * rexp<R>(pc<R>(ph.g, ph.g_f) * ld(U.zc + (0)) / (Rd * T0)));
+  const R ps = p0 * rexp<R>(pc<R>(ph.g, ph.g_f) * ld(U.zc + (0)) / (Rd * T0));
+  T.psurf[c] = ps;
+  T.psurf[G.colp + c] = R(1) / ps;
 }
 
 // XL: the low parts of a compensated state (null: none); there the friction
@@ -1014,7 +1016,7 @@ __device__ __forceinline__ void d_physics(const Geo<R>& G, const VR<R>& U, const
   const R gamma = pc<R>(ph.gamma, ph.gamma_f), inv_gamma = pc<R>(ph.inv_gamma, ph.inv_gamma_f),
           Rd = pc<R>(ph.Rd, ph.Rd_f), kappa = pc<R>(ph.kappa, ph.kappa_f);
   R sl = ld(G.sinlat + (c)), cl = ld(G.coslat + (c)), clcl = ld(G.xdir + (c));
-  const R inv_ps = ld(T.psurf + (c));
+  const R ps = ld(T.psurf + (c)), inv_ps = ld(T.psurf + (S + c));
   const R rdt = (R)dt;
   const int k0 = by * kchunk, k1 = min(G.nv, k0 + kchunk);
   const bool cmp = XL.rho != nullptr;
@@ -1048,13 +1050,13 @@ __device__ __forceinline__ void d_physics(const Geo<R>& G, const VR<R>& U, const
       }
     }
     R Temp = p / (rho * Rd);
-    R sigma = p * inv_ps;
+    R sigma = div_by(p, ps, inv_ps);
     R Kv, KT, Teq;
     if (forcing == THOR_FORCING_HELD_SUAREZ) {
       const R day = R(86400.0);
       const R kf = R(1) / day, ka = R(1) / (R(40) * day), ks = R(1) / (R(4) * day);
       const R sb = R(0.7);
-      R ramp = (sigma - sb) * (R(1) / (R(1) - sb));
+      R ramp = div_by(sigma - sb, R(1) - sb, R(1) / (R(1) - sb));
       ramp = ramp > R(0) ? ramp : R(0);
       Kv = kf * ramp;
       R c2 = cl * cl;
@@ -1063,7 +1065,7 @@ __device__ __forceinline__ void d_physics(const Geo<R>& G, const VR<R>& U, const
       Teq = Teq > R(200) ? Teq : R(200);
     } else {
       const R ss = R(0.12), zs = R(2.0e6);
-      const R bt = ld(U.zc + (k)) <= zs ? rsinpi<R>((sigma - ss) / (R(2) * (R(1) - ss))) : R(0);
+      const R bt = ld(U.zc + (k)) <= zs ? rsinpi<R>(div_by(sigma - ss, R(2) * (R(1) - ss), R(0.5) / (R(1) - ss))) : R(0);
       Kv = 0;
       KT = R(1) / R(1.5e5);
       Teq = ld(U.hjT + (k)) + bt * (R)hj_dT * clcl;
