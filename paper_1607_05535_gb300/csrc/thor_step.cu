@@ -85,7 +85,6 @@ __device__ __forceinline__ void d_derived(const Geo<R>& G, const VR<R>& U, const
       R pp = eos_level(U, ph, k, thp);
       R p = ld(U.pb + (k)) + pp;
       R inv = R(1) / rho;
-      R Temp = p * inv * inv_Rd;
       R wc = HO ? vint_centre(U, X.w, k, c, S, G.nv)
                            : ld(U.clo + (k)) * ld(X.w + (i)) + ld(U.chi + (k)) * ld(X.w + (i + S));
       R mx = ld(X.mx + (i)), my = ld(X.my + (i)), mz = ld(X.mz + (i));
@@ -95,7 +94,10 @@ __device__ __forceinline__ void d_derived(const Geo<R>& G, const VR<R>& U, const
       pi[i] = gamma * p / thfull;
       T.theta[i] = theta;
       st4(T.v4, i, (mx + wc * rx) * inv, (my + wc * ry) * inv, (mz + wc * rz) * inv, theta);
-      st4(T.vh4, i, mx * inv, my * inv, mz * inv, Temp - ld(U.Tb + (k)));
+      // T' = p / (rho Rd) - T_bar in one rounding of the difference, written out: left to
+      // contraction, the ensemble's kernel rounded T first, which as noise of 2^-25 of
+      // 300 K went through the hyperdiffusion (error of rho' after a step +11%)
+      st4(T.vh4, i, mx * inv, my * inv, mz * inv, fmar<R>(p * inv, inv_Rd, -ld(U.Tb + (k))));
       if (shallow) T.wc[i] = wc * inv;
     }
     if (k >= 1 && k < G.nv) {
