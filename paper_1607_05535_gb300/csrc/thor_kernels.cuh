@@ -170,12 +170,16 @@ template <> __device__ __forceinline__ float rpow<float>(float x, float y) { ret
 // at g6 x 32 1.066 -> 1.083 ms)
 template <typename R> __device__ __forceinline__ R rsinpi(R x) { return (R)sinpi((double)x); }
 
-// a / b where inv = 1 / b is at hand, rounded as the division: float divides;
-// float64 corrects the product by its exact remainder (Markstein 1990, IBM J.
-// Res. Dev. 34), 3 instructions of its narrow pipe against about 10 for the
-// division and 1 for the product alone, which is off by up to 1.5 units in
-// the last place. An infinite a gives NaN in float64.
-__device__ __forceinline__ float div_by(float a, float b, float) { return a / b; }
+// a / b where inv = 1 / b is at hand, rounded as the division: the product
+// corrected by its exact remainder (Markstein 1990, IBM J. Res. Dev. 34),
+// 3 instructions against about 10 for the division and 1 for the product alone,
+// which is off by up to 1.5 units in the last place (with float divisions
+// instead the 64-member ensemble took 24.16 ms for two large steps, with this
+// 23.78). An infinite a gives NaN.
+__device__ __forceinline__ float div_by(float a, float b, float inv) {
+  const float q = a * inv;
+  return fmaf(fmaf(-q, b, a), inv, q);
+}
 __device__ __forceinline__ double div_by(double a, double b, double inv) {
   const double q = a * inv;
   return fma(fma(-q, b, a), inv, q);
