@@ -169,7 +169,10 @@ __device__ __forceinline__ void d_slow(const Geo<R>& G, const VR<R>& U, const Ph
   Nbr7 nb = load_nbr(G, c);
   // the divergence and Laplacian weights; the gradient of p below is taken
   // with the divergence weights plus the centre correction, unprojected
-  // (S_M is projected as a whole)
+  // (S_M is projected as a whole). A constant has no tangential gradient, so float
+  // states take the differences to the centre, whose products round on the scale of
+  // the differences; the centre's own weights drop out
+  constexpr bool kByDifference = sizeof(R) == sizeof(float);
   W7x3<R> wd;
   W7<R> wl;
   load_w7x3_lap(G.wdiv, S0, c, wd, wl);
@@ -190,7 +193,7 @@ __device__ __forceinline__ void d_slow(const Geo<R>& G, const VR<R>& U, const Ph
     // advection and rho-theta divergences), the pressure gradient and the
     // second Laplacians of the hyperdiffusion
     R sa0 = 0, sa1 = 0, sa2 = 0, sa3 = 0, sdh = 0, sdt = 0, gx = 0, gy = 0, gz = 0;
-    R hr = 0, hx = 0, hy = 0, hz = 0, hT = 0;
+    R hr = 0, hx = 0, hy = 0, hz = 0, hT = 0, p0 = 0;
     // advected velocity (packed with theta or T'): the full 3-D one, or (SH)
     // the horizontal one and w
     const R* av4 = SH ? T.vh4 : T.v4;
@@ -206,13 +209,23 @@ __device__ __forceinline__ void d_slow(const Geo<R>& G, const VR<R>& U, const Ph
       sdh += f;
       sdt += (SH ? ld(T.theta + q) : av.w) * f;
       const R pq = ld(T.pp + q);
-      gx += wd.x[j] * pq;
-      gy += wd.y[j] * pq;
-      gz += wd.z[j] * pq;
-      if (j == 0) {
-        gx += gcx * pq;
-        gy += gcy * pq;
-        gz += gcz * pq;
+      if constexpr (kByDifference) {
+        if (j == 0) {
+          p0 = pq;
+        } else {
+          gx += wd.x[j] * (pq - p0);
+          gy += wd.y[j] * (pq - p0);
+          gz += wd.z[j] * (pq - p0);
+        }
+      } else {
+        gx += wd.x[j] * pq;
+        gy += wd.y[j] * pq;
+        gz += wd.z[j] * pq;
+        if (j == 0) {
+          gx += gcx * pq;
+          gy += gcy * pq;
+          gz += gcz * pq;
+        }
       }
       if (hyper) {
         const Q4<R> hq = ld4(T.q4, (size_t)q);
@@ -290,6 +303,17 @@ __device__ __forceinline__ void d_slow(const Geo<R>& G, const VR<R>& U, const Ph
 
     // the anelastic switch leaves the pressure force to the projection
     const R pgr = ph.anelastic ? R(0) : inv_r;
+    // Float: the advection's and the diffusion's radial parts go first, since a
+    // radial part leaks into the tangential one by the rounding of the basis
+    if constexpr (kByDifference) {
+      const R d = SH ? A[0] * rx + A[1] * ry + A[2] * rz : acr, f = FMx * rx + FMy * ry + FMz * rz;
+      A[0] -= d * rx;
+      A[1] -= d * ry;
+      A[2] -= d * rz;
+      FMx -= f * rx;
+      FMy -= f * ry;
+      FMz -= f * rz;
+    }
     // the tangential part of the sum, in the basis the small step works in
     // (tan_to with X = s rx, Y = s ry, s = sign(rz): one register instead of three)
     const R sx = -gx * pgr - A[0] + FMx, sy = -gy * pgr - A[1] + FMy, sz = -gz * pgr - A[2] + FMz;
