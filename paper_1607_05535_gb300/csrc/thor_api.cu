@@ -209,17 +209,17 @@ struct HostSetup {
   std::vector<int> ij0, cj0;      // [nv + 1], [nv]
 };
 // ((1 + x)^a - 1) / (a x) = 1 + g_1 x + g_2 x^2 + ... (Newton's binomial
-// series), and the largest power of two x at which the remainder after g_n,
-// sum over k > n of |g_k| x^k, is at most eps
+// series), and the largest x = 2^(-e / steps), e >= 3 steps, at which the
+// remainder after g_n, sum over k > n of |g_k| x^k, is at most eps
 struct PowSeries {
   double g[65];
   explicit PowSeries(double a) {
     g[0] = 1.0;
     for (int k = 1; k <= 64; ++k) g[k] = g[k - 1] * (a - k) / (k + 1);
   }
-  double range(int n, double eps) const {
-    for (int e = 3; e < 60; ++e) {
-      const double x = std::ldexp(1.0, -e);
+  double range(int n, double eps, int steps = 1) const {
+    for (int e = 3 * steps; e < 60 * steps; ++e) {
+      const double x = std::exp2(-(double)e / steps);
       double rest = 0.0;
       for (int k = 64; k > n; --k) rest = (rest + std::fabs(g[k])) * x;
       for (int k = 0; k < n; ++k) rest *= x;
@@ -794,10 +794,10 @@ int make_impl(thor_grid* grid, const thor_planet& pl, const thor_init& in, cudaS
     const PowSeries a(I->ph.gamma), b(I->ph.inv_gamma);
     for (int k = 0; k < 7; ++k) I->ph.pg[k] = a.g[k + 1];
     for (int k = 0; k < 6; ++k) I->ph.qg[k] = b.g[k + 1];
-    for (int k = 0; k < 3; ++k) I->ph.pg_f[k] = (float)a.g[k + 1];
+    for (int k = 0; k < 4; ++k) I->ph.pg_f[k] = (float)a.g[k + 1];
     I->ph.x4 = a.range(4, std::ldexp(1.0, -55));
     I->ph.x7 = a.range(7, std::ldexp(1.0, -55));
-    I->ph.x3_f = (float)a.range(3, std::ldexp(1.0, -26));
+    I->ph.x3_f = (float)a.range(4, std::ldexp(1.0, -26), 16);
   }
   I->ph.hydrostatic = in.hydrostatic ? 1 : 0;
   I->ph.vorder = in.vorder > 1 ? in.vorder : 1;
