@@ -373,8 +373,11 @@ int upload_tables(Impl<R>& I, const HostGrid& h, const std::vector<double>* vert
     if (I.U.pw && !pow_series_ok(I.ph.gamma)) I.U.pw = nullptr;
     if (I.U.pw) {
       for (int j = 0; j < kPowRows; ++j) {
-        const double c = 0.5 + j / 64.0, l = std::log1p(c - 1.0);
-        const double row[kPowCols] = {c - 1.0, 1.0 / c, std::expm1(I.ph.gamma * l), std::exp(I.ph.gamma * l), l, 0.0};
+        // from long double: a unit in the last place of a row would be one of every result that uses it
+        const double c = 0.5 + j / 64.0;
+        const long double l = std::log1p((long double)c - 1.0L), gl = I.ph.gamma * l, pm1 = std::expm1(gl);
+        const double hi = (double)pm1;
+        const double row[kPowCols] = {c - 1.0, 1.0 / c, hi, (double)std::exp(gl), (double)l, (double)(pm1 - hi)};
         std::copy(row, row + kPowCols, pw.begin() + (size_t)j * kPowCols);
       }
       e = e ? e : up(I.U.pw, pw.data(), pw.size() * sizeof(double));

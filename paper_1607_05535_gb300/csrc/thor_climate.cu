@@ -46,7 +46,7 @@ __global__ void __launch_bounds__(kZonalThreads)
   const int4 ch = chunk[blockIdx.x];               // band, first and last + 1 of order
   if (threadIdx.x == 0) sinv = 1.0 / V.thb[k];
   __syncthreads();
-  const double rhob = V.rhob[k], pb = V.pb[k], clo = V.clo[k], chi = V.chi[k], inv_thb = sinv;
+  const double rhob = V.rhob[k], thb = V.thb[k], pb = V.pb[k], clo = V.clo[k], chi = V.chi[k], inv_thb = sinv;
   const double vol = V.rc[k] * V.rc[k] * V.dz[k];
   double acc[kZonalQ] = {};
   for (int t = ch.y + threadIdx.x; t < ch.z; t += kZonalThreads) {
@@ -55,7 +55,7 @@ __global__ void __launch_bounds__(kZonalThreads)
     // the full value of a field: a compensated state adds its low part XL
     auto val = [&](const R* hi, const R* lo, size_t j) { return lo ? (double)hi[j] + (double)lo[j] : (double)hi[j]; };
     const double inv = 1.0 / (rhob + val(X.rho, XL.rho, i));
-    const double x = val(X.th, XL.th, i) * inv_thb;
+    const double x = div_by(val(X.th, XL.th, i), thb, inv_thb);
     double f, ln;
     if (!pow1p<false>(ph, pw, x, f, ln)) f = pow1p_general(x, ph.gamma).x;
     const double p = fma(pb, f, pb);

@@ -1056,7 +1056,7 @@ __device__ __forceinline__ void d_physics(const Geo<R>& G, const VR<R>& U, const
     const R p00 = R(1.0e5);
     R p, lpr = 0, prk = 0;
     if constexpr (sizeof(R) == sizeof(double)) {
-      const double x = thp * ld(U.inv_thb + (k));
+      const double x = div_by(thp, ld(U.thb + (k)), ld(U.inv_thb + (k)));
       double f, l;
       if (!pow1p<true>(ph, U.pw, x, f, l)) {
         const double2 g = pow1p_general(x, gamma);
