@@ -61,11 +61,14 @@ __global__ void k_an_predict(Geo<R> G, Xf<R> Xt, Slow<R> SL, Xf<R> Xo, double dt
       continue;
     }
     if (k < nv) {
-      R sx, sy, sz;
-      tan_from(load_tan(G.tb, S, c), ld2(SL.sm2, i), sx, sy, sz);
-      mx[i] = d_of(Xt.mx[i]) + dts * d_of(sx);
-      my[i] = d_of(Xt.my[i]) + dts * d_of(sy);
-      mz[i] = d_of(Xt.mz[i]) + dts * d_of(sz);
+      // the Cartesian S_M in float64, from the components and the basis as stored
+      const Tan<R> b = load_tan(G.tb, S, c);
+      const Q2<R> m = ld2(SL.sm2, i);
+      double sx, sy, sz;
+      tan_from(Tan<double>{d_of(b.X), d_of(b.Y), d_of(b.A)}, Q2<double>{d_of(m.x), d_of(m.y)}, sx, sy, sz);
+      mx[i] = d_of(Xt.mx[i]) + dts * sx;
+      my[i] = d_of(Xt.my[i]) + dts * sy;
+      mz[i] = d_of(Xt.mz[i]) + dts * sz;
       Xo.th[i] = (R)(d_of(Xt.th[i]) + dts * d_of(SL.sth[i]));
       Xo.rho[i] = R(0);
     }
