@@ -1874,10 +1874,8 @@ int closure_large_step(thor_state* s, int n_small, double dt) {
 
 void closure_release(thor_state* s) {
   if (s->closure.net) cudaStreamSynchronize(s->impl->stream);   // its last evaluation, before the network forgets it
-  if (s->closure.x) cudaFree(s->closure.x);
   if (s->closure.y) cudaFree(s->closure.y);
-  for (void* a : s->closure.act)
-    if (a) cudaFree(a);
+  if (s->closure.act[0]) cudaFree(s->closure.act[0]);
   s->closure = ClosureBinding();
 }
 
@@ -2001,13 +1999,15 @@ int thor_closure_attach(thor_state* s, thor_mlp* net, const float* in_mean, cons
   cb.out_mean = out_mean;
   cb.out_std = out_std;
   cb.period = period;
-  // network buffers for every column: x and y, and two of the widest layer
+  // network buffers for every column: the output, and two of the widest layer
+  // in bfloat16; the batched passes' float32 features lie over those two (they
+  // take no more: an input row is 2 x 5 nv wide)
   int wmax = 0;
   for (int l = 0; l < net->n_layers(); ++l) wmax = std::max(wmax, net->ps[l]);
   const size_t act = (size_t)ncol * wmax * sizeof(__nv_bfloat16);
-  bool ok = !cudaMalloc(&cb.x, (size_t)ncol * 2 * kClosureFields * nv * 4) &&
-            !cudaMalloc(&cb.y, (size_t)ncol * kClosureFields * nv * 4);
-  for (int q = 0; q < 2 && ok && net->tma_ok; ++q) ok = !cudaMalloc(&cb.act[q], act);
+  const bool ok = !cudaMalloc(&cb.act[0], 2 * act) && !cudaMalloc(&cb.y, (size_t)ncol * kClosureFields * nv * 4);
+  cb.act[1] = static_cast<char*>(cb.act[0]) + act;
+  cb.x = static_cast<float*>(cb.act[0]);
   if (!ok) {
     s->closure = cb;
     closure_release(s);

@@ -28,8 +28,9 @@ struct ClosureBinding {
   thor_mlp* net = nullptr;
   std::shared_ptr<ClosureUse> use;
   const float *in_mean = nullptr, *in_std = nullptr, *out_mean = nullptr, *out_std = nullptr;
-  float *x = nullptr, *y = nullptr;   // per-state feature / output buffers
-  void* act[2] = {nullptr, nullptr};  // bfloat16 layer inputs of every column (two of the widest layer)
+  float* y = nullptr;                 // output of every column
+  void* act[2] = {nullptr, nullptr};  // bfloat16 layer inputs of every column (two of the widest layer), one allocation
+  float* x = nullptr;                 // float32 features over the same memory (the thread-staged path)
   int period = 1;                     // large steps per closure window
   long long counter = 0;              // large steps since attach
 };
