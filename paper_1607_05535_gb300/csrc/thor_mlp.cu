@@ -995,18 +995,17 @@ using EncodeTiled = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, 
                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
+// looked up once; a second thread waits for the first one's answer
 EncodeTiled encode_tiled() {
-  static void* fn = nullptr;
-  static bool looked = false;
-  if (!looked) {
-    looked = true;
+  static const EncodeTiled fn = []() -> EncodeTiled {
+    void* f = nullptr;
     cudaDriverEntryPointQueryResult q;
-    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &fn, 12000, cudaEnableDefault, &q) !=
-            cudaSuccess ||
+    if (cudaGetDriverEntryPointByVersion("cuTensorMapEncodeTiled", &f, 12000, cudaEnableDefault, &q) != cudaSuccess ||
         q != cudaDriverEntryPointSuccess)
-      fn = nullptr;
-  }
-  return reinterpret_cast<EncodeTiled>(fn);
+      return nullptr;
+    return reinterpret_cast<EncodeTiled>(f);
+  }();
+  return fn;
 }
 
 // tensor map of a bfloat16 operand X [rows][ld] read along k (k < kext):
