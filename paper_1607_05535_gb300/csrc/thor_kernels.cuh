@@ -102,16 +102,17 @@ struct Phys {
   // float copies for the float kernels (a float64 conversion per thread costs
   // an issue slot of the GB300's narrow float64 pipe)
   float Rd_f, inv_Rd_f, gamma_f, inv_gamma_f, kappa_f, g_f, two_omega_f;
+  float x3_f = 0.0f;                // range of p_pert's float series (below)
   // ((1 + x)^gamma - 1) / (gamma x) = 1 + g1 x + g2 x^2 + ... (Newton's
   // binomial series; g_k = C(gamma, k + 1) / gamma), and the largest |x| at
   // which the terms kept reach the working precision: through g4 and g7 in
-  // float64 (powers of two), through g4 in float32, about 1/13 for air (p_pert);
+  // float64 (powers of two), through g4 in float32, about 1/13 for air (p_pert;
+  // x3_f lies in a gap of the record, whose size the ensemble's blocks feel);
   // set on the host
   double pg[7] = {};
   double x4 = 0.0, x7 = 0.0;
   double qg[6] = {};                // the same for the exponent 1 / gamma
   float pg_f[4] = {};
-  float x3_f = 0.0f;
   // hydrostatic switch (Sec. 3): delta on the vertical momentum's inertia,
   // 1 for the nonhydrostatic equations, 0 under the hydrostatic approximation
   double delta = 1.0;
@@ -260,7 +261,7 @@ __device__ __forceinline__ float p_pert(const Phys& ph, float pi, float th, floa
   const float x = __fdividef(d, th);
   if (fabsf(x) <= ph.x3_f) {
     const float t = pi * d;
-    return fmaf(t * x, fmaf(x, fmaf(x, fmaf(x, ph.pg_f[3], ph.pg_f[2]), ph.pg_f[1]), ph.pg_f[0]), t);
+    return fmaf(t, x * fmaf(x, fmaf(x, fmaf(x, ph.pg_f[3], ph.pg_f[2]), ph.pg_f[1]), ph.pg_f[0]), t);
   }
   return pi * th * ph.inv_gamma_f * expm1f(ph.gamma_f * log1pf(d / th));
 }
