@@ -401,7 +401,7 @@ int thor_zonal_read_w(thor_state* state, int nlat, double* out, size_t n, long l
  * levels, on two streams (graph branches), joined before the column solve:
  * the levels of a horizontal stencil do not depend on each other, and one
  * chain's kernels fill the SMs the other's leave idle while they start and
- * drain. Default 1 for states large enough to gain from it (from 800 000
+ * drain. Default 1 for states large enough to gain from it (from 600 000
  * cells in THOR_MIXED, 200 000 in THOR_FP64), else 0; the same numbers either
  * way (tested bit for bit). */
 

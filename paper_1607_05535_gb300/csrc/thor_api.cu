@@ -592,13 +592,18 @@ int Impl<R>::set_compensated(int on) {
 //  - at most a block per SM as launched, float: each kernel starts beside the
 //    one before it (7.7 k 166 -> 152; with more blocks the early ones take the
 //    room of the running ones, 77 k 220 -> 235).
+// Where the lines lie: g5 and g6 states, n_small 8, each forced into the shape of
+// few / middling / many cells: 164 k 278 / 291 / 336, 184 k 309 / 322 / 362,
+// 205 k 322 / 319 / 373, 246 k 363 / 362 / 407; 492 k - / 592 / 593, 573 k 640 / 637,
+// 655 k 706 / 700, 737 k 791 / 767, 819 k 856 / 810, 983 k 994 / 971.
 template <typename R>
 void Impl<R>::shape() {
   const long long cells = (long long)G.ncol * G.nv;
   const bool f32 = sizeof(R) == sizeof(float), few = cells < 200000;
-  kchunk = !f32 || few ? 1 : cells < 800000 ? 2 : 3;
-  level_split = cells >= (f32 ? 800000 : 200000);
-  dense = f32 && cells >= 800000;
+  const bool many = f32 && cells >= 600000;
+  kchunk = !f32 || few ? 1 : many ? 3 : 2;
+  level_split = f32 ? many : cells >= 200000;
+  dense = many;
   carveout = f32 && few ? 50 : -1;
   overlap = f32 && few;
   int dev = 0;
