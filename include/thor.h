@@ -343,8 +343,9 @@ int thor_zonal_accumulate(thor_state* state, int nlat);
 int thor_zonal_read(thor_state* state, int nlat, double* out, size_t n, int reset, long long* samples);
 int thor_zonal_read_w(thor_state* state, int nlat, double* out, size_t n, long long* samples);
 
-/* THOR_TUNE_BLOCK: threads (one per column) in a block of the stencil
- * kernels, a multiple of 32 in [32, 256] (default 128).
+/* THOR_TUNE_BLOCK: columns (one per thread) in a block of the stencil
+ * kernels, a multiple of 32 in [32, 256] (default 128; of an ensemble 256, and
+ * its blocks of fewer columns hold several level chunks of them).
  * THOR_TUNE_SOLVE_TMA: 1 (default) runs the column solve of a THOR_MIXED
  * state with its planes staged into shared memory by TMA bulk-tensor copies
  * (where the staging fits); 0 runs the direct-load solve. Same

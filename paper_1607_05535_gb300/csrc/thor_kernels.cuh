@@ -272,14 +272,14 @@ __device__ __forceinline__ float p_pert(const Phys& ph, float pi, float th, floa
 // |t| <= 1/64 and (1 + x)^gamma - 1 = (c^gamma - 1) + c^gamma (gamma t (1 + g1 t
 // + ... + g6 t^6)). Rows of the table: c - 1, 1 / c, c^gamma - 1, c^gamma,
 // ln c, the low part of c^gamma - 1. c = 1 about x = 0, where the small result keeps its relative accuracy.
-// 14 float64 instructions (LOG: 10 more) instead of about 45 for
+// 12 float64 instructions (LOG: 10 more) instead of about 45 for
 // expm1(gamma log1p(x)); false outside [1/2, 2] or without a table.
 // Error, rms in units of 2^-53, of the pressure law with x = th' / Th_bar, with
 // expm1 and log1p 0.83 to 0.86: 0.72 for |x| < 1e-2, 0.62 and 0.58 above (without
 // the low part, from a table formed in float64 and with th' times 1 / Th_bar: 0.95
 // to 1.15, at 0.5% of the float64 large step less).
 // At g6 x 32 float64 (bound by the float64 pipe): derived quantities 234 ->
-// 146 us, physics (which also took ln and a power of p) 787 -> 228 us.
+// 153 us, physics (which also took ln and a power of p) 787 -> 247 us.
 constexpr int kPowRows = 97, kPowCols = 6;
 template <bool LOG>
 __device__ __forceinline__ bool pow1p(const Phys& ph, const double* pw, double x, double& pm1, double& ln) {

@@ -488,9 +488,10 @@ size_t tc_smem_bytes(int nt) {
 // and the input gradient of a layer), and (3) the kernels of a pass are
 // launched with programmatic stream serialization, each set up (barriers,
 // tensor memory, descriptors) while the previous one drains. Training step of
-// 320-256-256-256-160 at batch 1024, 29 launches -> 10: 163 -> 76 us; forward
-// and gradients of 370-256-256-256-185 at batch 1000, which the thread-staged
-// kernel ran before the copies were padded: 510 -> 64 us.
+// 320-256-256-256-160, 29 launches -> 10: at batch 1024 163 -> 71 us, at 64, 4096,
+// 8192 and 10240 56, 101, 166 and 244 us (the host takes 21 us a step at each); forward and
+// gradients of 370-256-256-256-185 at batch 1000, which the thread-staged kernel
+// ran before the copies were padded: 510 -> 87 us (thor_mlp::aligned).
 
 constexpr int TMA_STAGES = 4, TMA_KC = 64, kMaxSplit = 8;
 

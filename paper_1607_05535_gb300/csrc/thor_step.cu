@@ -9,7 +9,8 @@
 //
 // The vertical solve is split: k_ss_flux (a stencil kernel like the others)
 // forms the per-cell parts of the column equations, and k_ss_solve runs the
-// tridiagonal elimination with two sweeping warps per 32 columns.
+// tridiagonal elimination from both ends: two sweeping warps per 32 columns in
+// float storage, the two halves of one warp per 16 columns in float64.
 #include "../../include/thor.h"
 #include "thor_impl.cuh"
 #include "thor_reduce.cuh"
@@ -457,11 +458,11 @@ __device__ __forceinline__ void d_stage_init(const Geo<R>& G, const VR<R>& U, co
 // L2 eviction priorities of the small step's planes (thor_tune
 // THOR_TUNE_L2_HINTS): bit 0 loads the stage constants evict-first, bit 1
 // keeps the perturbations and the split's intermediates evict-last. Default
-// 3 (both): at glevel 6 x 32 levels the large step takes 1.368 ms, against
-// 1.373 with the constants' hint alone and 1.402 without hints. Float64
-// states keep their perturbations at the normal priority whatever the mode:
-// their set is twice the size, and held evict-last it slowed the float64
-// large step from 9.85 to 11.1 ms.
+// 3 (both): at glevel 6 x 32 levels the large step takes 1.187 ms, against
+// 1.192 with the constants' hint alone, 1.227 with the other's and 1.233 without
+// hints. Float64 states keep their perturbations at the normal priority whatever
+// the mode: their set is twice the size, and held evict-last it slowed the
+// float64 large step by an eighth (then 9.85 ms; 6.15 now, in every mode).
 __constant__ int c_l2mode = 3;
 __device__ __forceinline__ uint64_t pol_stream() { return l2_policy((c_l2mode & 1) ? kL2First : kL2Normal); }
 template <typename R = float>
@@ -514,8 +515,8 @@ __device__ __forceinline__ void d_ss_lapd(const Geo<R>& G, const VR<R>& U, const
 // the low parts XsL -> XoL of a compensated state (null: none). Bound by the
 // gathers' latency (float) and by the float64 pipe's multiply-adds (float64):
 // at g6 x 32, float 28.7 us with two gathered scalars and three Cartesian
-// components, 25.2 with one scalar, 18.1 in the tangent basis (80 -> 48
-// registers); float64 147 -> 84 -> 54 us.
+// components, 25.2 with one scalar, 17.9 in the tangent basis (80 -> 48
+// registers); float64 147 -> 84 -> 52 us.
 template <typename R>
 __device__ __forceinline__ void d_ss_mom(const Geo<R>& G, const VR<R>& U, const Slow<R>& SL, const Pert<R>& P, const Work<R>& T, R dtau,
                                             int divdamp, const Xf<R>& Xs, const Xf<R>& Xo, const Xf<R>& XsL, const Xf<R>& XoL, int last,
@@ -650,8 +651,9 @@ __device__ __forceinline__ void fac_store(const Fac<R>& F, int i, double inv, do
 // df_mul_f: pivot reciprocals to about 2^-46) for float-storage states:
 // one half of the lanes eliminates rows 1..p downwards
 // (c'_m = up_m / (di_m - lo_m c'_m-1)), the other rows nv-1..p+1 upwards
-// (e'_m = lo_m / (di_m - up_m e'_m+1)). Stored per row: the pivot reciprocal, c' or e', and q = lo
-// or up times the pivot reciprocal; per column: 1 / (1 - c'_p e'_p+1) for the
+// (e'_m = lo_m / (di_m - up_m e'_m+1)). Stored per row (Fac): the pivot
+// reciprocal, and in float64 c' or e' and q = lo or up times the reciprocal, in
+// float storage lo and up themselves; per column: 1 / (1 - c'_p e'_p+1) for the
 // junction rows p, p+1.
 //
 // the matrix row m of column c in the storage type
@@ -1540,7 +1542,9 @@ __global__ void __launch_bounds__(32 * kSolveWarps, 6)
 // functions read its fields from there as they need them (by reference), so
 // that the record's pointers do not all occupy registers. The copy (1.3 KB and
 // a barrier) costs a block as much as a level of its stencils, so the stencil
-// blocks hold several level chunks of their columns (threadIdx.y).
+// blocks hold 256 threads: 256 columns by default, or, where the block is tuned to
+// fewer columns, several level chunks of them (threadIdx.y; 64
+// members at 8 levels a thread, 256 / 128 / 64 columns: 11.17 / 11.15 / 12.11 ms a step).
 template <typename T>
 __device__ __forceinline__ const T& stage_record(const T* src, T* dst) {
   static_assert(sizeof(T) % 4 == 0, "record of whole words");
