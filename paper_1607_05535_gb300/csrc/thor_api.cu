@@ -228,6 +228,45 @@ struct PowSeries {
     return 0.0;
   }
 };
+// An unevaluated sum of two doubles, about 100 bits (Hida, Li and Bailey 2001)
+struct Pair {
+  double h, l;
+};
+inline Pair operator+(Pair a, Pair b) {
+  const double s = a.h + b.h, t = s - a.h, e = (a.h - (s - t)) + (b.h - t) + (a.l + b.l), h = s + e;
+  return {h, e - (h - s)};
+}
+inline Pair operator*(Pair a, Pair b) {
+  const double p = a.h * b.h, e = std::fma(a.h, b.h, -p) + (a.h * b.l + a.l * b.h), h = p + e;
+  return {h, e - (h - p)};
+}
+// e^z - 1, |z| <= 2: Taylor's series at z / 64, then e <- e (2 + e) six times
+inline Pair pair_expm1(Pair z) {
+  z = {z.h / 64, z.l / 64};
+  Pair p = {1.0, 0.0};
+  for (int k = 11; k > 1; --k) {
+    p = z * p;
+    const double q = p.h / k;
+    p = Pair{1.0, 0.0} + Pair{q, (std::fma(-q, (double)k, p.h) + p.l) / k};
+  }
+  Pair e = z * p;
+  for (int i = 0; i < 6; ++i) e = e * (Pair{2.0, 0.0} + e);
+  return e;
+}
+// ln(1/2 + j / 64)
+inline const std::vector<Pair>& table_logs() {
+  static const std::vector<Pair> logs = [] {
+    std::vector<Pair> v(kPowRows);
+    for (int j = 0; j < kPowRows; ++j) {
+      const long double l = std::log1p(j / 64.0L - 0.5L);
+      v[j].h = (double)l;
+      v[j].l = (double)(l - v[j].h);
+    }
+    return v;
+  }();
+  return logs;
+}
+
 // pow1p and the physics' (1 + y)^(1 / gamma) keep g1 .. g6: exact to float64
 // rounding up to 1/128, where the result can be small, and to 2^-46 of the
 // last table interval's small share beyond
@@ -373,11 +412,10 @@ int upload_tables(Impl<R>& I, const HostGrid& h, const std::vector<double>* vert
     if (I.U.pw && !pow_series_ok(I.ph.gamma)) I.U.pw = nullptr;
     if (I.U.pw) {
       for (int j = 0; j < kPowRows; ++j) {
-        // from long double: a unit in the last place of a row would be one of every result that uses it
+        // a unit in the last place of a row would be one of every result that uses it
         const double c = 0.5 + j / 64.0;
-        const long double l = std::log1p((long double)c - 1.0L), gl = I.ph.gamma * l, pm1 = std::expm1(gl);
-        const double hi = (double)pm1;
-        const double row[kPowCols] = {c - 1.0, 1.0 / c, hi, (double)std::exp(gl), (double)l, (double)(pm1 - hi)};
+        const Pair l = table_logs()[j], pm1 = pair_expm1(Pair{I.ph.gamma, 0.0} * l);
+        const double row[kPowCols] = {c - 1.0, 1.0 / c, pm1.h, (Pair{1.0, 0.0} + pm1).h, l.h, pm1.l};
         std::copy(row, row + kPowCols, pw.begin() + (size_t)j * kPowCols);
       }
       e = e ? e : up(I.U.pw, pw.data(), pw.size() * sizeof(double));
