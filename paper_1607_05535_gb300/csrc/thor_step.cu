@@ -508,8 +508,8 @@ __device__ __forceinline__ void d_ss_lapd(const Geo<R>& G, const VR<R>& U, const
 // constant has no gradient): the one word q rounds away low bits of its smaller term,
 // and the sums of weight times value round on the scale of the values, which
 // is many times that of their differences (a long wave at glevel 4: 2.1e-7 of
-// the gradient; two stored words 1.7e-7; less the mean 1.1e-7; 14 operations a cell
-// that cost nothing beside the loads: g6 x 32 2 508 and 2 510 us for two large steps);
+// the gradient; two stored words 1.7e-7; less the mean 1.1e-7). The 14 operations
+// a cell wait for all seven values: g6 x 32 0.4% of a large step, g5 states 0.4 to 2%;
 // in the last small step of a stage also M^(s+1) = M^(s) + M* into Xo (which
 // may be Xs itself: each cell reads its own Xs value before writing it), with
 // the low parts XsL -> XoL of a compensated state (null: none). Bound by the
